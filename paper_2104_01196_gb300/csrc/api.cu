@@ -273,7 +273,7 @@ constexpr int kOffsetMax = 32;
 
 struct SellLayout {
   std::vector<int> cptr, coff, offs;
-  int offset_chunks = 0;
+  int offset_chunks = 0, wmax = 0;
 };
 
 static bool sell_layout(const std::vector<int>& rp, const int* ci, int n, SellLayout& out) {
@@ -281,7 +281,7 @@ static bool sell_layout(const std::vector<int>& rp, const int* ci, int n, SellLa
   out.cptr.assign(nc + 1, 0);
   out.coff.assign(nc, -1);
   out.offs.clear();
-  out.offset_chunks = 0;
+  out.offset_chunks = out.wmax = 0;
   int64_t total = 0;
   std::vector<int> u;
   int prev = -1, prev_len = 0;
@@ -314,6 +314,7 @@ static bool sell_layout(const std::vector<int>& rp, const int* ci, int n, SellLa
       }
       out.offset_chunks++;
     }
+    out.wmax = std::max(out.wmax, width);
     total += (int64_t)width * kSellC;
     if (total > INT32_MAX) return false;
     out.cptr[c + 1] = (int)total;
@@ -335,6 +336,7 @@ static void upload_sell(gs2_handle* h, DevCsr& M, const std::vector<int>& rp, co
   for (int k = 0; k < M.nnz; ++k) ncols = std::max(ncols, ci[k] + 1);
   M.sell_chunks = (int)cptr.size() - 1;
   M.sell_slots = (int)slots;
+  M.sell_wmax = lay.wmax;
   M.sell_ncols = ncols;
   M.sell_offset_chunks = lay.offset_chunks;
   M.sell_ptr = (int*)h->dalloc(sizeof(int) * cptr.size());

@@ -24,11 +24,19 @@ namespace gs2 {
 
 // ---------------------------------------------------------------------------
 // epilogues: pre(i) loads the row's operands before the gathers, finish(i,
-// s, pre) consumes the row sum
+// s, pre) consumes the row sum.  The FP64 pipe (2 FMA/clk/SM) bounds the FP64
+// row kernels, so an epilogue that only subtracts the row sum from an operand
+// lets the products do it (kSub): the sum starts at that operand and
+// subtracts each product, one FP64 operation a row fewer (a 7-point residual
+// has 8 instead of 9, an undamped inner sweep of a 3-entry triangle 3 or 4
+// instead of 5).  kUnroll: the widest stencil row that takes the unrolled form
+// (k_stencil).
 // ---------------------------------------------------------------------------
 
 // r = b - A x;  rhat = D^{-1} r   (Eq. 2 residual and Eq. 3 initial guess)
 struct EpiResid {
+  static constexpr bool kSub = true;
+  static constexpr int kUnroll = 6;
   const double* __restrict__ x;
   const double* __restrict__ b;
   const double* __restrict__ dinv;
@@ -40,8 +48,8 @@ struct EpiResid {
   };
   __device__ Pre pre(int i) const { return Pre{b[i], dinv[i]}; }
   __device__ double gather(int c) const { return __ldg(x + c); }
-  __device__ void finish(int i, double s, const Pre& p) const {
-    const double ri = p.b - s;
+  __device__ double begin(const Pre& p) const { return p.b; }
+  __device__ void finish(int i, double ri, const Pre& p) const {
     const double rh = p.d * ri;
     if (r) r[i] = ri;
     if (rhat64) rhat64[i] = rh;
@@ -50,16 +58,21 @@ struct EpiResid {
 };
 
 struct EpiSpmv {
+  static constexpr bool kSub = false;
+  static constexpr int kUnroll = 8;
   const double* __restrict__ x;
   double* __restrict__ y;
   struct Pre {};
   __device__ Pre pre(int) const { return Pre{}; }
   __device__ double gather(int c) const { return __ldg(x + c); }
+  __device__ double begin(const Pre&) const { return 0.0; }
   __device__ void finish(int i, double s, const Pre&) const { y[i] = s; }
 };
 
 // y += M x (multigrid prolongation)
 struct EpiSpmvAdd {
+  static constexpr bool kSub = false;
+  static constexpr int kUnroll = 8;
   const double* __restrict__ x;
   double* __restrict__ y;
   struct Pre {
@@ -67,11 +80,14 @@ struct EpiSpmvAdd {
   };
   __device__ Pre pre(int i) const { return Pre{y[i]}; }
   __device__ double gather(int c) const { return __ldg(x + c); }
-  __device__ void finish(int i, double s, const Pre& p) const { y[i] = p.y + s; }
+  __device__ double begin(const Pre& p) const { return p.y; }
+  __device__ void finish(int i, double s, const Pre&) const { y[i] = s; }
 };
 
 // x_out = x_in + omega D^{-1} (b - A x_in)   (damped JR, ping-pong buffers)
 struct EpiJr {
+  static constexpr bool kSub = true;
+  static constexpr int kUnroll = 8;
   const double* __restrict__ x;
   const double* __restrict__ b;
   const double* __restrict__ dinv;
@@ -82,18 +98,26 @@ struct EpiJr {
   };
   __device__ Pre pre(int i) const { return Pre{x[i], b[i], dinv[i]}; }
   __device__ double gather(int c) const { return __ldg(x + c); }
-  __device__ void finish(int i, double s, const Pre& p) const {
-    x_out[i] = p.x + omega * (p.d * (p.b - s));
+  __device__ double begin(const Pre& p) const { return p.b; }
+  __device__ void finish(int i, double r, const Pre& p) const {
+    x_out[i] = p.x + omega * (p.d * r);
   }
 };
 
 // inner JR sweep on the prescaled triangle T = D^{-1} L or D^{-1} U:
 //   g' = (1-gamma) g + gamma (rhat - omega T g)
-// DAMPED and SCALED (FP16 triangles with a per-row scale) are compile-time:
+// The form and SCALED (FP16 triangles with a per-row scale) are compile-time:
 // a runtime flag on a uniform kernel argument is predicated, and its FP64
-// instructions would then issue on every row.
-template <typename GT, typename AT, bool DAMPED, bool SCALED>
+// instructions would then issue on every row.  UNIT (FP64, omega = gamma = 1,
+// Eq. (4)-(5) as printed): g' is the row sum itself and the update adds or
+// stores it, without the products by omega.  The lower precisions keep the
+// general form, so that their rounding does not depend on omega.
+enum InnerForm { INNER_PLAIN, INNER_DAMPED, INNER_UNIT };
+
+template <typename GT, typename AT, InnerForm FORM, bool SCALED>
 struct EpiInner {
+  static constexpr bool kSub = FORM == INNER_UNIT;
+  static constexpr int kUnroll = 8;
   const GT* __restrict__ g_in;
   const GT* __restrict__ rhat;
   GT* __restrict__ g_out;
@@ -111,17 +135,28 @@ struct EpiInner {
   __device__ Pre pre(int i) const {
     Pre p;
     p.rh = (AT)rhat[i];
-    p.gi = DAMPED ? (AT)g_in[i] : AT(0);
+    p.gi = FORM == INNER_DAMPED ? (AT)g_in[i] : AT(0);
     p.sc = SCALED ? (AT)__int_as_float(((int)rowscale[i] + 127) << 23) : AT(1);
     p.xi = mode == INNER_LAST_ADD ? x[i] : 0.0;
     p.x32i = (mode == INNER_LAST_ADD32 || mode == INNER_LAST_ADD32_OUT) ? x32[i] : 0.f;
     return p;
   }
   __device__ AT gather(int c) const { return (AT)__ldg(g_in + c); }
+  __device__ AT begin(const Pre& p) const { return FORM == INNER_UNIT ? p.rh : AT(0); }
   __device__ void finish(int i, AT s, const Pre& p) const {
+    if (FORM == INNER_UNIT) {
+      if (mode == INNER_MID) {
+        g_out[i] = (GT)s;
+      } else {
+        double v = (double)s;
+        if (mode == INNER_LAST_ADD) v += p.xi;
+        x[i] = v;
+      }
+      return;
+    }
     if (SCALED) s *= p.sc;
     AT go = p.rh - omega * s;
-    if (DAMPED) go = (AT(1) - gamma) * p.gi + gamma * go;
+    if (FORM == INNER_DAMPED) go = (AT(1) - gamma) * p.gi + gamma * go;
     if (mode == INNER_MID) {
       g_out[i] = (GT)go;
     } else if (mode == INNER_LAST_ADD) {
@@ -143,6 +178,8 @@ struct EpiInner {
 //   rhat32 = (fl32(D^{-1} b) - x32) - O x32
 template <bool SCALED>
 struct EpiResidSweep {
+  static constexpr bool kSub = false;
+  static constexpr int kUnroll = 4;
   const float* __restrict__ bhat;
   const float* __restrict__ x32;
   const signed char* __restrict__ rowscale;
@@ -157,6 +194,7 @@ struct EpiResidSweep {
     return p;
   }
   __device__ float gather(int c) const { return __ldg(x32 + c); }
+  __device__ float begin(const Pre&) const { return 0.f; }
   __device__ void finish(int i, float s, const Pre& p) const {
     if (SCALED) s *= p.sc;
     rhat32[i] = p.bx - s;
@@ -166,6 +204,8 @@ struct EpiResidSweep {
 // compact right-hand side of Eq. (9) on the other prescaled triangle
 // T' = D^{-1} U (forward) or D^{-1} L (backward):  rhat = D^{-1} b - T' x
 struct EpiCompact {
+  static constexpr bool kSub = true;
+  static constexpr int kUnroll = 8;
   const double* __restrict__ x;
   const double* __restrict__ b;
   const double* __restrict__ dinv;
@@ -176,8 +216,8 @@ struct EpiCompact {
   };
   __device__ Pre pre(int i) const { return Pre{b[i], dinv[i]}; }
   __device__ double gather(int c) const { return __ldg(x + c); }
-  __device__ void finish(int i, double s, const Pre& p) const {
-    const double rh = p.d * p.b - s;
+  __device__ double begin(const Pre& p) const { return p.d * p.b; }
+  __device__ void finish(int i, double rh, const Pre&) const {
     if (rhat64) rhat64[i] = rh;
     if (rhat32) rhat32[i] = (float)rh;
   }
@@ -190,6 +230,8 @@ struct EpiCompact {
 //   x_r = (1 - omega) x_r + omega (bhat_r - sum_j (a_rj / a_rr) x_j)
 template <bool DAMPED>
 struct EpiColor {
+  static constexpr bool kSub = true;
+  static constexpr int kUnroll = 8;
   const int* __restrict__ rows;
   const double* __restrict__ bhat;
   double* x;
@@ -206,8 +248,8 @@ struct EpiColor {
     return p;
   }
   __device__ double gather(int c) const { return __ldg(x + c); }
-  __device__ void finish(int, double s, const Pre& p) const {
-    const double gs = p.bh - s;
+  __device__ double begin(const Pre& p) const { return p.bh; }
+  __device__ void finish(int, double gs, const Pre& p) const {
     x[p.r] = DAMPED ? p.xr + omega * (gs - p.xr) : gs;
   }
 };
@@ -370,8 +412,8 @@ float time_tile_probe(gs2_handle* h, const DevCsr& M, int reps, int role) {
     EpiResid e{h->t, h->g1, h->dinv, nullptr, h->rhat, nullptr};
     return time_epilogue(h, M, e, reps);
   }
-  EpiInner<double, double, false, false> e{h->g0, h->rhat, nullptr, h->z, nullptr,
-                                           1.0, 1.0, 1.0, INNER_LAST_ADD};
+  EpiInner<double, double, INNER_UNIT, false> e{h->g0, h->rhat, nullptr, h->z, nullptr,
+                                                1.0, 1.0, 1.0, INNER_LAST_ADD};
   return time_epilogue(h, M, e, reps);
 }
 
@@ -395,6 +437,9 @@ void launch_jr_matrix(gs2_handle* h, const DevCsr& M, const double* b, const dou
   dispatch<double>(h, M, M.va, e, skip);
 }
 
+template <InnerForm F>
+using Form = std::integral_constant<InnerForm, F>;
+
 void launch_inner(gs2_handle* h, const DevCsr& T, int prec, const void* rhat,
                   const void* g_in, void* g_out, double* x, double omega, double gamma,
                   int mode, const int* skip) {
@@ -407,41 +452,32 @@ void launch_inner(gs2_handle* h, const DevCsr& T, int prec, const void* rhat,
   KernelTimer tm(h, prec == GS2_FP64 ? "inner64" : (prec == GS2_FP32 ? "inner32" : "inner16"),
                  bytes);
   if (prec == GS2_FP64) {
-    if (damped) {
-      EpiInner<double, double, true, false> e{(const double*)g_in, (const double*)rhat,
-                                              (double*)g_out, x, nullptr, omega, gamma, omega,
-                                              mode};
+    auto run = [&](auto form) {
+      constexpr InnerForm F = decltype(form)::value;
+      EpiInner<double, double, F, false> e{(const double*)g_in, (const double*)rhat,
+                                           (double*)g_out, x, nullptr, omega, gamma, omega, mode};
       dispatch<double>(h, T, T.va, e, skip);
-    } else {
-      EpiInner<double, double, false, false> e{(const double*)g_in, (const double*)rhat,
-                                               (double*)g_out, x, nullptr, omega, gamma, omega,
-                                               mode};
-      dispatch<double>(h, T, T.va, e, skip);
-    }
-  } else if (prec == GS2_FP32) {
-    if (damped) {
-      EpiInner<float, float, true, false> e{(const float*)g_in, (const float*)rhat,
-                                            (float*)g_out, x, nullptr, (float)omega,
-                                            (float)gamma, omega, mode, h->x32};
-      dispatch<float>(h, T, T.va32, e, skip);
-    } else {
-      EpiInner<float, float, false, false> e{(const float*)g_in, (const float*)rhat,
-                                             (float*)g_out, x, nullptr, (float)omega,
-                                             (float)gamma, omega, mode, h->x32};
-      dispatch<float>(h, T, T.va32, e, skip);
-    }
+    };
+    if (damped) run(Form<INNER_DAMPED>());
+    else if (omega == 1.0) run(Form<INNER_UNIT>());
+    else run(Form<INNER_PLAIN>());
+    return;
+  }
+  auto run = [&](auto form, auto half) {
+    constexpr InnerForm F = decltype(form)::value;
+    constexpr bool H = decltype(half)::value;
+    EpiInner<float, float, F, H> e{(const float*)g_in, (const float*)rhat, (float*)g_out, x,
+                                   H ? T.scale16 : nullptr, (float)omega, (float)gamma, omega,
+                                   mode, h->x32};
+    if constexpr (H) dispatch<__half>(h, T, T.va16, e, skip);
+    else dispatch<float>(h, T, T.va32, e, skip);
+  };
+  if (prec == GS2_FP32) {
+    if (damped) run(Form<INNER_DAMPED>(), std::false_type());
+    else run(Form<INNER_PLAIN>(), std::false_type());
   } else {
-    if (damped) {
-      EpiInner<float, float, true, true> e{(const float*)g_in, (const float*)rhat,
-                                           (float*)g_out, x, T.scale16, (float)omega,
-                                           (float)gamma, omega, mode, h->x32};
-      dispatch<__half>(h, T, T.va16, e, skip);
-    } else {
-      EpiInner<float, float, false, true> e{(const float*)g_in, (const float*)rhat,
-                                            (float*)g_out, x, T.scale16, (float)omega,
-                                            (float)gamma, omega, mode, h->x32};
-      dispatch<__half>(h, T, T.va16, e, skip);
-    }
+    if (damped) run(Form<INNER_DAMPED>(), std::true_type());
+    else run(Form<INNER_PLAIN>(), std::true_type());
   }
 }
 

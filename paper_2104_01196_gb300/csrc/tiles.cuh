@@ -61,6 +61,13 @@ struct ValTraits<__half> {
   __device__ static float get(const __half* p, int k) { return __half2float(p[k]); }
 };
 
+// An epilogue's row sum: begin(pre) + sum_k a_k x_k, or with Epi::kSub
+// begin(pre) - sum_k a_k x_k (begin = 0 for a plain sum).
+template <class Epi, typename AT>
+__device__ __forceinline__ AT row_fma(AT a, AT x, AT s) {
+  return fma(Epi::kSub ? -a : a, x, s);
+}
+
 // ---------------------------------------------------------------------------
 // TMA bulk copies and mbarriers (inline PTX, sm_90+ / sm_103a)
 // ---------------------------------------------------------------------------
@@ -156,8 +163,8 @@ struct StageLayout {
   }
 };
 
-// Engine: for every row i, acc_i = sum_k va[k] * epi.gather(ci[k]), then
-// epi.finish(i, acc_i).  Double-buffered: while the block reduces tile t
+// Engine: for every row i, acc_i = begin +- sum_k va[k] * epi.gather(ci[k]),
+// then epi.finish(i, acc_i).  Double-buffered: while the block reduces tile t
 // from one shared-memory stage, one thread has TMA fill the other stage
 // with tile t + grid (its rowptr slice, columns and values), completion
 // tracked by one mbarrier per stage.  Rows are reduced by one thread each
@@ -234,11 +241,12 @@ k_tiles(TileMat<VT> M, Epi epi, const int* skip) {
     if (d.z < 0) {
       // one long row: whole block, straight from global memory
       const int a = -1 - d.z;
-      AT s = AT(0);
+      const typename Epi::Pre pv = epi.pre(d.x);
+      AT s = threadIdx.x == 0 ? epi.begin(pv) : AT(0);
       for (int k = a + threadIdx.x; k < d.w; k += blockDim.x)
-        s = fma((AT)ValTraits<VT>::get(M.va, k), (AT)epi.gather(M.ci[k]), s);
+        s = row_fma<Epi>((AT)ValTraits<VT>::get(M.va, k), (AT)epi.gather(M.ci[k]), s);
       s = block_sum<AT>(s, red);
-      if (threadIdx.x == 0) epi.finish(d.x, s, epi.pre(d.x));
+      if (threadIdx.x == 0) epi.finish(d.x, s, pv);
       __syncthreads();
       continue;
     }
@@ -254,6 +262,7 @@ k_tiles(TileMat<VT> M, Epi epi, const int* skip) {
       typename Epi::Pre pv{};
       if (row < d.y) {
         pv = epi.pre(row);
+        if (l == 0) s = epi.begin(pv);
         const int rs = s_rp[row - rpb] - d.z, re = s_rp[row + 1 - rpb] - d.z;
         int ks = rs, ke = re;
         if (K > 1) {
@@ -266,19 +275,19 @@ k_tiles(TileMat<VT> M, Epi epi, const int* skip) {
         for (; k + 4 <= ke; k += 4) {
           const AT x0 = (AT)epi.gather(s_ci[k]), x1 = (AT)epi.gather(s_ci[k + 1]);
           const AT x2 = (AT)epi.gather(s_ci[k + 2]), x3 = (AT)epi.gather(s_ci[k + 3]);
-          s = fma((AT)ValTraits<VT>::get(s_va, k), x0, s);
-          s = fma((AT)ValTraits<VT>::get(s_va, k + 1), x1, s);
-          s = fma((AT)ValTraits<VT>::get(s_va, k + 2), x2, s);
-          s = fma((AT)ValTraits<VT>::get(s_va, k + 3), x3, s);
+          s = row_fma<Epi>((AT)ValTraits<VT>::get(s_va, k), x0, s);
+          s = row_fma<Epi>((AT)ValTraits<VT>::get(s_va, k + 1), x1, s);
+          s = row_fma<Epi>((AT)ValTraits<VT>::get(s_va, k + 2), x2, s);
+          s = row_fma<Epi>((AT)ValTraits<VT>::get(s_va, k + 3), x3, s);
         }
         const int rem = ke - k;
         if (rem > 0) {
           const AT x0 = (AT)epi.gather(s_ci[k]);
           const AT x1 = rem > 1 ? (AT)epi.gather(s_ci[k + 1]) : AT(0);
           const AT x2 = rem > 2 ? (AT)epi.gather(s_ci[k + 2]) : AT(0);
-          s = fma((AT)ValTraits<VT>::get(s_va, k), x0, s);
-          if (rem > 1) s = fma((AT)ValTraits<VT>::get(s_va, k + 1), x1, s);
-          if (rem > 2) s = fma((AT)ValTraits<VT>::get(s_va, k + 2), x2, s);
+          s = row_fma<Epi>((AT)ValTraits<VT>::get(s_va, k), x0, s);
+          if (rem > 1) s = row_fma<Epi>((AT)ValTraits<VT>::get(s_va, k + 1), x1, s);
+          if (rem > 2) s = row_fma<Epi>((AT)ValTraits<VT>::get(s_va, k + 2), x2, s);
         }
       }
       if (K > 1) s = group_sum<K, AT>(s);
@@ -349,7 +358,7 @@ __device__ __forceinline__ bool sell_pair(int n, int c, const int* __restrict__ 
   const VT* v1 = va + b1 + lane;
   const int* o0 = offs + ob0;
   const int* o1 = offs + ob1;
-  AT s0 = AT(0), s1 = AT(0);
+  AT s0 = epi.begin(p0), s1 = epi.begin(p1);
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     if (k < L) {
@@ -357,8 +366,8 @@ __device__ __forceinline__ bool sell_pair(int n, int c, const int* __restrict__ 
       const int cb = min(max(r1 + __ldg(o1 + k), 0), cmax);
       const AT a = stream_val<VT>(v0 + 32 * k), b = stream_val<VT>(v1 + 32 * k);
       const AT xa = (AT)epi.gather(ca), xb = (AT)epi.gather(cb);
-      s0 = fma(a, xa, s0);
-      s1 = fma(b, xb, s1);
+      s0 = row_fma<Epi>(a, xa, s0);
+      s1 = row_fma<Epi>(b, xb, s1);
     }
   }
   if (r0 < n) epi.finish(r0, s0, p0);
@@ -391,7 +400,7 @@ k_sell(int n, int nchunks, const int* __restrict__ cptr, const int* __restrict__
     typename Epi::Pre pv{};
     if (row < n) pv = epi.pre(row);
     const VT* vv = va + base + lane;
-    AT s = AT(0);
+    AT s = epi.begin(pv);
     int k = 0;
     const int ob = __ldg(coff + c);
     if (ob >= 0) {
@@ -407,10 +416,10 @@ k_sell(int n, int nchunks, const int* __restrict__ cptr, const int* __restrict__
         const AT a2 = stream_val<VT>(vv + 64), a3 = stream_val<VT>(vv + 96);
         const AT x0 = (AT)epi.gather(c0), x1 = (AT)epi.gather(c1);
         const AT x2 = (AT)epi.gather(c2), x3 = (AT)epi.gather(c3);
-        s = fma(a0, x0, s);
-        s = fma(a1, x1, s);
-        s = fma(a2, x2, s);
-        s = fma(a3, x3, s);
+        s = row_fma<Epi>(a0, x0, s);
+        s = row_fma<Epi>(a1, x1, s);
+        s = row_fma<Epi>(a2, x2, s);
+        s = row_fma<Epi>(a3, x3, s);
       }
       const int rem = L - k;
       if (rem > 0) {
@@ -423,9 +432,9 @@ k_sell(int n, int nchunks, const int* __restrict__ cptr, const int* __restrict__
         const AT x0 = (AT)epi.gather(c0);
         const AT x1 = rem > 1 ? (AT)epi.gather(c1) : AT(0);
         const AT x2 = rem > 2 ? (AT)epi.gather(c2) : AT(0);
-        s = fma(a0, x0, s);
-        if (rem > 1) s = fma(a1, x1, s);
-        if (rem > 2) s = fma(a2, x2, s);
+        s = row_fma<Epi>(a0, x0, s);
+        if (rem > 1) s = row_fma<Epi>(a1, x1, s);
+        if (rem > 2) s = row_fma<Epi>(a2, x2, s);
       }
       if (row < n) epi.finish(row, s, pv);
       continue;
@@ -443,20 +452,20 @@ k_sell(int n, int nchunks, const int* __restrict__ cptr, const int* __restrict__
         const int n0 = __ldcs(cc), n1 = __ldcs(cc + 32), n2 = __ldcs(cc + 64), n3 = __ldcs(cc + 96);
         const AT b0 = stream_val<VT>(vv), b1 = stream_val<VT>(vv + 32);
         const AT b2 = stream_val<VT>(vv + 64), b3 = stream_val<VT>(vv + 96);
-        s = fma(a0, x0, s);
-        s = fma(a1, x1, s);
-        s = fma(a2, x2, s);
-        s = fma(a3, x3, s);
+        s = row_fma<Epi>(a0, x0, s);
+        s = row_fma<Epi>(a1, x1, s);
+        s = row_fma<Epi>(a2, x2, s);
+        s = row_fma<Epi>(a3, x3, s);
         c0 = n0; c1 = n1; c2 = n2; c3 = n3;
         a0 = b0; a1 = b1; a2 = b2; a3 = b3;
       }
       // the last preloaded group
       const AT x0 = (AT)epi.gather(c0), x1 = (AT)epi.gather(c1);
       const AT x2 = (AT)epi.gather(c2), x3 = (AT)epi.gather(c3);
-      s = fma(a0, x0, s);
-      s = fma(a1, x1, s);
-      s = fma(a2, x2, s);
-      s = fma(a3, x3, s);
+      s = row_fma<Epi>(a0, x0, s);
+      s = row_fma<Epi>(a1, x1, s);
+      s = row_fma<Epi>(a2, x2, s);
+      s = row_fma<Epi>(a3, x3, s);
       k += 4;
       cc += 128;
       vv += 128;
@@ -468,10 +477,10 @@ k_sell(int n, int nchunks, const int* __restrict__ cptr, const int* __restrict__
       const AT a2 = stream_val<VT>(vv + 64), a3 = stream_val<VT>(vv + 96);
       const AT x0 = (AT)epi.gather(c0), x1 = (AT)epi.gather(c1);
       const AT x2 = (AT)epi.gather(c2), x3 = (AT)epi.gather(c3);
-      s = fma(a0, x0, s);
-      s = fma(a1, x1, s);
-      s = fma(a2, x2, s);
-      s = fma(a3, x3, s);
+      s = row_fma<Epi>(a0, x0, s);
+      s = row_fma<Epi>(a1, x1, s);
+      s = row_fma<Epi>(a2, x2, s);
+      s = row_fma<Epi>(a3, x3, s);
     }
     // the last one to three slots, also issued together
     const int rem = L - k;
@@ -485,12 +494,116 @@ k_sell(int n, int nchunks, const int* __restrict__ cptr, const int* __restrict__
       const AT x0 = (AT)epi.gather(c0);
       const AT x1 = rem > 1 ? (AT)epi.gather(c1) : AT(0);
       const AT x2 = rem > 2 ? (AT)epi.gather(c2) : AT(0);
-      s = fma(a0, x0, s);
-      if (rem > 1) s = fma(a1, x1, s);
-      if (rem > 2) s = fma(a2, x2, s);
+      s = row_fma<Epi>(a0, x0, s);
+      if (rem > 1) s = row_fma<Epi>(a1, x1, s);
+      if (rem > 2) s = row_fma<Epi>(a2, x2, s);
     }
     if (row < n) epi.finish(row, s, pv);
   }
+  }
+}
+
+// The row sum of an offset row of exactly W slots: every slot's value and
+// gather is issued before the first product, so a row costs one round trip
+// to memory (in groups of four, a 5- or 7-slot row costs two).  Columns are
+// clamped into [0, cmax] for the zero slots of rows at a boundary (and the
+// rows past n of the last chunk).
+template <int W, typename VT, class Epi, typename AT>
+__device__ __forceinline__ AT stencil_row(AT s, int row, const int* __restrict__ oo,
+                                          const VT* __restrict__ vv, const Epi& epi, int cmax) {
+  AT a[W], x[W];
+  int c[W];
+#pragma unroll
+  for (int k = 0; k < W; ++k) a[k] = stream_val<VT>(vv + 32 * k);
+#pragma unroll
+  for (int k = 0; k < W; ++k) c[k] = min(max(row + __ldg(oo + k), 0), cmax);
+#pragma unroll
+  for (int k = 0; k < W; ++k) x[k] = (AT)epi.gather(c[k]);
+#pragma unroll
+  for (int k = 0; k < W; ++k) s = row_fma<Epi>(a[k], x[k], s);
+  return s;
+}
+
+// ... of L <= WM slots: L is the same for the whole warp, so the switch is a
+// uniform branch
+template <int WM, typename VT, class Epi, typename AT>
+__device__ __forceinline__ AT stencil_rows(AT s, int L, int row, const int* __restrict__ oo,
+                                           const VT* __restrict__ vv, const Epi& epi, int cmax) {
+  if (WM >= 7) {
+    switch (L) {
+      case 8: return stencil_row<8, VT>(s, row, oo, vv, epi, cmax);
+      case 7: return stencil_row<7, VT>(s, row, oo, vv, epi, cmax);
+      default: break;
+    }
+  }
+  if (WM >= 5) {
+    switch (L) {
+      case 6: return stencil_row<6, VT>(s, row, oo, vv, epi, cmax);
+      case 5: return stencil_row<5, VT>(s, row, oo, vv, epi, cmax);
+      default: break;
+    }
+  }
+  switch (L) {
+    case 4: return stencil_row<4, VT>(s, row, oo, vv, epi, cmax);
+    case 3: return stencil_row<3, VT>(s, row, oo, vv, epi, cmax);
+    case 2: return stencil_row<2, VT>(s, row, oo, vv, epi, cmax);
+    case 1: return stencil_row<1, VT>(s, row, oo, vv, epi, cmax);
+    default: return s;
+  }
+}
+
+// Matrices of offset chunks of at most WM slots (5- and 7-point stencils and
+// their triangles).  A warp loads the place and the offset list of its next
+// chunk while it works on the current one, so only its first chunk waits
+// for them: with all of a row's loads issued at once, a chunk costs one
+// dependent round trip to memory where k_sell's loop costs three.  Rows are
+// reduced in the same order.  On the 150^3 convection-diffusion matrix
+// (n = 3.4M) against k_sell: SpMV 52 -> 45 us (5.4 TB/s; the FP64 pipe needs
+// 40), FP64 inner sweep 30 -> 28, FP32 inner sweep 22 -> 18; on the 1000^2
+// Laplacian SpMV 18 -> 13 us, residual 19 -> 16, FP64 inner sweep 12 -> 8.
+// (The explicit minimum of one resident block lets ptxas hold all slots of a
+// row in registers -- 54 instead of 32 for the 7-point SpMV -- where its
+// default aims at full occupancy and puts the loads one after another again.)
+template <typename VT, class Epi, int WM>
+__global__ void __launch_bounds__(kRowThreads, 1)
+k_stencil(int n, int nchunks, const int* __restrict__ cptr, const int* __restrict__ ci,
+          const VT* __restrict__ va, Epi epi, const int* skip, const int* __restrict__ live,
+          const int* __restrict__ coff, const int* __restrict__ offs, int ncols) {
+  pdl_wait();
+  if (skip && *skip) return;
+  const int lane = threadIdx.x & 31;
+  const int nw = (gridDim.x * blockDim.x) >> 5;
+  const int cmax = ncols - 1;
+  int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (c >= nchunks) return;
+  int base = cptr[c], end = cptr[c + 1], ob = coff[c];
+  // a chunk whose rows belong only to finished systems of a pack is skipped
+  int on = live ? live[c] : 1;
+  for (;;) {
+    const int cn = c + nw;
+    int nbase = 0, nend = 0, nob = 0, non = 1;
+    if (cn < nchunks) {
+      nbase = cptr[cn];
+      nend = cptr[cn + 1];
+      nob = coff[cn];
+      if (live) non = live[cn];
+    }
+    if (on) {
+      const int row = c * 32 + lane;
+      typename Epi::Pre pv{};
+      if (row < n) pv = epi.pre(row);
+      const int L = (end - base) >> 5;
+      const VT* vv = va + base + lane;
+      auto s = epi.begin(pv);
+      s = stencil_rows<WM, VT>(s, L, row, offs + ob, vv, epi, cmax);
+      if (row < n) epi.finish(row, s, pv);
+    }
+    if (cn >= nchunks) return;
+    c = cn;
+    base = nbase;
+    end = nend;
+    ob = nob;
+    on = non;
   }
 }
 
@@ -541,6 +654,11 @@ inline void launch_sell(gs2_handle* h, const DevCsr& M, const VT* sv, const Epi&
   // the 192^3 convection-diffusion matrix 59 -> 51 us).  Rows of 3 entries
   // (the inner sweeps' triangles) lost occupancy to it (51 -> 57 us), and
   // FP64 rows are bound by the FP64 pipe, so they keep one chunk.
+  // Stencils (offset chunks only, at most 8 slots) take the unrolled form up
+  // to the width at which it is the faster one for the epilogue: for the FP64
+  // residual 6 slots (its two more row operands and 7 slots need 56
+  // registers, half the resident warps: 58 against 53 us on 7-point rows,
+  // n = 3.4M), for the whole-sweep residual 4.
   bool pair = false;
   auto fn = M.mean_row > kShortRowMean ? k_sell<VT, Epi, true, false> : k_sell<VT, Epi, false, false>;
   if constexpr (sizeof(VT) < sizeof(double)) {
@@ -548,6 +666,11 @@ inline void launch_sell(gs2_handle* h, const DevCsr& M, const VT* sv, const Epi&
       pair = true;
       fn = k_sell<VT, Epi, false, true>;
     }
+  }
+  constexpr int WM = Epi::kUnroll;
+  if (M.sell_offset_chunks == M.sell_chunks && M.sell_wmax <= WM) {
+    pair = false;
+    fn = M.sell_wmax <= 4 ? k_stencil<VT, Epi, 4> : k_stencil<VT, Epi, WM>;
   }
   const int per_sm = blocks_per_sm((const void*)fn, 0);
   const int warps = kRowThreads / 32;

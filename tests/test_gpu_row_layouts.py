@@ -1,0 +1,55 @@
+"""Row kernels at the edges of their layouts, against the FP64 oracle.
+
+Tolerance as for every FP64 sweep: rows are reduced in another order and
+scaled by a precomputed D^{-1}, a few ulps per entry, so 1e-12 relative.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2104_01196_gb300 import problems as P
+from test_gpu_parity import dev, g, host, rel, rhs_and_x0  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+TOL = 1e-12
+
+
+def band_matrix(n, width, seed):
+    """n rows on `width` diagonals, the main one and others near and far on either side; entries
+    outside [0, n) dropped, so the chunks at both ends are narrower."""
+    far = [-(n // 3) - 1, -7, -1, 1, 2, n // 4 + 3, -3, 5, -(n // 2)]
+    offs = sorted({0, *far[:width - 1]})
+    val = P.uniform_pm1(seed, n * len(offs)).reshape(n, len(offs))
+    rp, ci, va = [0], [], []
+    for i in range(n):
+        for q, o in enumerate(offs):
+            if 0 <= i + o < n:
+                ci.append(i + o)
+                va.append(len(offs) + 1.0 + val[i, q] if o == 0 else val[i, q])
+        rp.append(len(ci))
+    return np.array(rp, np.int64), np.array(ci, np.int32), np.array(va)
+
+
+# every unrolled stencil width (1 to 8 slots) and the first one beyond, on rows that fill a warp,
+# miss it by one, exceed it by one, and take several chunks per warp's neighbourhood
+@pytest.mark.parametrize("width", range(1, 10))
+@pytest.mark.parametrize("n", [31, 32, 33, 1000])
+def test_stencil_widths(g, width, n):  # noqa: F811
+    A = band_matrix(n, width, 7 * width + n)
+    b, x0 = rhs_and_x0(A, 5)
+    h = g.gs2_setup(A)
+    # (31 to 33 rows pad by more than 20% in some widths and stay row tiles)
+    assert n < 1000 or h.stats()["offset_frac_a"] == 1.0
+    y = dev(np.zeros(n))
+    g.gs2_spmv(h, dev(b), y)
+    assert rel(host(y), oracle.spmv(A, b)) <= TOL
+    for omega in (1.0, 0.9):
+        x = dev(x0)
+        g.gs2_apply(h, dev(b), x, 1, 2, omega, g.SYMMETRIC)
+        assert rel(host(x), oracle.gs2(A, b, x0, 1, 2, omega, 1.0, oracle.SYMMETRIC)) <= TOL
+    x = dev(x0)
+    g.jr_apply(h, dev(b), x, 2, 0.8)
+    assert rel(host(x), oracle.jr(A, b, x0, 2, 0.8)) <= TOL
+    x = dev(x0)
+    g.mtgs_apply(h, dev(b), x, 1, 1.1, g.SYMMETRIC)
+    assert rel(host(x), oracle.mtgs(A, b, x0, 1, 1.1, oracle.SYMMETRIC)) <= TOL
