@@ -571,13 +571,14 @@ void ensure_precision(gs2_handle* h, int prec) {
   }
 }
 
-// Level sets of the triangles (level-set scheduling, Sec. 3): level(i) =
-// 1 + max level over row i's dependencies; rows are grouped by level.
-// Level sets of a strict triangle: level(i) = 1 + the largest level of the
-// rows row i depends on (0 without any); rows grouped by level on the device.
-static void build_levels(gs2_handle* h, const HostTri& T, bool lower, std::vector<int>& ptr,
-                         int*& rows_dev) {
-  const int n = (int)h->n;
+// Level sets of a strict triangle (level-set scheduling, Sec. 3): level(i) =
+// 1 + the largest level of the rows row i depends on (0 without any); the
+// rows in level order and the places of their entries in that order.
+struct HostLevels {
+  std::vector<int> levels, rows, rp;
+};
+
+static void find_levels(const HostTri& T, int n, bool lower, HostLevels& out) {
   std::vector<int> lev(n, 0);
   int nlev = n ? 1 : 0;
   for (int s = 0; s < n; ++s) {
@@ -587,20 +588,52 @@ static void build_levels(gs2_handle* h, const HostTri& T, bool lower, std::vecto
     lev[i] = lv;
     nlev = std::max(nlev, lv + 1);
   }
+  std::vector<int>& ptr = out.levels;
   ptr.assign(nlev + 1, 0);
   for (int i = 0; i < n; ++i) ptr[lev[i] + 1]++;
   for (int l = 0; l < nlev; ++l) ptr[l + 1] += ptr[l];
-  std::vector<int> fill(ptr.begin(), ptr.end() - 1), rows(std::max(n, 1));
-  for (int i = 0; i < n; ++i) rows[fill[lev[i]]++] = i;
-  rows_dev = (int*)h->dalloc(sizeof(int) * std::max(n, 1));
-  h->h2d(rows_dev, rows.data(), sizeof(int) * std::max(n, 1));
+  std::vector<int> fill(ptr.begin(), ptr.end() - 1);
+  out.rows.resize(n);
+  out.rp.assign(n + 1, 0);
+  for (int i = 0; i < n; ++i) {
+    const int p = fill[lev[i]]++;
+    out.rows[p] = i;
+    out.rp[p + 1] = T.rp[i + 1] - T.rp[i];
+  }
+  for (int p = 0; p < n; ++p) out.rp[p + 1] += out.rp[p];
+}
+
+// both triangles of one splitting, found side by side
+static void build_levels(gs2_handle* h, const HostTri& L, const HostTri& U, const DevCsr& dL,
+                         const DevCsr& dU, TriSolve& tL, TriSolve& tU) {
+  const int n = (int)h->n;
+  HostLevels hl[2];
+  std::exception_ptr failed;
+  std::thread other([&] {
+    try {
+      find_levels(L, n, true, hl[0]);
+    } catch (...) {
+      failed = std::current_exception();
+    }
+  });
+  try {
+    find_levels(U, n, false, hl[1]);
+  } catch (...) {
+    other.join();
+    throw;
+  }
+  other.join();
+  if (failed) std::rethrow_exception(failed);
+  tL.levels = hl[0].levels;
+  tU.levels = hl[1].levels;
+  tri_upload(h, dL, hl[0].rows, hl[0].rp, tL);
+  tri_upload(h, dU, hl[1].rows, hl[1].rp, tU);
 }
 
 void ensure_levels(gs2_handle* h) {
   if (h->levels_ready) return;
   gs2_host_side* hs = host_side(h);
-  build_levels(h, hs->L, true, h->lev_ptr_L, h->lev_rows_L);
-  build_levels(h, hs->U, false, h->lev_ptr_U, h->lev_rows_U);
+  build_levels(h, hs->L, hs->U, h->L, h->U, h->triL, h->triU);
   h->levels_ready = true;
 }
 
@@ -738,8 +771,7 @@ Hybrid* ensure_hybrid(gs2_handle* h, const gs2_params* p) {
     // local exact GS: level sets of the local triangles (each block's own
     // dependency chains side by side)
     auto& tris = hs->hyb[P];
-    build_levels(h, tris.first, true, y->lev_ptr_L, y->lev_rows_L);
-    build_levels(h, tris.second, false, y->lev_ptr_U, y->lev_rows_U);
+    build_levels(h, tris.first, tris.second, y->Lloc, y->Uloc, y->triL, y->triU);
     y->levels_ready = true;
   }
   return y;
@@ -1189,8 +1221,8 @@ gs2_status gs2_get_stats(const gs2_handle* h, gs2_handle_stats* out) {
   out->nnz = h->nnz;
   out->nnz_lower = h->L.nnz;
   out->nnz_upper = h->U.nnz;
-  out->levels_lower = h->levels_ready ? (int)h->lev_ptr_L.size() - 1 : 0;
-  out->levels_upper = h->levels_ready ? (int)h->lev_ptr_U.size() - 1 : 0;
+  out->levels_lower = h->levels_ready ? (int)h->triL.levels.size() - 1 : 0;
+  out->levels_upper = h->levels_ready ? (int)h->triU.levels.size() - 1 : 0;
   out->device_bytes = h->dev_bytes + amg_device_bytes(h);
   out->tpr_a = h->A.tpr;
   out->tpr_tri = h->L.tpr;

@@ -129,6 +129,30 @@ struct Profiler;
 struct AmgHierarchy;
 struct Pack;
 
+// A strict triangle prepared for the exact triangular solve (trisolve.cu):
+// rows in level order (level v: places levels[v] .. levels[v + 1)), entries
+// with the place of their column in that order, chunks of 32 / lanes rows of
+// one level, and the solution g in that order.
+struct TriSolve {
+  std::vector<int> levels;  // host
+  int lanes = 1, width = 0, nchunks = 0;  // lanes and entries (longest) of a row
+  int *rows = nullptr, *rp = nullptr, *ci = nullptr;
+  double* va = nullptr;
+  int2* chunk = nullptr;  // {first place, rows}
+  unsigned long long* g = nullptr;
+  int* ticket = nullptr;  // the next chunk to be taken
+};
+struct TriView {
+  int nchunks;
+  const int2* __restrict__ chunk;
+  const int* __restrict__ rows;
+  const int* __restrict__ rp;
+  const int* __restrict__ ci;
+  const double* __restrict__ va;
+  unsigned long long* g;
+  int* ticket;
+};
+
 // Hybrid (block-Jacobi) form of the relaxations (Sec. 3): the rows in
 // `parts` contiguous blocks (block p: rows [p n / P, (p+1) n / P)), A split
 // into the entries inside a row's block (Aloc) and the couplings to other
@@ -139,9 +163,7 @@ struct Hybrid {
   double* c = nullptr;  // b - E x of the current exchange
   // level sets of the local triangles (local exact GS), built on first use
   bool levels_ready = false;
-  std::vector<int> lev_ptr_L, lev_ptr_U;
-  int* lev_rows_L = nullptr;
-  int* lev_rows_U = nullptr;
+  TriSolve triL, triU;
 };
 
 }  // namespace gs2
@@ -173,9 +195,7 @@ struct gs2_handle {
 
   // level sets (lazy)
   bool levels_ready = false;
-  std::vector<int> lev_ptr_L, lev_ptr_U;  // host, nlev + 1
-  int* lev_rows_L = nullptr;
-  int* lev_rows_U = nullptr;
+  gs2::TriSolve triL, triU;
 
   // multicolour GS (lazy): colour c holds the rows color_rows[c] (ascending)
   // and their off-diagonal entries prescaled by D^{-1}, as its own matrix
@@ -364,9 +384,13 @@ void launch_jr(gs2_handle* h, const double* b, const double* x_in,
                double* x_out, double omega, const int* skip);
 void launch_jr_matrix(gs2_handle* h, const DevCsr& M, const double* b, const double* x_in,
                       double* x_out, double omega, const int* skip);
-void launch_level(gs2_handle* h, const DevCsr& T, const int* rows, int r0,
-                  int r1, const double* rhat, double* g, double* x,
-                  double omega, const int* skip);
+// the exact triangular solve by T and x += omega g (x_zero: x = omega g)
+void launch_trisolve(gs2_handle* h, const TriSolve& T, const double* rhat, double* x,
+                     double omega, bool x_zero, const int* skip);
+// T's device arrays for the triangle M; T.levels is set, rows are M's rows
+// in level order and rp the places of their entries
+void tri_upload(gs2_handle* h, const DevCsr& M, const std::vector<int>& rows,
+                const std::vector<int>& rp, TriSolve& T);
 
 // one colour of a multicolour GS sweep: for each row i of the colour matrix
 // C (original row rows[i]), x_r = (1 - omega) x_r + omega (bhat_r - (C x)_i)

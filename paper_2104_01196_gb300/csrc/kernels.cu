@@ -29,7 +29,8 @@ namespace gs2 {
 // lets the products do it (kSub): the sum starts at that operand and
 // subtracts each product, one FP64 operation a row fewer (a 7-point residual
 // has 8 instead of 9, an undamped inner sweep of a 3-entry triangle 3 or 4
-// instead of 5).  kUnroll: the widest stencil row that takes the unrolled form
+// instead of 5; a few more roundings of the operand's size: sweeps are 2e-16 from
+// the 64-bit result where they were 1.6e-16).  kUnroll: the widest stencil row that takes the unrolled form
 // (k_stencil).
 // ---------------------------------------------------------------------------
 
@@ -662,59 +663,6 @@ void launch_copy(gs2_handle* h, double* dst, const double* src) {
   if (h->n == 0 || dst == src) return;
   GS2_CUDA(cudaMemcpyAsync(dst, src, sizeof(double) * h->n, cudaMemcpyDeviceToDevice,
                            h->stream));
-}
-
-// ---------------------------------------------------------------------------
-// level-scheduled triangular solve (exact GS baseline)
-// ---------------------------------------------------------------------------
-
-// Rows of one level are independent: g_i = rhat_i - omega sum_k T_ik g_k over
-// dependencies k in earlier levels (final already), then x_i += omega g_i.
-// This is the forward recurrence of (D + omega L) g = r scaled by D^{-1}.
-template <int K>
-__global__ void __launch_bounds__(kRowThreads)
-k_level(const int* __restrict__ rows, int r0, int r1, const int* __restrict__ rp,
-        const int* __restrict__ ci, const double* __restrict__ va,
-        const double* __restrict__ rhat, double* g, double* x, double omega,
-        const int* skip) {
-  // launched with programmatic dependent launch: the next level's launch
-  // overlaps this one; its rows wait here for the previous level's results
-  pdl_wait();
-  if (skip && *skip) return;
-  const int q = threadIdx.x / K, l = threadIdx.x % K;
-  constexpr int G = kRowThreads / K;
-  for (int base = r0 + blockIdx.x * G; base < r1; base += gridDim.x * G) {
-    const int idx = base + q;
-    double s = 0.0;
-    int row = -1;
-    if (idx < r1) {
-      row = rows[idx];
-      for (int k = rp[row] + l; k < rp[row + 1]; k += K) s = fma(va[k], g[ci[k]], s);
-    }
-    s = group_sum<K, double>(s);
-    if (row >= 0 && l == 0) {
-      const double gi = rhat[row] - omega * s;
-      g[row] = gi;
-      x[row] += omega * gi;
-    }
-  }
-}
-
-void launch_level(gs2_handle* h, const DevCsr& T, const int* rows, int r0, int r1,
-                  const double* rhat, double* g, double* x, double omega,
-                  const int* skip) {
-  const int cnt = r1 - r0;
-  if (cnt <= 0) return;
-  const int K = T.tpr >= 8 ? 8 : 1;
-  const int G = kRowThreads / K;
-  const int grid = std::max(1, std::min((cnt + G - 1) / G, h->nsm * 8));
-  if (K == 8)
-    launch_pdl(k_level<8>, grid, kRowThreads, 0, h->stream, rows, r0, r1, (const int*)T.rp,
-               (const int*)T.ci, (const double*)T.va, rhat, g, x, omega, skip);
-  else
-    launch_pdl(k_level<1>, grid, kRowThreads, 0, h->stream, rows, r0, r1, (const int*)T.rp,
-               (const int*)T.ci, (const double*)T.va, rhat, g, x, omega, skip);
-  GS2_LAUNCH_CHECK();
 }
 
 }  // namespace gs2

@@ -1,5 +1,5 @@
 // Relaxation drivers: GS2 (non-compact Eq. 2 and compact Eq. 9), exact
-// GS/SOR by level-scheduled triangular solves, damped JR, and the
+// GS/SOR by triangular solves (trisolve.cu), damped JR, and the
 // zero-start preconditioner application used by the Krylov solvers.
 #include <algorithm>
 
@@ -156,9 +156,8 @@ static int global_sweeps(const gs2_params* p) {
 // the rhat buffer of the sweep precision.
 // ---------------------------------------------------------------------------
 
-static void gs_half_levels(gs2_handle* h, const DevCsr& T, const std::vector<int>& ptr,
-                           const int* rows, const DevCsr& R, const double* b, double* x,
-                           double omega, bool x_zero, const int* skip);
+static void gs_half(gs2_handle* h, const DevCsr& T, const TriSolve& S, const DevCsr& R,
+                    const double* b, double* x, double omega, bool x_zero, const int* skip);
 
 static void hybrid_apply(gs2_handle* h, const gs2_params* p, const Hybrid& Y, const double* b,
                          double* x, bool x_zero, const int* skip) {
@@ -184,13 +183,11 @@ static void hybrid_apply(gs2_handle* h, const gs2_params* p, const Hybrid& Y, co
       if (p->kind == GS2_PC_GS) {
         // local exact GS / SOR: the local triangular solves by level sets
         if (p->direction == GS2_FORWARD || p->direction == GS2_SYMMETRIC) {
-          gs_half_levels(h, Y.Lloc, Y.lev_ptr_L, Y.lev_rows_L, Y.Aloc, c, x, p->omega, zero,
-                         skip);
+          gs_half(h, Y.Lloc, Y.triL, Y.Aloc, c, x, p->omega, zero, skip);
           zero = false;
         }
         if (p->direction == GS2_BACKWARD || p->direction == GS2_SYMMETRIC) {
-          gs_half_levels(h, Y.Uloc, Y.lev_ptr_U, Y.lev_rows_U, Y.Aloc, c, x, p->omega, zero,
-                         skip);
+          gs_half(h, Y.Uloc, Y.triU, Y.Aloc, c, x, p->omega, zero, skip);
           zero = false;
         }
         continue;
@@ -239,30 +236,22 @@ void gs2_relax(gs2_handle* h, const double* b, double* x, const gs2_params* p) {
 }
 
 // ---------------------------------------------------------------------------
-// exact GS / SOR baseline: x += omega (D + omega T)^{-1} (b - A x), the
-// triangular solve by level sets (one launch per level)
+// exact GS / SOR baseline: x += omega (D + omega T)^{-1} (b - A x)
 // ---------------------------------------------------------------------------
 
-// One exact half sweep by level sets of T: r-hat = D^{-1} (b - R x) (R = A;
-// the local block in the hybrid form), then the triangular solve level by
-// level with the x update.  x_zero: x = 0 and D^{-1} b is in h->rhat.
-static void gs_half_levels(gs2_handle* h, const DevCsr& T, const std::vector<int>& ptr,
-                           const int* rows, const DevCsr& R, const double* b, double* x,
-                           double omega, bool x_zero, const int* skip) {
-  if (x_zero) {
-    launch_fill(h, x, 0.0, skip);
-  } else {
-    launch_resid_matrix(h, R, b, x, nullptr, h->rhat, nullptr, skip);
-  }
+// One exact half sweep with the triangle T (prepared as S): r-hat = D^{-1}
+// (b - R x) (R = A; the local block in the hybrid form), then the triangular
+// solve with the x update.  x_zero: x = 0 and D^{-1} b is in h->rhat.
+static void gs_half(gs2_handle* h, const DevCsr& T, const TriSolve& S, const DevCsr& R,
+                    const double* b, double* x, double omega, bool x_zero, const int* skip) {
+  if (!x_zero) launch_resid_matrix(h, R, b, x, nullptr, h->rhat, nullptr, skip);
   KernelTimer tm(h, "levels", T.nnz * 12.0 + 4.0 * (h->n + 1) + 32.0 * h->n);
-  for (size_t l = 0; l + 1 < ptr.size(); ++l)
-    launch_level(h, T, rows, ptr[l], ptr[l + 1], h->rhat, h->g0, x, omega, skip);
+  launch_trisolve(h, S, h->rhat, x, omega, x_zero, skip);
 }
 
 static void gs_half(gs2_handle* h, bool lower, const double* b, double* x, double omega,
                     bool x_zero, const int* skip) {
-  gs_half_levels(h, lower ? h->L : h->U, lower ? h->lev_ptr_L : h->lev_ptr_U,
-                 lower ? h->lev_rows_L : h->lev_rows_U, h->A, b, x, omega, x_zero, skip);
+  gs_half(h, lower ? h->L : h->U, lower ? h->triL : h->triU, h->A, b, x, omega, x_zero, skip);
 }
 
 void gs_relax(gs2_handle* h, const double* b, double* x, int sweeps, double omega,

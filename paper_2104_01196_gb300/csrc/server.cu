@@ -75,7 +75,7 @@ static int64_t sell_bytes(int64_t entries, int64_t n, int vbytes) {
 // two prescaled triangles, their sliced-ELL copies, the resident vectors,
 // the Krylov basis and the optional lower-precision, level-set and colour
 // storage (mirrors setup_handle, upload_sell, ensure_precision,
-// ensure_levels, ensure_colors and ensure_krylov).
+// ensure_levels (tri_upload), ensure_colors and ensure_krylov).
 static int64_t footprint(const gs2_server_cfg& c, int64_t n, int64_t nnz) {
   const int64_t off = std::max<int64_t>(nnz - n, 0);
   const int64_t m = std::max(c.restart, 1);
@@ -95,7 +95,10 @@ static int64_t footprint(const gs2_server_cfg& c, int64_t n, int64_t nnz) {
       b += 12 * off + 4 * (n + 17) + (n / 16 + 16) * 16 + sell_bytes(off, n, 8) +
            (vp == GS2_FP32 ? 8 : 4) * off + 2 * n + 8 * n + 4 * (n / 32 + 2);
   }
-  if (c.has_precond && c.precond.kind == GS2_PC_GS) b += 8 * n;
+  // exact GS: the triangles in level order (of the hybrid form too), with
+  // row lists, chunks and the solution
+  if (c.has_precond && c.precond.kind == GS2_PC_GS)
+    b += (c.precond.parts > 1 ? 2 : 1) * (12 * off + 2 * 28 * n);
   // hybrid form: the local block of A, the couplings, the local triangles
   // (with their low-precision copies) and the exchange vector
   if (c.has_precond && c.precond.parts > 1) {

@@ -1,0 +1,216 @@
+// The triangular solve of exact Gauss-Seidel / SOR, (D + omega T) g = r by
+// D^{-1}:  g_i = rhat_i - omega sum_k T_ik g_k, then x_i += omega g_i, in one
+// launch for the whole triangle.
+//
+// What bounds it is the chain of levels: a 100^3 stencil has 298 of them,
+// each a dependent step, against 24 us of memory traffic for the sweep.  One
+// launch per level cost 4.9 us a step (1450 us per half sweep); a grid
+// barrier per level would cost 1.3 us on top of a level's own round trips.
+// Here no level waits for another as a whole: rows are solved as soon as
+// their own dependencies are.  g is its own flag -- every entry starts as
+// kPending, a NaN pattern no result takes, and a reader polls the eight bytes
+// it needs anyway -- so a step costs one store to L2, one load from it and
+// the row's products.
+//
+// Rows are stored in level order, entries with the place of their column in
+// that order, so the rows of a warp (one chunk: rows of one level) write one
+// run of g and read a few runs of it; in natural order a level's rows are
+// strided and every lane would poll a sector of its own.  A warp takes the
+// next chunk from a counter.  Chunks are handed out in level order and a warp
+// finishes its chunk before its next one, so the first unfinished chunk
+// always has its dependencies solved and a running warp: the kernel needs no
+// co-resident grid.  Waits are bounded all the same; a warp that gives up
+// records GS2_ERR_TIMEOUT and leaves.
+//
+// Measured, a symmetric sweep (two half sweeps, residuals included): 100^3
+// Laplacian (298 levels) 2908 -> 512 us, 0.8 us a level; 500^2 Laplacian (999
+// levels) 6508 -> 1099; 40^2 426 -> 75; Q1 elasticity on 20^3 nodes 5931 ->
+// 900.  One, two and four blocks per SM differ by 3%.
+#include "tiles.cuh"
+
+namespace gs2 {
+
+constexpr unsigned long long kPending = ~0ull;
+constexpr int kTriThreads = 256;
+constexpr int kTriBlocksPerSm = 2;
+
+// every entry of g pending, the chunk counter at 0
+__global__ void k_tri_begin(int n, unsigned long long* g, int* ticket, const int* skip) {
+  pdl_wait();
+  if (skip && *skip) return;
+  const int i0 = blockIdx.x * blockDim.x + threadIdx.x;
+  for (int i = i0; i < n; i += gridDim.x * blockDim.x) g[i] = kPending;
+  if (i0 == 0) *ticket = 0;
+}
+
+__device__ __forceinline__ unsigned long long ld_relaxed(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.relaxed.gpu.global.b64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_relaxed(unsigned long long* p, unsigned long long v) {
+  asm volatile("st.relaxed.gpu.global.b64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
+// K lanes per row (32 / K rows a chunk): lane l of a row takes entries l,
+// l + K, ..., G of them in flight at once.  The row's sum starts at rhat and
+// the values are multiplied by omega before the wait, so that only the
+// products stand between the last dependency's arrival and g (a dependent
+// FP64 operation takes 33 ns: 3% of the solve against rhat - omega * sum).
+// Skipping the empty slots' products by a branch cost more than they do
+// (+10%), and so did waiting by warp instead of by lane (+5%, +50% on rows
+// of a few dozen entries); a sleep between polls changed nothing.
+template <int K, int G>
+__global__ void __launch_bounds__(kTriThreads, kTriBlocksPerSm)
+k_trisolve(TriView T, const double* __restrict__ rhat, double* x, double omega, int x_zero,
+           const int* skip, int* err) {
+  pdl_wait();
+  if (skip && *skip) return;
+  const int lane = threadIdx.x & 31, q = lane / K, l = lane % K;
+  int c = 0;
+  if (lane == 0) c = atomicAdd(T.ticket, 1);
+  c = __shfl_sync(0xffffffffu, c, 0);
+  while (c < T.nchunks) {
+    int next = 0;
+    if (lane == 0) next = atomicAdd(T.ticket, 1);  // arrives while this chunk waits
+    const int2 ch = __ldg(T.chunk + c);
+    const int p = ch.x + q;
+    const bool own = q < ch.y;
+    int a = 0, e = 0, row = 0;
+    double s = 0.0, xi = 0.0;
+    if (own) {
+      a = __ldg(T.rp + p);
+      e = __ldg(T.rp + p + 1);
+      if (l == 0) {
+        row = __ldg(T.rows + p);
+        s = rhat[row];
+        if (!x_zero) xi = x[row];
+      }
+    }
+    bool ok = true;
+    for (int k = a + l; k < e; k += G * K) {
+      int d[G];
+      double v[G];
+      unsigned long long y[G];
+#pragma unroll
+      for (int j = 0; j < G; ++j) {
+        const bool in = k + j * K < e;
+        d[j] = in ? __ldg(T.ci + k + j * K) : -1;
+        v[j] = in ? -omega * __ldg(T.va + k + j * K) : 0.0;
+      }
+#pragma unroll
+      for (int j = 0; j < G; ++j) y[j] = d[j] >= 0 ? ld_relaxed(T.g + d[j]) : 0ull;
+      long long t0 = 0;
+      for (;;) {
+        bool wait = false;
+#pragma unroll
+        for (int j = 0; j < G; ++j) wait = wait || y[j] == kPending;
+        if (!wait) break;
+#pragma unroll
+        for (int j = 0; j < G; ++j)
+          if (y[j] == kPending) y[j] = ld_relaxed(T.g + d[j]);
+        const long long t = clock64();
+        if (t0 == 0) t0 = t;
+        if (t - t0 > kWaitBudgetCycles) {
+          ok = false;
+          break;
+        }
+      }
+      if (!ok) break;
+#pragma unroll
+      for (int j = 0; j < G; ++j)
+        s = fma(v[j], __longlong_as_double((long long)y[j]), s);
+    }
+    if (__any_sync(0xffffffffu, !ok)) {
+      if (lane == 0 && err) atomicExch(err, (int)GS2_ERR_TIMEOUT);
+      return;
+    }
+    if (K > 1) s = group_sum<K, double>(s);
+    if (own && l == 0) {
+      unsigned long long bits = (unsigned long long)__double_as_longlong(s);
+      if (bits == kPending) bits = 0x7ff8000000000000ull;  // a NaN, but not that one
+      st_relaxed(T.g + p, bits);
+      x[row] = xi + omega * s;
+    }
+    c = __shfl_sync(0xffffffffu, next, 0);
+  }
+}
+
+// entries of the rows in level order (rp: their places): the place of each
+// entry's column, and its value
+__global__ void k_tri_place(int n, const int* __restrict__ rows, int* place) {
+  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < n; p += gridDim.x * blockDim.x)
+    place[rows[p]] = p;
+}
+__global__ void k_tri_entries(int n, const int* __restrict__ rows, const int* __restrict__ place,
+                              const int* __restrict__ rp0, const int* __restrict__ ci0,
+                              const double* __restrict__ va0, const int* __restrict__ rp, int* ci,
+                              double* va) {
+  for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < n; p += gridDim.x * blockDim.x) {
+    const int a0 = rp0[rows[p]], a = rp[p], len = rp[p + 1] - a;
+    for (int k = 0; k < len; ++k) {
+      ci[a + k] = place[ci0[a0 + k]];
+      va[a + k] = va0[a0 + k];
+    }
+  }
+}
+
+void tri_upload(gs2_handle* h, const DevCsr& M, const std::vector<int>& rows,
+                const std::vector<int>& rp, TriSolve& T) {
+  const int n = M.n;
+  if (n == 0) return;
+  // lanes per row: short rows one, so that a chunk is 32 rows; longer rows
+  // more, as a lane's groups of four entries wait one after another (Q1
+  // elasticity, 37 entries: 8 lanes 965 us a sweep, 16 lanes 921)
+  T.lanes = M.mean_row <= 6.0 ? 1 : M.mean_row <= 24.0 ? 4 : 16;
+  T.width = 0;
+  for (int p = 0; p < n; ++p) T.width = std::max(T.width, rp[p + 1] - rp[p]);
+  const int per = 32 / T.lanes;
+  std::vector<int2> chunk;
+  chunk.reserve(n / per + T.levels.size());
+  for (size_t v = 0; v + 1 < T.levels.size(); ++v)
+    for (int p = T.levels[v]; p < T.levels[v + 1]; p += per)
+      chunk.push_back(make_int2(p, std::min(per, T.levels[v + 1] - p)));
+  T.nchunks = (int)chunk.size();
+  T.rows = (int*)h->dalloc(sizeof(int) * n);
+  T.rp = (int*)h->dalloc(sizeof(int) * (n + 1));
+  T.ci = (int*)h->dalloc(sizeof(int) * std::max(M.nnz, 1));
+  T.va = (double*)h->dalloc(sizeof(double) * std::max(M.nnz, 1));
+  T.chunk = (int2*)h->dalloc(sizeof(int2) * chunk.size());
+  T.g = (unsigned long long*)h->dalloc(sizeof(double) * n);
+  T.ticket = (int*)h->dalloc(sizeof(int));
+  h->h2d(T.rows, rows.data(), sizeof(int) * n);
+  h->h2d(T.rp, rp.data(), sizeof(int) * (n + 1));
+  h->h2d(T.chunk, chunk.data(), sizeof(int2) * chunk.size());
+  // the column -> place map is needed only here: it lies in g until the
+  // first solve
+  int* place = (int*)T.g;
+  k_tri_place<<<vec_blocks(h, n), kVecThreads, 0, h->stream>>>(n, T.rows, place);
+  GS2_LAUNCH_CHECK();
+  k_tri_entries<<<vec_blocks(h, n), kVecThreads, 0, h->stream>>>(n, T.rows, place, M.rp, M.ci,
+                                                                M.va, T.rp, T.ci, T.va);
+  GS2_LAUNCH_CHECK();
+}
+
+void launch_trisolve(gs2_handle* h, const TriSolve& T, const double* rhat, double* x,
+                     double omega, bool x_zero, const int* skip) {
+  if (h->n == 0) return;
+  const int n = (int)h->n;
+  launch_pdl(k_tri_begin, vec_blocks(h, n), kVecThreads, 0, h->stream, n, T.g, T.ticket, skip);
+  GS2_LAUNCH_CHECK();
+  const TriView v{T.nchunks, T.chunk, T.rows, T.rp, T.ci, T.va, T.g, T.ticket};
+  const int warps = kTriThreads / 32;
+  const int grid = std::max(1, std::min((T.nchunks + warps - 1) / warps,
+                                        kTriBlocksPerSm * h->nsm));
+  // one lane a row: no more slots in flight than the longest row has
+  auto fn = T.lanes == 16  ? k_trisolve<16, 4>
+            : T.lanes == 4 ? k_trisolve<4, 4>
+            : T.width > 3  ? k_trisolve<1, 4>
+            : T.width == 3 ? k_trisolve<1, 3>
+                           : k_trisolve<1, 2>;
+  launch_pdl(fn, grid, kTriThreads, 0, h->stream, v, rhat, x, omega, x_zero ? 1 : 0, skip,
+             h->dev_err);
+  GS2_LAUNCH_CHECK();
+}
+
+}  // namespace gs2

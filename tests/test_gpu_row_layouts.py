@@ -53,3 +53,56 @@ def test_stencil_widths(g, width, n):  # noqa: F811
     x = dev(x0)
     g.mtgs_apply(h, dev(b), x, 1, 1.1, g.SYMMETRIC)
     assert rel(host(x), oracle.mtgs(A, b, x0, 1, 1.1, oracle.SYMMETRIC)) <= TOL
+
+
+def chain_matrix(n):
+    """Every row needs the one before it (and, backwards, the one after it): n levels of one row."""
+    i = np.arange(n)
+    M = np.zeros((n, n))
+    M[i, i] = 4.0
+    M[i[1:], i[:-1]] = -1.0 + 0.001 * i[1:]
+    M[i[:-1], i[1:]] = 0.5
+    return P.dense_to_csr(M)
+
+
+# the triangular solve: one row, chains of single rows, levels that fill a chunk and exceed it, and
+# rows that take 1, 4 and 16 lanes with a remainder of every size, one of them longer than a group
+TRI = {
+    "n1": (np.array([0, 1]), np.array([0], np.int32), np.array([3.0])),
+    "chain_2": chain_matrix(2),
+    "chain_300": chain_matrix(300),
+    "one_level_65": P.dense_to_csr(np.diag(np.arange(1.0, 66.0))),
+    "stencil_33": P.poisson2d_matrix(33),
+    "stencil_3d_9": P.poisson3d_matrix(9),
+    "lanes_1_long_row": P.random_csr(700, 3, mean_offdiag=4.0, long_rows=[(650, 300)]),
+    "lanes_4": P.random_csr(500, 4, mean_offdiag=20.0),
+    "lanes_16": P.random_csr(400, 5, mean_offdiag=90.0, long_rows=[(390, 380)]),
+}
+
+
+@pytest.mark.parametrize("name", list(TRI))
+@pytest.mark.parametrize("direction", [0, 1, 2])
+def test_triangular_solve(g, name, direction):  # noqa: F811
+    A = TRI[name]
+    b, x0 = rhs_and_x0(A, 21)
+    h = g.gs2_setup(A)
+    for sweeps, omega in ((1, 1.0), (2, 1.2)):
+        x = dev(x0)
+        g.gs_apply(h, dev(b), x, sweeps, omega, direction)
+        assert rel(host(x), oracle.gs(A, b, x0, sweeps, omega, direction)) <= TOL
+    h.check()
+
+
+# NaN right-hand sides -- the pattern that marks an unsolved row among them -- reach the rows that
+# depend on them and no others, and nothing waits for them
+@pytest.mark.parametrize("bits", [0x7ff8000000000000, 0xffffffffffffffff, 0xfff8000000000001])
+def test_triangular_solve_nan(g, bits):  # noqa: F811
+    A = chain_matrix(100)
+    b, x0 = rhs_and_x0(A, 22)
+    b[40] = np.array([bits], np.uint64).view(np.float64)[0]
+    h = g.gs2_setup(A)
+    x = dev(x0)
+    g.gs_apply(h, dev(b), x, 1, 1.0, 0)
+    h.check()
+    got = host(x)
+    assert np.isnan(got[40:]).all() and not np.isnan(got[:40]).any()
