@@ -254,9 +254,16 @@ void retile(gs2_handle* h, DevCsr& M, const std::vector<int>& rp, int K, int RPT
 // row issues only the row's FMAs, with no segment reduction and no idle
 // lanes, which matters on this part's FP64 pipe (on the 81-entry rows of Q1
 // elasticity the residual went from 2.8 to 5.0 TB/s against the best
-// row-tile shape, 8 lanes per row).  Smaller long-row matrices (coarse
-// multigrid levels) are latency-bound and keep the row tiles, whose K lanes
-// per row shorten each row's chain of dependent gathers.
+// row-tile shape, 8 lanes per row).  Long rows of smaller matrices (coarse
+// multigrid levels) are latency-bound: K lanes per row shorten each row's
+// chain of dependent gathers.  Their FP64 values, and those of matrices of
+// uneven rows, get lane slices, which reduce a row in K segments as the row
+// tiles do without staging it through shared memory (the stages limit a tile
+// kernel to 2 to 3 blocks per SM, and its barriers idle the short rows'
+// lanes): symmetric FP64 sweep on 300,007 uneven rows 115 -> 70 us, on Q1
+// elasticity with 28^3 nodes 105 -> 58.  FP32 and FP16 values, half the bytes
+// through the same stages, stay in the row tiles (inner sweep on the uneven
+// rows 7.1 us against 10.5 in lane slices, on 40^3 nodes 15.4 against 19.8).
 constexpr int kSellC = 32;                       // rows per chunk (one warp)
 constexpr double kSellMaxPadding = 1.2;          // slots / entries
 constexpr double kSellStreamBytes = 128.0 * (1 << 20);  // CSR bytes beyond L2
@@ -267,7 +274,8 @@ constexpr double kSellStreamBytes = 128.0 * (1 << 20);  // CSR bytes beyond L2
 // at most its longest row + kOffsetSlack and at most 32 (stencil rows: the
 // rows at a grid boundary miss some offsets and get zero slots there).
 // Consecutive chunks with the same offset list share one copy.  Returns
-// false when the slots would not fit 32-bit offsets.
+// false when the layout pads too much or its slots would not fit 32-bit
+// offsets.
 constexpr int kOffsetSlack = 2;
 constexpr int kOffsetMax = 32;
 
@@ -316,41 +324,139 @@ static bool sell_layout(const std::vector<int>& rp, const int* ci, int n, SellLa
     }
     out.wmax = std::max(out.wmax, width);
     total += (int64_t)width * kSellC;
-    if (total > INT32_MAX) return false;
+    if (total > INT32_MAX || total > kSellMaxPadding * rp[n]) return false;
     out.cptr[c + 1] = (int)total;
   }
   return true;
 }
 
+constexpr int kLaneWindow = 1024;    // rows sorted together
+constexpr int kLaneWarpsPerSm = 16;  // warps that a matrix should give each SM
+constexpr int kLaneMaxSlots = 128;   // of one chunk: longer rows need a whole block
+
+// Lanes per row: at most 24 entries a lane on average; with fewer than 16
+// warps per SM more lanes, down to 4 entries each (a warp's groups of four
+// slots wait one after another, 0.4 us each out of L2: Q1 elasticity on 16^3
+// nodes, SpMV 7.1 -> 5.0 us with 8 lanes instead of 4); and two where the
+// longest row exceeds 32 entries a lane (the 300,007 uneven rows, 64 at most:
+// a symmetric sweep 79 -> 70 us).  With more than 16 warps per SM further
+// lanes only add shuffles and FP64 adds (elasticity on 28^3 nodes: 58 us with
+// 4 lanes, 98 with 16).  A pack's lanes do not depend on its size.
+static int lane_count(const gs2_handle* h, int64_t n, double mean, int longest) {
+  int K = choose_lanes(mean);
+  if (h->for_pack) return K;
+  auto more = [&] { return K < 16 && mean > 4.0 * K; };
+  while (more() && (n * K < 32 * (int64_t)kLaneWarpsPerSm * h->nsm || longest > 32 * K)) K *= 2;
+  return K;
+}
+
+// Lane-slice layout: K lanes per row, rows sorted by their number of slots
+// inside windows of kLaneWindow rows where the padding calls for it (the sort
+// is stable and local, so neighbouring rows' gathers stay near one another).
+// Returns false when the slots would not fit 32-bit offsets.
+
+struct LaneLayout {
+  std::vector<int> cptr, row;  // row empty: in order
+};
+
+static bool lane_layout(const std::vector<int>& rp, int n, int K, LaneLayout& out) {
+  const int per = 32 / K;
+  std::vector<int> width(n);
+  for (int i = 0; i < n; ++i) width[i] = (rp[i + 1] - rp[i] + K - 1) / K;
+  auto chunks = [&](const std::vector<int>& row) {
+    out.cptr.assign((n + per - 1) / per + 1, 0);
+    int64_t total = 0;
+    for (size_t c = 0; c + 1 < out.cptr.size(); ++c) {
+      if (total > kSellMaxPadding * rp[n]) return false;
+      int w = 0;
+      for (int p = (int)c * per; p < std::min(n, ((int)c + 1) * per); ++p)
+        w = std::max(w, width[row.empty() ? p : row[p]]);
+      total += 32 * (int64_t)w;
+      if (total > INT32_MAX) return false;
+      out.cptr[c + 1] = (int)total;
+    }
+    return total <= kSellMaxPadding * rp[n];
+  };
+  out.row.clear();
+  if (chunks(out.row)) return true;
+  std::vector<int> row(n);
+  // counting sort, widest first (windows that start in a thread's range are its)
+  parallel_ranges(n, [&](int64_t i0, int64_t i1, int) {
+    std::vector<int> at(kLaneMaxSlots + 2);
+    for (int64_t w0 = (i0 + kLaneWindow - 1) / kLaneWindow * kLaneWindow; w0 < i1;
+         w0 += kLaneWindow) {
+      const int w1 = (int)std::min<int64_t>(n, w0 + kLaneWindow);
+      std::fill(at.begin(), at.end(), 0);
+      for (int i = (int)w0; i < w1; ++i) at[width[i]]++;
+      int next = (int)w0;
+      for (int v = kLaneMaxSlots; v >= 0; --v) {
+        const int count = at[v];
+        at[v] = next;
+        next += count;
+      }
+      for (int i = (int)w0; i < w1; ++i) row[at[width[i]]++] = i;
+    }
+  });
+  out.row.swap(row);
+  return chunks(out.row);
+}
+
 // The sliced-ELL arrays are filled on the device from the CSR arrays already
-// there (launch_to_sell); only the chunk layout is computed here.
+// there (launch_to_sell, launch_to_lanes); only the chunk layout is computed
+// here.
 static void upload_sell(gs2_handle* h, DevCsr& M, const std::vector<int>& rp, const int* ci) {
   const int n = M.n;
   if (n == 0 || M.nnz == 0) return;
-  if (M.mean_row > kShortRowMean && 12.0 * M.nnz < kSellStreamBytes) return;
   SellLayout lay;
-  if (!sell_layout(rp, ci, n, lay) || lay.cptr.back() > kSellMaxPadding * M.nnz) return;
-  const std::vector<int>& cptr = lay.cptr;
+  const bool sliced = (M.mean_row <= kShortRowMean || 12.0 * M.nnz >= kSellStreamBytes) &&
+                      sell_layout(rp, ci, n, lay);
+  LaneLayout lanes;
+  if (!sliced) {
+    // rows of uneven length, and long rows in a matrix that fits L2
+    int longest = 0;
+    for (int i = 0; i < n; ++i) longest = std::max(longest, rp[i + 1] - rp[i]);
+    const int K = lane_count(h, n, M.mean_row, longest);
+    M.sell_lanes = K;
+    if (longest > kLaneMaxSlots * K || !lane_layout(rp, n, K, lanes)) {
+      M.sell_lanes = 0;
+      return;  // row tiles
+    }
+  }
+  const std::vector<int>& cptr = sliced ? lay.cptr : lanes.cptr;
   const size_t slots = std::max(cptr.back(), 1);
-  int ncols = 1;
-  for (int k = 0; k < M.nnz; ++k) ncols = std::max(ncols, ci[k] + 1);
+  std::vector<int> top(kHostThreads, 0);
+  parallel_ranges(M.nnz, [&](int64_t k0, int64_t k1, int t) {
+    int v = 0;
+    for (int64_t k = k0; k < k1; ++k) v = std::max(v, ci[k]);
+    top[t] = v;
+  });
+  const int ncols = 1 + *std::max_element(top.begin(), top.end());
   M.sell_chunks = (int)cptr.size() - 1;
   M.sell_slots = (int)slots;
-  M.sell_wmax = lay.wmax;
   M.sell_ncols = ncols;
-  M.sell_offset_chunks = lay.offset_chunks;
   M.sell_ptr = (int*)h->dalloc(sizeof(int) * cptr.size());
   M.sell_ci = (int*)h->dalloc(sizeof(int) * slots);
   M.sell_va = (double*)h->dalloc(sizeof(double) * slots);
+  h->dzero(M.sell_va, sizeof(double) * slots);
+  h->h2d(M.sell_ptr, cptr.data(), sizeof(int) * cptr.size());
+  M.sell = true;
+  if (!sliced) {
+    GS2_CUDA(cudaMemsetAsync(M.sell_ci, 0xff, sizeof(int) * slots, h->stream));
+    if (!lanes.row.empty()) {
+      M.sell_row = (int*)h->dalloc(sizeof(int) * n);
+      h->h2d(M.sell_row, lanes.row.data(), sizeof(int) * n);
+    }
+    launch_to_lanes(h, M);
+    return;
+  }
+  M.sell_wmax = lay.wmax;
+  M.sell_offset_chunks = lay.offset_chunks;
   M.sell_coff = (int*)h->dalloc(sizeof(int) * std::max<size_t>(lay.coff.size(), 1));
   M.sell_off = (int*)h->dalloc(sizeof(int) * std::max<size_t>(lay.offs.size(), 1));
   h->dzero(M.sell_ci, sizeof(int) * slots);
-  h->dzero(M.sell_va, sizeof(double) * slots);
-  h->h2d(M.sell_ptr, cptr.data(), sizeof(int) * cptr.size());
   h->h2d(M.sell_coff, lay.coff.data(), sizeof(int) * lay.coff.size());
   if (!lay.offs.empty()) h->h2d(M.sell_off, lay.offs.data(), sizeof(int) * lay.offs.size());
   launch_to_sell(h, M, M.va, M.sell_va, true);
-  M.sell = true;
 }
 
 static void upload_csr(gs2_handle* h, DevCsr& M, int n, const std::vector<int>& rp,
@@ -409,7 +515,8 @@ static void prepare_lowprec(gs2_handle* h, DevCsr& M, const HostTri&, int prec) 
     // and the upload were most of a lower-precision request's setup)
     M.va32 = (float*)h->dalloc(sizeof(float) * nz);
     launch_values_to_fp32(h, M, (int64_t)nz);
-    if (M.sell_chunks > 0) {  // the layout exists (the autotuner may turn it off and on)
+    // the layout exists (the autotuner may turn it off and on)
+    if (M.sell_chunks > 0 && !M.sell_lanes) {
       const size_t slots = M.sell_slots;
       M.sell_va32 = (float*)h->dalloc(sizeof(float) * slots);
       h->dzero(M.sell_va32, sizeof(float) * slots);
@@ -426,7 +533,8 @@ static void prepare_lowprec(gs2_handle* h, DevCsr& M, const HostTri&, int prec) 
     M.scale16 = (signed char*)h->dalloc(sizeof(signed char) * std::max(M.n, 1));
     h->dzero(M.va16, sizeof(__half) * nz);
     launch_values_to_fp16(h, M);
-    if (M.sell_chunks > 0) {  // the layout exists (the autotuner may turn it off and on)
+    // the layout exists (the autotuner may turn it off and on)
+    if (M.sell_chunks > 0 && !M.sell_lanes) {
       const size_t slots = M.sell_slots;
       M.sell_va16 = (__half*)h->dalloc(sizeof(__half) * slots);
       h->dzero(M.sell_va16, sizeof(__half) * slots);
@@ -1084,7 +1192,8 @@ void gs2::validate_csr(int64_t n, int64_t nnz, const int64_t* RP, const int32_t*
 // temporaries.  Throws gs2::Error; a partly built handle is released.
 gs2_handle* gs2::setup_handle(int64_t n, int64_t nnz, const int64_t* rowptr,
                               const int32_t* col, const double* val, int on_device,
-                              unsigned precisions, cudaStream_t stream, bool async_alloc) {
+                              unsigned precisions, cudaStream_t stream, bool async_alloc,
+                              bool for_pack) {
   gs2_handle* h = nullptr;
   try {
   if (n < 0 || nnz < 0) GS2_THROW(GS2_ERR_INVALID_ARG, "negative size");
@@ -1168,6 +1277,7 @@ gs2_handle* gs2::setup_handle(int64_t n, int64_t nnz, const int64_t* rowptr,
   GS2_CUDA(cudaDeviceGetAttribute(&h->nsm, cudaDevAttrMultiProcessorCount, h->device));
   h->stream = stream;
   h->async_alloc = async_alloc;
+  h->for_pack = for_pack;
   h->n = n;
   h->nnz = nnz;
   upload_csr(h, h->A, (int)n, rp32, CI, VA, (int)nnz);
@@ -1455,7 +1565,7 @@ gs2_status gs2_pack_setup(int count, const int64_t* n, const int64_t* const* row
   gs2_handle* h = nullptr;
   try {
     h = setup_handle(off.back(), (int64_t)ci.size(), rp.data(), ci.data(), va.data(), 0,
-                     precisions, (cudaStream_t)stream, false);
+                     precisions, (cudaStream_t)stream, false, true);
   } catch (const gs2::Error& e) {
     // "... in row <g>": name the system and its own row
     const size_t sp = e.msg.find_last_of(' ');

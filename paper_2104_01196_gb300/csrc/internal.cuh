@@ -106,6 +106,15 @@ struct DevCsr {
   double* sell_va = nullptr;
   float* sell_va32 = nullptr;
   __half* sell_va16 = nullptr;
+  // Lane slices (sell_lanes = K > 0, FP64 values only), for matrices that the
+  // layout above does not suit: K lanes per row as in the row tiles, so a chunk holds 32 / K
+  // rows; lane l of a row takes its l-th K-th part (ceil(length / K)
+  // consecutive entries), slot k of the warp's lanes side by side at
+  // sell_ptr[c] + 32 k + lane; padding slots have column -1.  Rows of uneven
+  // length are sorted by it inside windows: sell_row[p] is the row at place p
+  // (null: in order).
+  int sell_lanes = 0;
+  int* sell_row = nullptr;
 };
 
 // Device-resident GMRES / CG state, one per handle.
@@ -221,8 +230,11 @@ struct gs2_handle {
   gs2::AmgHierarchy* amg = nullptr;
 
   // a pack of independent systems (gs2_pack_setup): the matrix is their
-  // block-diagonal concatenation; null for a single system
+  // block-diagonal concatenation; null for a single system.  for_pack is set
+  // before the matrix is uploaded: how a row is reduced must not depend on
+  // the pack's size, so that a system's result does not depend on the others
   gs2::Pack* pack = nullptr;
+  bool for_pack = false;
   // hybrid forms built so far, one per partition (ensure_precond)
   std::vector<gs2::Hybrid*> hybrids;
 
@@ -404,6 +416,9 @@ void launch_to_sell(gs2_handle* h, const DevCsr& M, const double* va, double* sv
 void launch_to_sell(gs2_handle* h, const DevCsr& M, const float* va, float* sva, bool with_ci);
 void launch_to_sell(gs2_handle* h, const DevCsr& M, const __half* va, __half* sva, bool with_ci);
 
+// ... and columns into lane slices (M.sell_lanes > 0; columns preset to -1)
+void launch_to_lanes(gs2_handle* h, const DevCsr& M);
+
 // y = M x (accumulate: y += M x) for any tiled matrix M whose columns index x
 void launch_spmv_matrix(gs2_handle* h, const DevCsr& M, const double* x, double* y,
                         bool accumulate, const int* skip);
@@ -556,7 +571,7 @@ void validate_csr(int64_t n, int64_t nnz, const int64_t* rowptr, const int32_t* 
 // handle creation / destruction shared by gs2_setup and the server
 gs2_handle* setup_handle(int64_t n, int64_t nnz, const int64_t* rowptr, const int32_t* col,
                          const double* val, int on_device, unsigned precisions,
-                         cudaStream_t stream, bool async_alloc);
+                         cudaStream_t stream, bool async_alloc, bool for_pack = false);
 void destroy_handle(gs2_handle* h);
 
 // small pinned, device-mapped host buffers, recycled process-wide (freeing

@@ -383,6 +383,30 @@ void launch_to_sell(gs2_handle* h, const DevCsr& M, const __half* va, __half* sv
   to_sell(h, M, va, sva, with_ci);
 }
 
+// CSR rows into lane slices (DevCsr::sell_lanes), one thread per lane of a row
+__global__ void k_to_lanes(int n, int K, const int* __restrict__ rp, const int* __restrict__ ci,
+                           const double* __restrict__ va, const int* __restrict__ cptr,
+                           const int* __restrict__ perm, int* sci, double* sva) {
+  const int64_t total = (int64_t)n * K;
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
+       t += (int64_t)gridDim.x * blockDim.x) {
+    const int p = (int)(t / K), l = (int)(t % K);
+    const int row = perm ? perm[p] : p;
+    const int a = rp[row], len = rp[row + 1] - a, seg = (len + K - 1) / K;
+    const int base = cptr[t >> 5] + (int)(t & 31);
+    for (int k = 0; k < seg && l * seg + k < len; ++k) {
+      sva[base + 32 * k] = va[a + l * seg + k];
+      sci[base + 32 * k] = ci[a + l * seg + k];
+    }
+  }
+}
+
+void launch_to_lanes(gs2_handle* h, const DevCsr& M) {
+  k_to_lanes<<<vec_blocks(h, (int64_t)M.n * M.sell_lanes), kVecThreads, 0, h->stream>>>(
+      M.n, M.sell_lanes, M.rp, M.ci, M.va, M.sell_ptr, M.sell_row, M.sell_ci, M.sell_va);
+  GS2_LAUNCH_CHECK();
+}
+
 // Autotuner probe: milliseconds per launch of M's most frequent kernel with
 // M's current tile shape, best of `reps`: the residual for A (role 0), the
 // inner sweep with the x update for a triangle (roles 1, 2).  The operands

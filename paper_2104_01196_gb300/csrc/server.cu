@@ -66,9 +66,9 @@ struct Group {
 
 // Bytes of the sliced-ELL copy of a matrix with this many entries (at most
 // 1.2 slots per entry, else no copy is made) holding vbytes-byte values, with
-// its chunk offsets.
+// its chunk offsets and row order (lane slices: up to a chunk per two rows).
 static int64_t sell_bytes(int64_t entries, int64_t n, int vbytes) {
-  return (entries * 6 / 5 + 1) * (4 + vbytes) + 4 * (n / 32 + 2);
+  return (entries * 6 / 5 + 1) * (4 + vbytes) + 4 * (n / 2 + 2) + 4 * n;
 }
 
 // Device bytes a request of this size holds once admitted: the matrix, its
@@ -304,7 +304,7 @@ static void prepare_group(gs2_server* s, Group* g) {
       const gs2_params* pc = s->cfg.has_precond ? &s->cfg.precond : nullptr;
       if (pc && pc->kind == GS2_PC_GS2) prec = 1u << pc->precision;
       g->h = setup_handle(off.back(), (int64_t)cci.size(), crp.data(), cci.data(), cva.data(), 0,
-                          prec, g->stream, true);
+                          prec, g->stream, true, true);
       pack_attach(g->h, off);
       ensure_precond(g->h, pc);
       g->h->graph_mode = 1;

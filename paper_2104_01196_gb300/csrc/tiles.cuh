@@ -607,7 +607,68 @@ k_stencil(int n, int nchunks, const int* __restrict__ cptr, const int* __restric
   }
 }
 
+// Lane slices (DevCsr::sell_lanes): K lanes per row, 32 / K rows a warp, each
+// lane its consecutive part of the row as in the row tiles, read slot by slot
+// as coalesced loads.  One warp per chunk: the
+// rows of a window are sorted longest first, so the long chunks of every
+// window start early and the hardware's block scheduler fills in the short
+// ones.  The next group's four slots are loaded while the current group's
+// gathers are in flight; padding slots (column -1) gather nothing, so an
+// infinity elsewhere cannot reach the row.
+// (Five resident blocks: at the 66 registers ptxas takes unasked, three fit
+// and the uneven rows' sweep takes 91 instead of 70 us; at eight it takes 101.)
+template <int K, class Epi>
+__global__ void __launch_bounds__(kRowThreads, 5)
+k_lanes(int n, int nchunks, const int* __restrict__ cptr, const int* __restrict__ ci,
+        const double* __restrict__ va, Epi epi, const int* skip, const int* __restrict__ live,
+        const int* __restrict__ perm) {
+  pdl_wait();
+  if (skip && *skip) return;
+  const int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (c >= nchunks) return;
+  const int lane = threadIdx.x & 31, l = lane % K;
+  const int p = c * (32 / K) + lane / K;
+  // rows in order: all of them belong to one 32-row chunk of finished systems
+  if (live && !perm && live[(c * (32 / K)) >> 5] == 0) return;
+  const int base = cptr[c], L = (cptr[c + 1] - base) >> 5;
+  const bool own = p < n;
+  const int row = own ? (perm ? __ldg(perm + p) : p) : 0;
+  const int* cc = ci + base + lane;
+  const double* vv = va + base + lane;
+  int c0 = -1, c1 = -1, c2 = -1, c3 = -1;
+  double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+  auto load = [&](int k) {
+    c0 = c1 = c2 = c3 = -1;
+    a0 = a1 = a2 = a3 = 0.0;
+    if (k < L) { c0 = __ldcs(cc); a0 = __ldcs(vv); }
+    if (k + 1 < L) { c1 = __ldcs(cc + 32); a1 = __ldcs(vv + 32); }
+    if (k + 2 < L) { c2 = __ldcs(cc + 64); a2 = __ldcs(vv + 64); }
+    if (k + 3 < L) { c3 = __ldcs(cc + 96); a3 = __ldcs(vv + 96); }
+    cc += 128;
+    vv += 128;
+  };
+  load(0);
+  typename Epi::Pre pv{};
+  if (own) pv = epi.pre(row);
+  double s = l == 0 ? epi.begin(pv) : 0.0;
+  for (int k = 0; k < L; k += 4) {
+    const double x0 = c0 >= 0 ? epi.gather(c0) : 0.0;
+    const double x1 = c1 >= 0 ? epi.gather(c1) : 0.0;
+    const double x2 = c2 >= 0 ? epi.gather(c2) : 0.0;
+    const double x3 = c3 >= 0 ? epi.gather(c3) : 0.0;
+    const double b0 = a0, b1 = a1, b2 = a2, b3 = a3;
+    load(k + 4);
+    s = row_fma<Epi>(b0, x0, s);
+    if (k + 1 < L) s = row_fma<Epi>(b1, x1, s);
+    if (k + 2 < L) s = row_fma<Epi>(b2, x2, s);
+    if (k + 3 < L) s = row_fma<Epi>(b3, x3, s);
+  }
+  if (K > 1) s = group_sum<K, double>(s);
+  if (own && l == 0) epi.finish(row, s, pv);
+}
+
 inline const double* sell_values(const DevCsr& M, const double*) { return M.sell_va; }
+// (lane slices hold FP64 values only: sell_va32 and sell_va16 are null there)
 inline const float* sell_values(const DevCsr& M, const float*) { return M.sell_va32; }
 inline const __half* sell_values(const DevCsr& M, const __half*) { return M.sell_va16; }
 
@@ -639,6 +700,26 @@ inline void launch_k(gs2_handle* h, const DevCsr& M, const VT* va, const Epi& ep
   const int per_sm = blocks_per_sm((const void*)fn, smem);
   const int grid = std::min(M.ntiles, per_sm * h->nsm);
   launch_pdl(fn, grid, kRowThreads, smem, h->stream, view<VT>(h, M, va), epi, skip);
+  GS2_LAUNCH_CHECK();
+}
+
+// chunk liveness (packs) applies to the matrices whose rows are the handle's
+inline const int* live_rows(const gs2_handle* h, const DevCsr& M) {
+  return (h->row_live && (&M == &h->A || &M == &h->L || &M == &h->U)) ? h->row_live : nullptr;
+}
+
+template <class Epi>
+inline void launch_lanes(gs2_handle* h, const DevCsr& M, const double* sv, const Epi& epi,
+                         const int* skip) {
+  auto fn = M.sell_lanes == 1   ? k_lanes<1, Epi>
+            : M.sell_lanes == 2 ? k_lanes<2, Epi>
+            : M.sell_lanes == 4 ? k_lanes<4, Epi>
+            : M.sell_lanes == 8 ? k_lanes<8, Epi>
+                                : k_lanes<16, Epi>;
+  const int warps = kRowThreads / 32;
+  const int grid = (M.sell_chunks + warps - 1) / warps;
+  launch_pdl(fn, grid, kRowThreads, 0, h->stream, M.n, M.sell_chunks, (const int*)M.sell_ptr,
+             (const int*)M.sell_ci, sv, epi, skip, live_rows(h, M), (const int*)M.sell_row);
   GS2_LAUNCH_CHECK();
 }
 
@@ -677,11 +758,8 @@ inline void launch_sell(gs2_handle* h, const DevCsr& M, const VT* sv, const Epi&
   // (FP32 / FP16 values: a warp takes chunks in pairs)
   const int tasks = pair ? (M.sell_chunks + 1) / 2 : M.sell_chunks;
   const int grid = std::max(1, std::min((tasks + warps - 1) / warps, per_sm * h->nsm));
-  // chunk liveness applies to the matrices whose rows are the handle's rows
-  const int* live =
-      (h->row_live && (&M == &h->A || &M == &h->L || &M == &h->U)) ? h->row_live : nullptr;
   launch_pdl(fn, grid, kRowThreads, 0, h->stream, M.n, M.sell_chunks,
-             (const int*)M.sell_ptr, (const int*)M.sell_ci, sv, epi, skip, live,
+             (const int*)M.sell_ptr, (const int*)M.sell_ci, sv, epi, skip, live_rows(h, M),
              (const int*)M.sell_coff, (const int*)M.sell_off, M.sell_ncols);
   GS2_LAUNCH_CHECK();
 }
@@ -693,6 +771,12 @@ inline void dispatch(gs2_handle* h, const DevCsr& M, const VT* va, const Epi& ep
                      const int* skip) {
   const VT* sv = M.sell ? sell_values(M, va) : nullptr;
   if (sv) {
+    if constexpr (sizeof(VT) == sizeof(double)) {
+      if (M.sell_lanes) {
+        launch_lanes<Epi>(h, M, sv, epi, skip);
+        return;
+      }
+    }
     launch_sell<VT, Epi>(h, M, sv, epi, skip);
     return;
   }

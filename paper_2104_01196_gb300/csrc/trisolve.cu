@@ -163,6 +163,7 @@ void tri_upload(gs2_handle* h, const DevCsr& M, const std::vector<int>& rows,
   // more, as a lane's groups of four entries wait one after another (Q1
   // elasticity, 37 entries: 8 lanes 965 us a sweep, 16 lanes 921)
   T.lanes = M.mean_row <= 6.0 ? 1 : M.mean_row <= 24.0 ? 4 : 16;
+  if (h->for_pack) T.lanes = M.tpr >= 8 ? 16 : 1;  // (as far as can be, whatever the others)
   T.width = 0;
   for (int p = 0; p < n; ++p) T.width = std::max(T.width, rp[p + 1] - rp[p]);
   const int per = 32 / T.lanes;

@@ -106,3 +106,63 @@ def test_triangular_solve_nan(g, bits):  # noqa: F811
     h.check()
     got = host(x)
     assert np.isnan(got[40:]).all() and not np.isnan(got[:40]).any()
+
+
+def uneven_matrix(n, mean, longest, seed):
+    """Row lengths spread evenly over 1 .. longest around `mean`, unsorted columns."""
+    M = P.random_csr(n, seed, mean_offdiag=mean, empty_frac=0.1,
+                     long_rows=[(n // 2, longest)] if longest else [])
+    return M
+
+
+# lane slices: every lane count, rows in order and sorted by length, empty rows, n not a multiple of
+# a chunk or of the sort's window, and a row too long for them (row tiles)
+LANES = {
+    "uneven_1500": uneven_matrix(1500, 9.0, 0, 31),
+    "uneven_1024": uneven_matrix(1024, 9.0, 60, 32),
+    "uneven_5003": uneven_matrix(5003, 14.0, 100, 33),
+    "uneven_40001": uneven_matrix(40001, 3.0, 0, 34),
+    "long_777": uneven_matrix(777, 40.0, 130, 35),
+    "long_90": uneven_matrix(90, 60.0, 80, 36),
+    "too_long_4000": uneven_matrix(4000, 6.0, 3000, 37),
+}
+
+
+@pytest.mark.parametrize("name", list(LANES))
+def test_lane_slices(g, name):  # noqa: F811
+    A = LANES[name]
+    n = len(A[0]) - 1
+    b, x0 = rhs_and_x0(A, 41)
+    h = g.gs2_setup(A)
+    y = dev(np.zeros(n))
+    g.gs2_spmv(h, dev(b), y)
+    assert rel(host(y), oracle.spmv(A, b)) <= TOL
+    for inner, omega in ((1, 1.0), (2, 0.9)):
+        x = dev(x0)
+        g.gs2_apply(h, dev(b), x, 1, inner, omega, g.SYMMETRIC)
+        assert rel(host(x), oracle.gs2(A, b, x0, 1, inner, omega, 1.0, oracle.SYMMETRIC)) <= TOL
+    x = dev(x0)
+    g.jr_apply(h, dev(b), x, 2, 0.8)
+    assert rel(host(x), oracle.jr(A, b, x0, 2, 0.8)) <= TOL
+    x = dev(x0)
+    g.mtgs_apply(h, dev(b), x, 1, 1.1, g.SYMMETRIC)
+    assert rel(host(x), oracle.mtgs(A, b, x0, 1, 1.1, oracle.SYMMETRIC)) <= TOL
+
+
+# an infinity in x reaches the rows that hold its column, as an infinity, and no padding slot
+def test_lane_slices_infinity(g):  # noqa: F811
+    A = LANES["uneven_5003"]
+    n = len(A[0]) - 1
+    x = P.uniform_pm1(43, n)
+    x[[0, 777]] = np.inf
+    h = g.gs2_setup(A)
+    y = dev(np.zeros(n))
+    g.gs2_spmv(h, dev(x), y)
+    rows = np.repeat(np.arange(n), np.diff(A[0]))
+    hit = np.zeros(n, bool)
+    hit[rows[np.isin(A[1], [0, 777])]] = True
+    got = host(y)
+    assert np.isfinite(got[~hit]).all() and not np.isfinite(got[hit]).any()
+    one = np.zeros(n, int)
+    np.add.at(one, rows[np.isin(A[1], [0, 777])], 1)
+    assert np.isinf(got[one == 1]).all()
