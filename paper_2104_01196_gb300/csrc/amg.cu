@@ -467,6 +467,7 @@ void amg_prepare(gs2_handle* h, const gs2_params* p) {
 // x = C b for the dense coarsest inverse: one warp per row
 __global__ void k_dense_mv(int n, const double* __restrict__ c, const double* __restrict__ b,
                            double* x, const int* skip) {
+  pdl_wait();
   if (skip && *skip) return;
   const int lane = threadIdx.x & 31;
   const int row = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
@@ -484,7 +485,8 @@ static void cycle(AmgHierarchy* H, size_t l, const gs2_params& sp, const double*
   gs2_handle* hl = L.h;
   if (l + 1 == H->lv.size()) {
     KernelTimer tm(hl, "amg_coarse", 8.0 * H->nc * (H->nc + 2));
-    k_dense_mv<<<(int)((H->nc + 7) / 8), 256, 0, hl->stream>>>((int)H->nc, H->cinv, b, x, skip);
+    launch_pdl(k_dense_mv, (int)((H->nc + 7) / 8), 256, 0, hl->stream, (int)H->nc, H->cinv, b, x,
+               skip);
     GS2_LAUNCH_CHECK();
     return;
   }

@@ -1298,11 +1298,6 @@ gs2_handle* gs2::setup_handle(int64_t n, int64_t nnz, const int64_t* rowptr,
   h->bstage = (double*)h->dalloc(sizeof(double) * nv);
   h->xstage = (double*)h->dalloc(sizeof(double) * nv);
   h->nblk = vec_blocks(h, n);
-  // reductions: at least ~16 rows per thread and one block per SM (the
-  // widest CGS2 kernels hold ~150 registers per thread, one 256-thread block
-  // per SM), so the per-block reduction stays small next to the FP64 work
-  h->nblk_dot = (int)std::max<int64_t>(
-      1, std::min<int64_t>((n + kVecThreads * 16 - 1) / (kVecThreads * 16), h->nsm));
   h->part_cap = h->nblk * (kMaxRestart + 2);
   h->part = (double*)h->dalloc(sizeof(double) * h->part_cap);
   for (int p = 1; p <= 4; ++p)

@@ -130,8 +130,7 @@ struct KrylovState {
   double beta;     // ||r0|| of the cycle
   double hn;       // last H(j+1, j)
   double inv_hn;
-  double rz;       // CG: r.z
-  double alpha;
+  double rz[2];    // CG: r.z before and after an iteration, by its parity
 };
 
 struct Profiler;
@@ -198,8 +197,7 @@ struct gs2_handle {
   // whole-sweep precisions: fl32(D^{-1} b) and the FP32 iterate
   float *bhat32 = nullptr, *x32 = nullptr;
   double* part = nullptr;  // per-block partial sums
-  int nblk = 0;            // blocks of the elementwise vector kernels
-  int nblk_dot = 0;        // blocks of the reduction kernels (<= nblk)
+  int nblk = 0;            // blocks of the vector and reduction kernels
   int part_cap = 0;        // doubles in `part`
 
   // level sets (lazy)

@@ -545,6 +545,7 @@ void launch_color(gs2_handle* h, const DevCsr& C, const int* rows, const double*
 __global__ void k_prep_rhat(int n, const double* __restrict__ v,
                             const double* __restrict__ dinv, double* rhat64, float* rhat32,
                             const int* skip) {
+  pdl_wait();
   if (skip && *skip) return;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const double rh = dinv[i] * v[i];
@@ -556,6 +557,7 @@ __global__ void k_prep_rhat(int n, const double* __restrict__ v,
 template <typename GT>
 __global__ void k_rhat_update(int n, const GT* __restrict__ rhat, double* x, double omega,
                               int add, const int* skip) {
+  pdl_wait();
   if (skip && *skip) return;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const double u = omega * (double)rhat[i];
@@ -567,6 +569,7 @@ __global__ void k_rhat_update(int n, const GT* __restrict__ rhat, double* x, dou
 // iterate x32 + omega rhat (or omega rhat), to x32 or converted to x
 __global__ void k_rhat_update32(int n, const float* __restrict__ rhat, float* x32, double* x,
                                 float omega, int mode, const int* skip) {
+  pdl_wait();
   if (skip && *skip) return;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const float u = omega * rhat[i];
@@ -578,6 +581,7 @@ __global__ void k_rhat_update32(int n, const float* __restrict__ rhat, float* x3
 }
 
 __global__ void k_to32(int n, const double* __restrict__ x, float* x32, const int* skip) {
+  pdl_wait();
   if (skip && *skip) return;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
     x32[i] = (float)x[i];
@@ -611,6 +615,7 @@ __global__ void k_values_to_fp16(int n, const int* __restrict__ rp, const double
 
 __global__ void k_axpy(int n, double* y, double a, const double* __restrict__ x,
                        const int* skip) {
+  pdl_wait();
   if (skip && *skip) return;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
     y[i] += a * x[i];
@@ -626,8 +631,8 @@ void launch_prep_rhat(gs2_handle* h, const double* v, double* rhat64, float* rha
                       const int* skip) {
   if (h->n == 0) return;
   KernelTimer tm(h, "prep_rhat", 16.0 * h->n + (rhat64 ? 8.0 : 4.0) * h->n);
-  k_prep_rhat<<<vec_blocks(h, h->n), kVecThreads, 0, h->stream>>>(
-      (int)h->n, v, h->dinv, rhat64, rhat32, skip);
+  launch_pdl(k_prep_rhat, vec_blocks(h, h->n), kVecThreads, 0, h->stream, (int)h->n, v, h->dinv,
+             rhat64, rhat32, skip);
   GS2_LAUNCH_CHECK();
 }
 
@@ -637,11 +642,11 @@ void launch_rhat_update(gs2_handle* h, int prec, const void* rhat, double* x, do
   KernelTimer tm(h, "rhat_update", (prec == GS2_FP64 ? 8.0 : 4.0) * h->n +
                  (add ? 16.0 : 8.0) * h->n);
   if (prec == GS2_FP64)
-    k_rhat_update<double><<<vec_blocks(h, h->n), kVecThreads, 0, h->stream>>>(
-        (int)h->n, (const double*)rhat, x, omega, add ? 1 : 0, skip);
+    launch_pdl(k_rhat_update<double>, vec_blocks(h, h->n), kVecThreads, 0, h->stream, (int)h->n,
+               (const double*)rhat, x, omega, add ? 1 : 0, skip);
   else
-    k_rhat_update<float><<<vec_blocks(h, h->n), kVecThreads, 0, h->stream>>>(
-        (int)h->n, (const float*)rhat, x, omega, add ? 1 : 0, skip);
+    launch_pdl(k_rhat_update<float>, vec_blocks(h, h->n), kVecThreads, 0, h->stream, (int)h->n,
+               (const float*)rhat, x, omega, add ? 1 : 0, skip);
   GS2_LAUNCH_CHECK();
 }
 
@@ -652,8 +657,8 @@ void launch_rhat_update32(gs2_handle* h, const float* rhat, double* x, double om
   const bool out = mode == INNER_LAST_ADD32_OUT || mode == INNER_LAST_SET32_OUT;
   KernelTimer tm(h, "rhat_update", 4.0 * h->n + (add ? 4.0 : 0.0) * h->n +
                  (out ? 8.0 : 4.0) * h->n);
-  k_rhat_update32<<<vec_blocks(h, h->n), kVecThreads, 0, h->stream>>>(
-      (int)h->n, rhat, h->x32, x, (float)omega, mode, skip);
+  launch_pdl(k_rhat_update32, vec_blocks(h, h->n), kVecThreads, 0, h->stream, (int)h->n, rhat,
+             h->x32, x, (float)omega, mode, skip);
   GS2_LAUNCH_CHECK();
 }
 
@@ -672,14 +677,14 @@ void launch_values_to_fp16(gs2_handle* h, const DevCsr& M) {
 void launch_to32(gs2_handle* h, const double* x, float* x32, const int* skip) {
   if (h->n == 0) return;
   KernelTimer tm(h, "to32", 12.0 * h->n);
-  k_to32<<<vec_blocks(h, h->n), kVecThreads, 0, h->stream>>>((int)h->n, x, x32, skip);
+  launch_pdl(k_to32, vec_blocks(h, h->n), kVecThreads, 0, h->stream, (int)h->n, x, x32, skip);
   GS2_LAUNCH_CHECK();
 }
 
 void launch_axpy(gs2_handle* h, double* y, double a, const double* x, const int* skip) {
   if (h->n == 0) return;
   KernelTimer tm(h, "axpy", 24.0 * h->n);
-  k_axpy<<<vec_blocks(h, h->n), kVecThreads, 0, h->stream>>>((int)h->n, y, a, x, skip);
+  launch_pdl(k_axpy, vec_blocks(h, h->n), kVecThreads, 0, h->stream, (int)h->n, y, a, x, skip);
   GS2_LAUNCH_CHECK();
 }
 

@@ -182,6 +182,7 @@ __global__ void k_scale_next(int n, const double* __restrict__ w, double* vnext,
 // y = R^{-1} g over the k steps of the cycle (backsolve_block)
 __global__ void k_backsolve(const double* __restrict__ H, int ldh, const double* gv, double* y,
                             const KrylovState* st) {
+  pdl_wait();
   backsolve_block(H, ldh, gv, y, st->k);
 }
 
@@ -191,6 +192,7 @@ __global__ void __launch_bounds__(kVecThreads)
 k_combine(int n, const double* __restrict__ V, const double* __restrict__ y, double* u,
           const double* __restrict__ dinv, double* rhat64, float* rhat32,
           const KrylovState* st) {
+  pdl_wait();
   __shared__ double ys[MAXK];
   const int k = st->k;
   for (int i = threadIdx.x; i < MAXK; i += blockDim.x) ys[i] = i < k ? y[i] : 0.0;
@@ -199,28 +201,35 @@ k_combine(int n, const double* __restrict__ V, const double* __restrict__ y, dou
                      k, u, dinv, rhat64, rhat32);
 }
 
-// per-block partial sums of x^T x
-__global__ void __launch_bounds__(kVecThreads)
-k_norm_part(int n, const double* __restrict__ x, double* part, int nblk) {
-  double acc[1] = {0.0};
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    acc[0] = fma(x[i], x[i], acc[0]);
-  block_partials<1>(acc, 1, part, nblk);
+// Vector kernels that end in one sum: two blocks of 512 threads per SM with
+// several rows in flight per thread, so that the partials are few enough for
+// the kernel that needs the sum to add them up itself (sum_partials).
+constexpr int kSumThreads = 512;
+static int sum_blocks(const gs2_handle* h) {
+  return (int)std::max<int64_t>(
+      1, std::min<int64_t>((h->n + kSumThreads - 1) / kSumThreads, 2 * (int64_t)h->nsm));
+}
+
+// per-block partial sums of a^T b
+__global__ void __launch_bounds__(kSumThreads, 2)
+k_dot_part(int n, const double* __restrict__ a, const double* __restrict__ b, double* part,
+           const int* skip) {
+  pdl_wait();
+  if (skip && *skip) return;
+  double s = 0.0;
+#pragma unroll 4
+  for (int i = blockIdx.x * kSumThreads + threadIdx.x; i < n; i += gridDim.x * kSumThreads)
+    s = fma(a[i], b[i], s);
+  s = block_total<kSumThreads>(s);
+  if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
 
 // beta = sqrt(sum part) into st->beta (which = 0) or st->bnorm (which = 1)
 __global__ void k_norm_final(const double* __restrict__ part, int nblk, KrylovState* st,
                              int which) {
-  __shared__ double red[32];
-  double s = 0.0;
-  for (int b = threadIdx.x; b < nblk; b += blockDim.x) s += part[b];
-  s = warp_sum(s);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) red[wid] = s;
-  __syncthreads();
+  pdl_wait();
+  const double t = sum_partials(part, nblk);
   if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
     if (which == 0) st->beta = sqrt(t);
     else st->bnorm = sqrt(t);
   }
@@ -230,6 +239,7 @@ __global__ void k_norm_final(const double* __restrict__ part, int nblk, KrylovSt
 __global__ void k_cycle_start(int n, const double* __restrict__ r, double* v0,
                               const double* __restrict__ dinv, double* rhat64, float* rhat32,
                               double* gv, int m, KrylovState* st) {
+  pdl_wait();
   const double beta = st->beta;
   scale_rows(blockIdx.x * blockDim.x + threadIdx.x, n, gridDim.x * blockDim.x, 1.0 / beta, r, v0,
              dinv, rhat64, rhat32);
@@ -238,6 +248,7 @@ __global__ void k_cycle_start(int n, const double* __restrict__ r, double* v0,
 }
 
 __global__ void k_state_init(KrylovState* st, double tol, int max_iters) {
+  pdl_wait();
   st->stop = 0;
   st->status = GS2_OK;
   st->k = 0;
@@ -247,6 +258,7 @@ __global__ void k_state_init(KrylovState* st, double tol, int max_iters) {
 }
 
 __global__ void k_cycle_reset(KrylovState* st) {
+  pdl_wait();
   st->stop = 0;
   st->k = 0;
 }
@@ -382,19 +394,25 @@ static void launch_combine(gs2_handle* h, int m, double* u, double* r64, float* 
   KernelTimer tm(h, "combine", 8.0 * h->n * (m + 1));
   const int n = (int)h->n, nb = h->nblk;
   switch (maxk_for(m)) {
-    case 8: k_combine<8><<<nb, kVecThreads, 0, h->stream>>>(n, h->V, h->y, u, h->dinv, r64, r32, h->st); break;
-    case 16: k_combine<16><<<nb, kVecThreads, 0, h->stream>>>(n, h->V, h->y, u, h->dinv, r64, r32, h->st); break;
-    case 32: k_combine<32><<<nb, kVecThreads, 0, h->stream>>>(n, h->V, h->y, u, h->dinv, r64, r32, h->st); break;
-    default: k_combine<64><<<nb, kVecThreads, 0, h->stream>>>(n, h->V, h->y, u, h->dinv, r64, r32, h->st); break;
+    case 8: launch_pdl(k_combine<8>, nb, kVecThreads, 0, h->stream, n, h->V, h->y, u, h->dinv, r64,
+             r32, h->st); break;
+    case 16: launch_pdl(k_combine<16>, nb, kVecThreads, 0, h->stream, n, h->V, h->y, u, h->dinv,
+             r64, r32, h->st); break;
+    case 32: launch_pdl(k_combine<32>, nb, kVecThreads, 0, h->stream, n, h->V, h->y, u, h->dinv,
+             r64, r32, h->st); break;
+    default: launch_pdl(k_combine<64>, nb, kVecThreads, 0, h->stream, n, h->V, h->y, u, h->dinv,
+             r64, r32, h->st); break;
   }
   GS2_LAUNCH_CHECK();
 }
 
 static void launch_norm(gs2_handle* h, const double* x, int which) {
   KernelTimer tm(h, "norm", 8.0 * h->n);
-  k_norm_part<<<h->nblk_dot, kVecThreads, 0, h->stream>>>((int)h->n, x, h->part, h->nblk_dot);
+  const int nb = sum_blocks(h);
+  launch_pdl(k_dot_part, nb, kSumThreads, 0, h->stream, (int)h->n, x, x, h->part,
+             (const int*)nullptr);
   GS2_LAUNCH_CHECK();
-  k_norm_final<<<1, 256, 0, h->stream>>>(h->part, h->nblk_dot, h->st, which);
+  launch_pdl(k_norm_final, 1, 32, 0, h->stream, (const double*)h->part, nb, h->st, which);
   GS2_LAUNCH_CHECK();
 }
 
@@ -463,7 +481,7 @@ struct GmresRun {
       else r64 = (double*)rb;
     }
     launch_norm(h, b, 1);
-    k_state_init<<<1, 1, 0, h->stream>>>(h->st, tol, max_iters);
+    launch_pdl(k_state_init, 1, 1, 0, h->stream, h->st, tol, max_iters);
     GS2_LAUNCH_CHECK();
     launch_true_residual();
   }
@@ -637,10 +655,10 @@ struct GmresRun {
     const int n = (int)h->n;
     const int ldh = m + 1;
     *h->stop_mapped = 0;
-    k_cycle_reset<<<1, 1, 0, h->stream>>>(h->st);
+    launch_pdl(k_cycle_reset, 1, 1, 0, h->stream, h->st);
     GS2_LAUNCH_CHECK();
-    k_cycle_start<<<vec_blocks(h, n), kVecThreads, 0, h->stream>>>(n, h->r, h->V, h->dinv, r64,
-                                                                  r32, h->gvec, m, h->st);
+    launch_pdl(k_cycle_start, vec_blocks(h, n), kVecThreads, 0, h->stream, n, h->r, h->V, h->dinv,
+               r64, r32, h->gvec, m, h->st);
     GS2_LAUNCH_CHECK();
     cycle_ran = true;
     if (use_graph()) {
@@ -655,7 +673,7 @@ struct GmresRun {
       profile_capture_step(h, -1);
     }
     // x += M^{-1} V y
-    k_backsolve<<<1, 64, 0, h->stream>>>(h->H, ldh, h->gvec, h->y, h->st);
+    launch_pdl(k_backsolve, 1, 64, 0, h->stream, h->H, ldh, h->gvec, h->y, h->st);
     GS2_LAUNCH_CHECK();
     launch_combine(h, m, h->w, r64, r32);
     precond_apply(h, pc, h->w, h->z, wants, nullptr);
@@ -887,99 +905,82 @@ gs2_status gmres_batch(gs2_handle* const* hs, const double* const* bs, double* c
 // preconditioned CG
 // ---------------------------------------------------------------------------
 
-// part = [p.q partials]
-__global__ void __launch_bounds__(kVecThreads)
-k_dot_part(int n, const double* __restrict__ a, const double* __restrict__ b, double* part,
-           int nblk, const int* skip) {
-  if (skip && *skip) return;
-  double acc[1] = {0.0};
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    acc[0] = fma(a[i], b[i], acc[0]);
-  block_partials<1>(acc, 1, part, nblk);
+// An iteration is the row kernels of A p and of the preconditioner and four
+// vector kernels.  The scalars have no kernels of their own: each block of the
+// kernel that needs one sums the partials of the kernel before (sum_partials),
+// alpha in k_cg_xr, beta and the stopping test in k_cg_p.  The residual test
+// comes after the preconditioner, whose last application is then not used.
+
+// r.z of a (re)started search direction
+__global__ void k_cg_start(const double* __restrict__ part, int nblk, KrylovState* st) {
+  pdl_wait();
+  const double t = sum_partials(part, nblk);
+  if (threadIdx.x == 0) st->rz[0] = t;
 }
 
-// reduce part into a scalar: what = 0 -> alpha = rz / (p.q) (breakdown if
-// p.q == 0); what = 1 -> beta_cg = rz_new / rz, rz = rz_new (stored in hn)
-__global__ void k_cg_scalar(const double* __restrict__ part, int nblk, KrylovState* st,
-                            int what, const int* skip) {
+// alpha = r.z / p.q from the partials of p.q (breakdown if that is 0);
+// x += alpha p ; r -= alpha q ; partials of r.r ; and the preconditioner's
+// D^{-1} r in its sweep precision (whichever of rhat64, rhat32 is non-null)
+__global__ void __launch_bounds__(kSumThreads, 2)
+k_cg_xr(int n, double* __restrict__ x, double* __restrict__ r, const double* __restrict__ p,
+        const double* __restrict__ q, const double* __restrict__ part_pq, double* part_rr,
+        int nblk, KrylovState* st, int parity, volatile int* stop_host, const int* skip,
+        const double* __restrict__ dinv, double* __restrict__ rhat64,
+        float* __restrict__ rhat32) {
+  pdl_wait();
   if (skip && *skip) return;
-  __shared__ double red[32];
-  double s = 0.0;
-  for (int b = threadIdx.x; b < nblk; b += blockDim.x) s += part[b];
-  s = warp_sum(s);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) red[wid] = s;
-  __syncthreads();
-  if (threadIdx.x != 0) return;
-  double t = 0.0;
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-  if (what == 0) {
-    if (t == 0.0) {
+  const double pq = sum_partials(part_pq, nblk);
+  if (pq == 0.0) {
+    // (every block sees it, or the flag)
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
       st->status = GS2_ERR_BREAKDOWN;
       st->stop = 1;
-      return;
+      *stop_host = 1;
     }
-    st->alpha = st->rz / t;
-  } else if (what == 1) {
-    st->hn = t / st->rz;  // beta of CG
-    st->rz = t;
-  } else {
-    st->rz = t;
+    return;
   }
-}
-
-// x += alpha p ; r -= alpha q ; part = r.r ; and the preconditioner's
-// D^{-1} r in its sweep precision (whichever of rhat64, rhat32 is non-null)
-__global__ void __launch_bounds__(kVecThreads)
-k_cg_xr(int n, double* x, double* r, const double* __restrict__ p, const double* __restrict__ q,
-        double* part, int nblk, const KrylovState* st, const int* skip,
-        const double* __restrict__ dinv, double* rhat64, float* rhat32) {
-  if (skip && *skip) return;
-  const double a = st->alpha;
-  double acc[1] = {0.0};
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+  const double a = st->rz[parity] / pq;
+  double s = 0.0;
+#pragma unroll 2
+  for (int i = blockIdx.x * kSumThreads + threadIdx.x; i < n; i += gridDim.x * kSumThreads) {
     x[i] = fma(a, p[i], x[i]);
     const double ri = fma(-a, q[i], r[i]);
     r[i] = ri;
-    acc[0] = fma(ri, ri, acc[0]);
+    s = fma(ri, ri, s);
     if (rhat64) rhat64[i] = dinv[i] * ri;
     if (rhat32) rhat32[i] = (float)(dinv[i] * ri);
   }
-  block_partials<1>(acc, 1, part, nblk);
+  s = block_total<kSumThreads>(s);
+  if (threadIdx.x == 0) part_rr[blockIdx.x] = s;
 }
 
-// ||r|| test after an iteration: stop the loop of launches when converged
-__global__ void k_cg_check(const double* __restrict__ part, int nblk, KrylovState* st,
-                           volatile int* stop_host, const int* skip) {
+// beta = r.z / (r.z before) ; p = z + beta p ; the ||r|| test of the iteration
+// (block 0; p is not used again once it stops the loop of launches)
+__global__ void __launch_bounds__(kSumThreads, 2)
+k_cg_p(int n, double* __restrict__ p, const double* __restrict__ z,
+       const double* __restrict__ part_rr, const double* __restrict__ part_rz, int nblk,
+       KrylovState* st, int parity, volatile int* stop_host, const int* skip) {
+  pdl_wait();
   if (skip && *skip) return;
-  __shared__ double red[32];
-  double s = 0.0;
-  for (int b = threadIdx.x; b < nblk; b += blockDim.x) s += part[b];
-  s = warp_sum(s);
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  if (lane == 0) red[wid] = s;
-  __syncthreads();
-  if (threadIdx.x != 0) return;
-  double t = 0.0;
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-  const double rn = sqrt(t);
-  st->iters += 1;
-  st->beta = rn;
-  if (isnan(rn) || isinf(rn)) {
-    st->status = GS2_ERR_NAN;
-    st->stop = 1;
-  } else if (rn <= st->tol_abs || st->iters >= st->max_iters) {
-    st->stop = 1;
+  const double rz = sum_partials(part_rz, nblk);
+  const double bt = rz / st->rz[parity];
+  if (blockIdx.x == 0) {
+    const double rn = sqrt(sum_partials(part_rr, nblk));
+    if (threadIdx.x == 0) {
+      st->rz[parity ^ 1] = rz;
+      st->iters += 1;
+      st->beta = rn;
+      if (isnan(rn) || isinf(rn)) {
+        st->status = GS2_ERR_NAN;
+        st->stop = 1;
+      } else if (rn <= st->tol_abs || st->iters >= st->max_iters) {
+        st->stop = 1;
+      }
+      if (st->stop) *stop_host = 1;
+    }
   }
-  if (st->stop) *stop_host = 1;
-}
-
-// p = z + beta p
-__global__ void k_cg_p(int n, double* p, const double* __restrict__ z, const KrylovState* st,
-                       const int* skip) {
-  if (skip && *skip) return;
-  const double bt = st->hn;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+#pragma unroll 4
+  for (int i = blockIdx.x * kSumThreads + threadIdx.x; i < n; i += gridDim.x * kSumThreads)
     p[i] = fma(bt, p[i], z[i]);
 }
 
@@ -1005,15 +1006,17 @@ gs2_status cg_run(gs2_handle* h, const double* b, double* x, double tol, int max
   }
   ensure_krylov(h, 1);
   const gs2_params* pc = (p && p->kind != GS2_PC_NONE) ? p : nullptr;
-  const int n = (int)h->n, nb = h->nblk_dot;
+  const int n = (int)h->n, nb = sum_blocks(h);
   const int* skip = &h->st->stop;
+  // partials of p.q, r.r and r.z
+  double *part_pq = h->part, *part_rr = h->part + nb, *part_rz = h->part + 2 * nb;
   double* r = h->r;
   double* z = h->z;
   double* pv = h->p;
   double* q = h->q;
 
   launch_norm(h, b, 1);
-  k_state_init<<<1, 1, 0, h->stream>>>(h->st, tol, max_iters);
+  launch_pdl(k_state_init, 1, 1, 0, h->stream, h->st, tol, max_iters);
   GS2_LAUNCH_CHECK();
   read_state(h);
   const double bnorm = h->st_host->bnorm;
@@ -1032,18 +1035,25 @@ gs2_status cg_run(gs2_handle* h, const double* b, double* x, double tol, int max
     if (rb == (void*)h->rhat32 || rb == (void*)h->bhat32) r32 = (float*)rb;
     else r64 = (double*)rb;
   }
-  // one CG iteration (every kernel a no-op once the device has stopped)
-  auto enqueue_iter = [&]() {
+  // one CG iteration (every kernel a no-op once the device has stopped); the
+  // number of iterations per check is even, so an iteration's parity is that
+  // of its place among them
+  auto enqueue_iter = [&](int it) {
     launch_spmv(h, pv, q, skip);
-    k_dot_part<<<nb, kVecThreads, 0, h->stream>>>(n, pv, q, h->part, nb, skip);
-    k_cg_scalar<<<1, 256, 0, h->stream>>>(h->part, nb, h->st, 0, skip);
-    k_cg_xr<<<nb, kVecThreads, 0, h->stream>>>(n, x, r, pv, q, h->part, nb, h->st, skip,
-                                               h->dinv, r64, r32);
-    k_cg_check<<<1, 256, 0, h->stream>>>(h->part, nb, h->st, h->stop_mapped_dev, skip);
+    launch_pdl(k_dot_part, nb, kSumThreads, 0, h->stream, n, (const double*)pv, (const double*)q,
+               part_pq, skip);
+    GS2_LAUNCH_CHECK();
+    launch_pdl(k_cg_xr, nb, kSumThreads, 0, h->stream, n, x, r, (const double*)pv,
+               (const double*)q, (const double*)part_pq, part_rr, nb, h->st, it & 1,
+               (volatile int*)h->stop_mapped_dev, skip, (const double*)h->dinv, r64, r32);
+    GS2_LAUNCH_CHECK();
     precond_apply(h, pc, r, z, wants, skip);
-    k_dot_part<<<nb, kVecThreads, 0, h->stream>>>(n, r, z, h->part, nb, skip);
-    k_cg_scalar<<<1, 256, 0, h->stream>>>(h->part, nb, h->st, 1, skip);
-    k_cg_p<<<vec_blocks(h, n), kVecThreads, 0, h->stream>>>(n, pv, z, h->st, skip);
+    launch_pdl(k_dot_part, nb, kSumThreads, 0, h->stream, n, (const double*)r, (const double*)z,
+               part_rz, skip);
+    GS2_LAUNCH_CHECK();
+    launch_pdl(k_cg_p, nb, kSumThreads, 0, h->stream, n, pv, (const double*)z,
+               (const double*)part_rr, (const double*)part_rz, nb, h->st, it & 1,
+               (volatile int*)h->stop_mapped_dev, skip);
     GS2_LAUNCH_CHECK();
   };
   constexpr int kCheckEvery = 16;
@@ -1081,7 +1091,7 @@ gs2_status cg_run(gs2_handle* h, const double* b, double* x, double tol, int max
       try {
         for (int it = 0; it < kCheckEvery; ++it) {
           profile_capture_step(h, it);
-          enqueue_iter();
+          enqueue_iter(it);
         }
       } catch (...) {
         profile_capture_end(h);
@@ -1127,11 +1137,13 @@ gs2_status cg_run(gs2_handle* h, const double* b, double* x, double tol, int max
     }
     loc.cycles++;
     *h->stop_mapped = 0;
-    k_cycle_reset<<<1, 1, 0, h->stream>>>(h->st);
+    launch_pdl(k_cycle_reset, 1, 1, 0, h->stream, h->st);
     precond_apply(h, pc, r, z, false, nullptr);
     launch_copy(h, pv, z);
-    k_dot_part<<<nb, kVecThreads, 0, h->stream>>>(n, r, z, h->part, nb, nullptr);
-    k_cg_scalar<<<1, 256, 0, h->stream>>>(h->part, nb, h->st, 2, nullptr);
+    launch_pdl(k_dot_part, nb, kSumThreads, 0, h->stream, n, (const double*)r, (const double*)z,
+               part_rz, (const int*)nullptr);
+    GS2_LAUNCH_CHECK();
+    launch_pdl(k_cg_start, 1, 32, 0, h->stream, (const double*)part_rz, nb, h->st);
     GS2_LAUNCH_CHECK();
     for (;;) {
       const int before = h->st_host->iters;
@@ -1146,7 +1158,7 @@ gs2_status cg_run(gs2_handle* h, const double* b, double* x, double tol, int max
         for (int it = 0; it < kCheckEvery; ++it) {
           if (*h->stop_mapped) break;
           profile_capture_step(h, it);
-          enqueue_iter();
+          enqueue_iter(it);
         }
         profile_capture_step(h, -1);
       }

@@ -13,6 +13,44 @@ __device__ __forceinline__ double warp_sum(double s) {
   return s;
 }
 
+// Sum of the partial sums part[0 .. nblk) in every thread of the block, by
+// its first warp: a fixed order, so that every block and every kernel that
+// sums them gets the same bits.  (Two blocks per SM that sum 304 partials out
+// of L2 spend about 1 us at their start; a kernel of its own between producer
+// and consumers costs 3 to 4.  Summed by all warps of eight blocks per SM the
+// FP64 adds alone took 5 us.)
+__device__ __forceinline__ double sum_partials(const double* __restrict__ part, int nblk) {
+  __shared__ double total;
+  __syncthreads();  // total may still be read from an earlier call
+  if (threadIdx.x < 32) {
+    double s = 0.0;
+#pragma unroll 4
+    for (int b = threadIdx.x; b < nblk; b += 32) s += part[b];
+    s = warp_sum(s);
+    if (threadIdx.x == 0) total = s;
+  }
+  __syncthreads();
+  return total;
+}
+
+// Sum of v over a block of T threads, valid in thread 0: the values through
+// shared memory, then T / 32 adds a lane and one shuffle tree in the first
+// warp -- a tree in every warp would issue five FP64 instructions each on a
+// pipe that takes 16 cycles an instruction.
+template <int T>
+__device__ __forceinline__ double block_total(double v) {
+  __shared__ double vals[T];
+  vals[threadIdx.x] = v;
+  __syncthreads();
+  double s = 0.0;
+  if (threadIdx.x < 32) {
+#pragma unroll
+    for (int w = 0; w < T / 32; ++w) s += vals[threadIdx.x + 32 * w];
+    s = warp_sum(s);
+  }
+  return s;
+}
+
 template <int N>
 struct Pow2 {
   static constexpr int value = N <= 1 ? 1 : 2 * Pow2<(N + 1) / 2>::value;

@@ -8,19 +8,21 @@
 namespace gs2 {
 
 __global__ void k_fill(int n, double* y, double v, const int* skip) {
+  pdl_wait();
   if (skip && *skip) return;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
     y[i] = v;
 }
 
 __global__ void k_copy(int n, double* y, const double* __restrict__ x, const int* skip) {
+  pdl_wait();
   if (skip && *skip) return;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
     y[i] = x[i];
 }
 
 static void launch_fill(gs2_handle* h, double* y, double v, const int* skip) {
-  k_fill<<<vec_blocks(h, h->n), kVecThreads, 0, h->stream>>>((int)h->n, y, v, skip);
+  launch_pdl(k_fill, vec_blocks(h, h->n), kVecThreads, 0, h->stream, (int)h->n, y, v, skip);
   GS2_LAUNCH_CHECK();
 }
 
@@ -28,7 +30,7 @@ void launch_fill_value(gs2_handle* h, double* y, double v) { launch_fill(h, y, v
 
 static void launch_copy_skip(gs2_handle* h, double* y, const double* x, const int* skip) {
   KernelTimer tm(h, "copy", 16.0 * h->n);
-  k_copy<<<vec_blocks(h, h->n), kVecThreads, 0, h->stream>>>((int)h->n, y, x, skip);
+  launch_pdl(k_copy, vec_blocks(h, h->n), kVecThreads, 0, h->stream, (int)h->n, y, x, skip);
   GS2_LAUNCH_CHECK();
 }
 
