@@ -185,7 +185,7 @@ gs2_status gs2_autotune(gs2_handle* h);
  * FP64 non-compact GS2, per-kernel profiling off) the whole solve in one
  * kernel -- inside one thread-block cluster as in mode 4 when the system's
  * rows fit its shared memory, else as one cooperative launch whose blocks
- * meet at bounded grid barriers (n <= 16,384) -- every restart cycle,
+ * meet at bounded grid barriers (GMRES n <= 8,192, CG n <= 16,384) -- every restart cycle,
  * preconditioner application and Givens step included; otherwise as in
  * mode 1; 1 = each restart cycle's steps
  * as one replayed CUDA graph; 2 = as separate launches; 3 = the one-launch

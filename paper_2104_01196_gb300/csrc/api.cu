@@ -425,11 +425,13 @@ static void upload_sell(gs2_handle* h, DevCsr& M, const std::vector<int>& rp, co
   const std::vector<int>& cptr = sliced ? lay.cptr : lanes.cptr;
   const size_t slots = std::max(cptr.back(), 1);
   std::vector<int> top(kHostThreads, 0);
-  parallel_ranges(M.nnz, [&](int64_t k0, int64_t k1, int t) {
+  auto largest = [&](int64_t k0, int64_t k1, int t) {
     int v = 0;
     for (int64_t k = k0; k < k1; ++k) v = std::max(v, ci[k]);
     top[t] = v;
-  });
+  };
+  if (M.nnz < (1 << 22)) largest(0, M.nnz, 0);  // (sooner done than threads are started)
+  else parallel_ranges(M.nnz, largest);
   const int ncols = 1 + *std::max_element(top.begin(), top.end());
   M.sell_chunks = (int)cptr.size() - 1;
   M.sell_slots = (int)slots;

@@ -487,7 +487,7 @@ gs2_status gmres_batch(gs2_handle* const* hs, const double* const* bs,
 void read_state(gs2_handle* h);
 
 // GMRES(m) of a small system as one cooperative launch (persist.cu): n up
-// to 65,536 rows (16,384 when chosen automatically), m <= 32, no
+// to 65,536 rows (16,384 at most when chosen automatically), m <= 32, no
 // preconditioner, FP64 non-compact GS2 or JR
 bool persistent_eligible(const gs2_handle* h, int m, const gs2_params* p, bool automatic);
 void longest_rows(gs2_handle* h);

@@ -311,14 +311,17 @@ static int maxk_for(int jc) {
   X(31) X(32)
 
 // Grid of a reduction kernel: at most `per_sm_max` blocks per SM (0 = as
-// many as stay resident, queried once per instantiation), at least ~8 rows
-// per thread, no more blocks than the partial-sum buffer holds, and a whole
-// multiple of the SM count when there are at least that many (even load per
-// SM).  The dot-product pass (one FMA per loaded value) is latency-bound and
-// wants every resident warp; the update passes (two FMAs per value for
-// w -= Vh, V^T w) are bound by the FP64 pipe and ran fastest at two blocks
-// per SM, the update-and-norm pass at three (measured at n = 2.1M), where the
-// per-block butterfly reductions stay a few percent of the work.
+// many as stay resident, queried once per instantiation), no more blocks than
+// the partial-sum buffer holds, and a whole multiple of the SM count when
+// there are at least that many (even load per SM).  Up to one block per SM a
+// row per thread is enough, beyond that four: the block's butterfly reduction
+// costs about as much on the FP64 pipe as a few rows.  (At eight rows per
+// thread everywhere, 185,193 rows kept 91 of the 152 SMs busy, 20 to 27 us a
+// pass at 16 basis vectors; GMRES per Arnoldi step 72 -> 62 us, at 27,000
+// rows 61 -> 39.)  The dot-product pass (one FMA per loaded value) is
+// latency-bound and wants every resident warp; the update passes (two FMAs
+// per value for w -= Vh, V^T w) are bound by the FP64 pipe and ran fastest at
+// two blocks per SM, the update-and-norm pass at three (measured at n = 2.1M).
 constexpr int kDotBlocksPerSm = 0, kUpdBlocksPerSm = 2, kNormBlocksPerSm = 3;
 static int reduction_grid(gs2_handle* h, const void* fn, int per_sm_max) {
   static std::mutex mu;
@@ -335,7 +338,8 @@ static int reduction_grid(gs2_handle* h, const void* fn, int per_sm_max) {
     per_sm = it->second;
   }
   if (per_sm_max > 0) per_sm = std::min(per_sm, per_sm_max);
-  const int64_t want = (h->n + kVecThreads * 8 - 1) / (kVecThreads * 8);
+  auto blocks = [&](int rows) { return (h->n + kVecThreads * rows - 1) / (kVecThreads * rows); };
+  const int64_t want = std::max(std::min<int64_t>(blocks(1), h->nsm), blocks(4));
   int64_t nb = std::min<int64_t>({want, (int64_t)per_sm * h->nsm, (int64_t)h->nblk});
   if (nb >= h->nsm) nb -= nb % h->nsm;
   return (int)std::max<int64_t>(1, nb);
@@ -787,6 +791,13 @@ int autotune_gmres(gs2_handle* h, int m, const gs2_params* p) {
   return best;
 }
 
+// GMRES: one launch up to this size where one cluster does not take the
+// system, cycle graphs above (CG: up to kPersistAutoRows).  Measured with
+// SGS2(1,1): 8,000 rows of convection-diffusion, 14 iterations, 575 us in one
+// launch and 616 as a graph, half of whose 30 steps run as no-ops; 15,625 rows
+// 726 and 643; 10,000 rows of the 2D Laplacian, 54 iterations, 2479 and 1840.
+constexpr int64_t kGmresOneLaunchRows = 8192;
+
 static gs2_status gmres_run_mode(gs2_handle* h, const double* b, double* x, int m, double tol,
                                  int max_iters, const gs2_params* p, gs2_solve_info* info) {
   // small systems: the whole solve inside one cluster when its rows fit the
@@ -796,7 +807,8 @@ static gs2_status gmres_run_mode(gs2_handle* h, const double* b, double* x, int 
   if (h->graph_mode == 4 || (automatic && cluster_eligible(h, m, p)))
     return gmres_cluster(h, b, x, m, tol, max_iters, p, info);
   const bool forced = h->graph_mode == 3;
-  if ((forced || automatic) && persistent_eligible(h, m, p, !forced))
+  if ((forced || (automatic && h->n <= kGmresOneLaunchRows)) &&
+      persistent_eligible(h, m, p, !forced))
     return gmres_persistent(h, b, x, m, tol, max_iters, p, info);
   if (h->graph_mode == 3)
     GS2_THROW(GS2_ERR_INVALID_ARG, "the one-launch solver takes n <= 65536, restart <= 32 and "

@@ -89,6 +89,7 @@ __global__ void __launch_bounds__(kVecThreads)
 k_pdots(int ld, const int4* __restrict__ blk, const int* __restrict__ items,
         const int* __restrict__ nitems, const KrylovState* st, const double* __restrict__ V,
         const double* __restrict__ w, double* part, int nb) {
+  pdl_wait();
   const int nq = *nitems;
   for (int q = blockIdx.x; q < nq; q += gridDim.x) {
     const int e = items[q];
@@ -110,6 +111,7 @@ k_pupdate(int ld, const int4* __restrict__ blk, const int* __restrict__ items,
           const int* __restrict__ nitems, const KrylovState* st, const double* __restrict__ V,
           const double* __restrict__ hbuf, int hb_stride, double* __restrict__ w, double* part,
           int nb) {
+  pdl_wait();
   __shared__ double hneg[JC];
   const int nq = *nitems;
   for (int q = blockIdx.x; q < nq; q += gridDim.x) {
@@ -135,6 +137,7 @@ __global__ void __launch_bounds__(kVecThreads)
 k_pdots_rt(int ld, const int4* __restrict__ blk, const int* __restrict__ items,
            const int* __restrict__ nitems, const KrylovState* st, const double* __restrict__ V,
            int jc, const double* __restrict__ w, double* part, int nb) {
+  pdl_wait();
   const int nq = *nitems;
   for (int q = blockIdx.x; q < nq; q += gridDim.x) {
     const int e = items[q];
@@ -160,6 +163,7 @@ k_pupdate_rt(int ld, const int4* __restrict__ blk, const int* __restrict__ items
              const int* __restrict__ nitems, const KrylovState* st,
              const double* __restrict__ V, int jc, const double* __restrict__ hbuf,
              int hb_stride, double* w, double* part, int nb) {
+  pdl_wait();
   __shared__ double hneg[MAXK];
   const int nq = *nitems;
   for (int q = blockIdx.x; q < nq; q += gridDim.x) {
@@ -199,6 +203,7 @@ __global__ void k_preduce(const double* __restrict__ part, int nb, const int* __
                           const int* __restrict__ sys, const int* __restrict__ nsys,
                           const KrylovState* st, double* H, size_t hstride, int ldh, int j,
                           double* hbuf, int hb_stride, int mode, int jc) {
+  pdl_wait();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int nq = *nsys;
   for (int q = blockIdx.x; q < nq; q += gridDim.x) {
@@ -228,6 +233,7 @@ __global__ void k_pgivens(const double* __restrict__ part, const int* __restrict
                           double* cs, double* sn, double* gv, int vstride, int* nactive,
                           const int* __restrict__ off, int* live_run, KrylovState* pack_st,
                           volatile int* stop_host) {
+  pdl_wait();
   const int nq = *nsys;
   for (int q = blockIdx.x; q < nq; q += gridDim.x) {
     const int s = sys[q];
@@ -264,6 +270,7 @@ __device__ __forceinline__ int system_of(const int* __restrict__ off, int count,
 // 32-row chunk that take the cycle
 __global__ void k_plive_init(int nchunks, int n, const int* __restrict__ off, int count,
                              const int* __restrict__ active, int* live_cycle, int* live_run) {
+  pdl_wait();
   for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < nchunks; c += gridDim.x * blockDim.x) {
     const int s0 = system_of(off, count, 32 * c);
     const int s1 = system_of(off, count, min(32 * c + 31, n - 1));
@@ -278,6 +285,7 @@ __global__ void k_plive_init(int nchunks, int n, const int* __restrict__ off, in
 __global__ void __launch_bounds__(kVecThreads)
 k_paxpy(const int4* __restrict__ blk, const int* __restrict__ items,
         const int* __restrict__ nitems, double* x, const double* __restrict__ z) {
+  pdl_wait();
   const int nq = *nitems;
   for (int q = blockIdx.x; q < nq; q += gridDim.x) {
     const int4 b = blk[items[q]];
@@ -291,6 +299,7 @@ k_pscale_next(const int4* __restrict__ blk, const int* __restrict__ items,
               const int* __restrict__ nitems, const KrylovState* st,
               const double* __restrict__ w, double* vnext, const double* __restrict__ dinv,
               double* rhat64, float* rhat32) {
+  pdl_wait();
   const int nq = *nitems;
   for (int q = blockIdx.x; q < nq; q += gridDim.x) {
     const int4 b = blk[items[q]];
@@ -305,6 +314,7 @@ __global__ void __launch_bounds__(kVecThreads)
 k_pnorm_part(const int4* __restrict__ blk, const int* __restrict__ items,
              const int* __restrict__ nitems, const double* __restrict__ x, double* part,
              int nb) {
+  pdl_wait();
   const int nq = *nitems;
   for (int q = blockIdx.x; q < nq; q += gridDim.x) {
     const int e = items[q];
@@ -321,6 +331,7 @@ k_pnorm_part(const int4* __restrict__ blk, const int* __restrict__ items,
 __global__ void k_pnorm_final(const double* __restrict__ part, const int* __restrict__ seg_blk,
                               const int* __restrict__ sys, const int* __restrict__ nsys,
                               KrylovState* st, int which) {
+  pdl_wait();
   __shared__ double red[32];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int nq = *nsys;
@@ -342,6 +353,7 @@ __global__ void k_pnorm_final(const double* __restrict__ part, const int* __rest
 }
 
 __global__ void k_pstate_init(KrylovState* st, int count, double tol, int max_iters) {
+  pdl_wait();
   for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < count; s += gridDim.x * blockDim.x) {
     KrylovState& q = st[s];
     q.stop = 0;
@@ -357,6 +369,7 @@ __global__ void k_pstate_init(KrylovState* st, int count, double tol, int max_it
 // nactive counts the others.
 __global__ void k_pcycle_reset(KrylovState* st, const int* __restrict__ active, int count,
                                int* nactive, KrylovState* pack_st) {
+  pdl_wait();
   __shared__ int cnt;
   if (threadIdx.x == 0) cnt = 0;
   __syncthreads();
@@ -382,6 +395,7 @@ k_pcycle_start(const int4* __restrict__ blk, const int* __restrict__ items,
                const int* __restrict__ nitems, const KrylovState* st,
                const double* __restrict__ r, double* v0, const double* __restrict__ dinv,
                double* rhat64, float* rhat32, double* gv, int vstride, int m) {
+  pdl_wait();
   const int nq = *nitems;
   for (int q = blockIdx.x; q < nq; q += gridDim.x) {
     const int4 b = blk[items[q]];
@@ -399,6 +413,7 @@ __global__ void k_pbacksolve(const double* __restrict__ H, size_t hstride, int l
                              const double* gv, double* y, int vstride,
                              const int* __restrict__ sys, const int* __restrict__ nsys,
                              const KrylovState* st) {
+  pdl_wait();
   const int nq = *nsys;
   for (int q = blockIdx.x; q < nq; q += gridDim.x) {
     const int s = sys[q];
@@ -415,6 +430,7 @@ k_pcombine(int ld, const int4* __restrict__ blk, const int* __restrict__ items,
            const int* __restrict__ nitems, const KrylovState* st,
            const double* __restrict__ V, const double* __restrict__ y, int vstride, double* u,
            const double* __restrict__ dinv, double* rhat64, float* rhat32) {
+  pdl_wait();
   __shared__ double ys[MAXK];
   const int nq = *nitems;
   for (int q = blockIdx.x; q < nq; q += gridDim.x) {
@@ -642,7 +658,8 @@ struct PackRun {
     }
     upload_lists();  // every system
     launch_norms(b, 1);
-    k_pstate_init<<<(P->count + 255) / 256, 256, 0, h->stream>>>(P->st, P->count, tol, max_iters);
+    launch_pdl(k_pstate_init, (P->count + 255) / 256, 256, 0, h->stream, P->st, P->count, tol,
+               max_iters);
     GS2_LAUNCH_CHECK();
     launch_true_residual();
   }
@@ -671,11 +688,11 @@ struct PackRun {
   // per-system ||v|| into st.beta (which = 0) or st.bnorm (which = 1)
   void launch_norms(const double* v, int which) {
     KernelTimer tm(h, "norm", 8.0 * h->n);
-    k_pnorm_part<<<P->gb, kVecThreads, 0, h->stream>>>(P->blk, P->items, P->cnt, v, P->part,
-                                                       P->nb);
+    launch_pdl(k_pnorm_part, P->gb, kVecThreads, 0, h->stream, P->blk, P->items, P->cnt, v, P->part,
+               P->nb);
     GS2_LAUNCH_CHECK();
-    k_pnorm_final<<<P->gs, 256, 0, h->stream>>>(P->part, P->seg_blk, P->sys, P->cnt + 1, P->st,
-                                                which);
+    launch_pdl(k_pnorm_final, P->gs, 256, 0, h->stream, P->part, P->seg_blk, P->sys, P->cnt + 1, P->st,
+               which);
     GS2_LAUNCH_CHECK();
   }
 
@@ -763,15 +780,14 @@ struct PackRun {
     switch (jc) {
 #define GS2_PDOTS_CASE(J)                                                               \
   case J:                                                                               \
-    k_pdots<J><<<P->gb, kVecThreads, 0, h->stream>>>(N, P->blk, P->items, P->cnt, P->st, \
-                                                     h->V, h->w, P->part, P->nb);       \
+    launch_pdl(k_pdots<J>, P->gb, kVecThreads, 0, h->stream, N, P->blk, P->items, P->cnt, P->st, h->V,  \
+               h->w, P->part, P->nb);                                                               \
     break;
       GS2_PJC_CASES(GS2_PDOTS_CASE)
 #undef GS2_PDOTS_CASE
       default:
-        k_pdots_rt<64><<<P->gb, kVecThreads, 0, h->stream>>>(N, P->blk, P->items, P->cnt,
-                                                             P->st, h->V, jc, h->w, P->part,
-                                                             P->nb);
+        launch_pdl(k_pdots_rt<64>, P->gb, kVecThreads, 0, h->stream, N, P->blk, P->items, P->cnt, P->st,
+                   h->V, jc, h->w, P->part, P->nb);
         break;
     }
     GS2_LAUNCH_CHECK();
@@ -785,14 +801,14 @@ struct PackRun {
     switch (jc) {
 #define GS2_PUPD_CASE(J)                                                                \
   case J:                                                                               \
-    k_pupdate<J, NORM><<<P->gb, kVecThreads, 0, h->stream>>>(                           \
-        N, P->blk, P->items, P->cnt, P->st, h->V, P->hbuf, hs, h->w, P->part, P->nb);   \
+    launch_pdl(k_pupdate<J, NORM>, P->gb, kVecThreads, 0, h->stream, N, P->blk, P->items, P->cnt,     \
+               P->st, h->V, P->hbuf, hs, h->w, P->part, P->nb);                                        \
     break;
       GS2_PJC_CASES(GS2_PUPD_CASE)
 #undef GS2_PUPD_CASE
       default:
-        k_pupdate_rt<64, NORM><<<P->gb, kVecThreads, 0, h->stream>>>(
-            N, P->blk, P->items, P->cnt, P->st, h->V, jc, P->hbuf, hs, h->w, P->part, P->nb);
+        launch_pdl(k_pupdate_rt<64, NORM>, P->gb, kVecThreads, 0, h->stream, N, P->blk, P->items, P->cnt,
+                   P->st, h->V, jc, P->hbuf, hs, h->w, P->part, P->nb);
         break;
     }
     GS2_LAUNCH_CHECK();
@@ -800,9 +816,8 @@ struct PackRun {
 
   void launch_reduce(int j, int jc, int mode) {
     KernelTimer tm(h, "reduce_cols", 8.0 * jc * P->nb);
-    k_preduce<<<P->gs, 256, 0, h->stream>>>(P->part, P->nb, P->seg_blk, P->sys, P->cnt + 1,
-                                            P->st, P->H, P->hstride(), ldh(), j, P->hbuf,
-                                            (int)P->vstride(), mode, jc);
+    launch_pdl(k_preduce, P->gs, 256, 0, h->stream, P->part, P->nb, P->seg_blk, P->sys, P->cnt + 1, P->st,
+               P->H, P->hstride(), ldh(), j, P->hbuf, (int)P->vstride(), mode, jc);
     GS2_LAUNCH_CHECK();
   }
 
@@ -828,19 +843,16 @@ struct PackRun {
     launch_update<true>(jc);
     {
       KernelTimer tm(h, "givens", 8.0 * P->nb + 8.0 * 4 * (j + 2) * P->count);
-      k_pgivens<<<P->gs, 128, 0, h->stream>>>(P->part, P->seg_blk, P->sys, P->cnt + 1, P->st,
-                                              P->H, P->hstride(), ldh(), j, P->cs, P->sn,
-                                              P->gvec, (int)P->vstride(), P->nactive,
-                                              P->off_dev, P->live_run, h->st,
-                                              h->stop_mapped_dev);
+      launch_pdl(k_pgivens, P->gs, 128, 0, h->stream, P->part, P->seg_blk, P->sys, P->cnt + 1, P->st, P->H,
+                 P->hstride(), ldh(), j, P->cs, P->sn, P->gvec, (int)P->vstride(), P->nactive, P->off_dev,
+                 P->live_run, h->st, h->stop_mapped_dev);
       GS2_LAUNCH_CHECK();
     }
     if (j + 1 < m) {
       KernelTimer tm(h, "scale_next",
                      16.0 * N + (r64 ? 16.0 * N : 0.0) + (r32 ? 12.0 * N : 0.0));
-      k_pscale_next<<<P->gb, kVecThreads, 0, h->stream>>>(P->blk, P->items, P->cnt, P->st,
-                                                          h->w, h->V + (size_t)(j + 1) * N,
-                                                          h->dinv, r64, r32);
+      launch_pdl(k_pscale_next, P->gb, kVecThreads, 0, h->stream, P->blk, P->items, P->cnt, P->st, h->w,
+                 h->V + (size_t)(j + 1) * N, h->dinv, r64, r32);
       GS2_LAUNCH_CHECK();
     }
   }
@@ -898,14 +910,13 @@ struct PackRun {
     *h->stop_mapped = 0;
     GS2_CUDA(cudaMemcpyAsync(P->active, P->active_host, sizeof(int) * P->count,
                              cudaMemcpyHostToDevice, h->stream));
-    k_pcycle_reset<<<1, 1024, 0, h->stream>>>(P->st, P->active, P->count, P->nactive, h->st);
+    launch_pdl(k_pcycle_reset, 1, 1024, 0, h->stream, P->st, P->active, P->count, P->nactive, h->st);
     GS2_LAUNCH_CHECK();
-    k_plive_init<<<(P->nchunks + 255) / 256, 256, 0, h->stream>>>(
-        P->nchunks, (int)h->n, P->off_dev, P->count, P->active, P->live_cycle, P->live_run);
+    launch_pdl(k_plive_init, (P->nchunks + 255) / 256, 256, 0, h->stream, P->nchunks, (int)h->n,
+               P->off_dev, P->count, P->active, P->live_cycle, P->live_run);
     GS2_LAUNCH_CHECK();
-    k_pcycle_start<<<P->gb, kVecThreads, 0, h->stream>>>(P->blk, P->items, P->cnt, P->st, h->r,
-                                                         h->V, h->dinv, r64, r32, P->gvec,
-                                                         (int)P->vstride(), m);
+    launch_pdl(k_pcycle_start, P->gb, kVecThreads, 0, h->stream, P->blk, P->items, P->cnt, P->st, h->r,
+               h->V, h->dinv, r64, r32, P->gvec, (int)P->vstride(), m);
     GS2_LAUNCH_CHECK();
     cycle_ran = true;
     if (use_graph()) {
@@ -926,17 +937,16 @@ struct PackRun {
       profile_capture_step(h, -1);
     }
     // x += M^{-1} V y per system (u = 0 for systems without a step)
-    k_pbacksolve<<<P->gs, 64, 0, h->stream>>>(P->H, P->hstride(), ldh(), P->gvec, P->y,
-                                              (int)P->vstride(), P->sys, P->cnt + 1, P->st);
+    launch_pdl(k_pbacksolve, P->gs, 64, 0, h->stream, P->H, P->hstride(), ldh(), P->gvec, P->y,
+               (int)P->vstride(), P->sys, P->cnt + 1, P->st);
     GS2_LAUNCH_CHECK();
     {
       KernelTimer tm(h, "combine", 8.0 * h->n * (m + 1));
       const int N = (int)h->n;
       const int vs = (int)P->vstride();
 #define GS2_PCOMBINE(M)                                                                  \
-  k_pcombine<M><<<P->gb, kVecThreads, 0, h->stream>>>(N, P->blk, P->items, P->cnt, P->st, \
-                                                      h->V, P->y, vs, h->w, h->dinv, r64,  \
-                                                      r32)
+  launch_pdl(k_pcombine<M>, P->gb, kVecThreads, 0, h->stream, N, P->blk, P->items, P->cnt, P->st, h->V, \
+             P->y, vs, h->w, h->dinv, r64, r32)
       if (m <= 8) GS2_PCOMBINE(8);
       else if (m <= 16) GS2_PCOMBINE(16);
       else if (m <= 32) GS2_PCOMBINE(32);
@@ -948,7 +958,7 @@ struct PackRun {
       // systems that took no part in the cycle keep their x and skip the rows
       LiveRows lr(h, P->live_cycle);
       precond_apply(h, pc, h->w, h->z, wants, nullptr);
-      k_paxpy<<<P->gb, kVecThreads, 0, h->stream>>>(P->blk, P->items, P->cnt, x, h->z);
+      launch_pdl(k_paxpy, P->gb, kVecThreads, 0, h->stream, P->blk, P->items, P->cnt, x, h->z);
       GS2_LAUNCH_CHECK();
       launch_true_residual();
     }

@@ -35,9 +35,9 @@ constexpr int kPerThreads = 128;
 constexpr int kPerMaxBlocks = 128;
 constexpr long long kBarrierCycles = 4LL << 30;  // ~2 s at 2.07 GHz
 constexpr int64_t kPersistMaxRows = 1 << 16;
-// chosen automatically up to this size: measured on the 2D Laplacian with
-// GS2(1,1), GMRES(30): 4,096 rows 10.1 ms one launch vs 15.3 ms replayed
-// graphs, 16,384 rows 25.7 vs 27.9 ms, 62,500 rows 82 vs 76 ms
+// chosen automatically up to this size at most: CG with SGS2(1,1) per
+// iteration 26.1 us in one launch and 33.1 as graphs at 8,000 rows, 26.1 and
+// 30.7 at 15,625 (GMRES: a lower line, kGmresOneLaunchRows)
 constexpr int64_t kPersistAutoRows = 1 << 14;
 
 struct PersistArgs {
