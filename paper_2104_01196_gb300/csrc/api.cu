@@ -268,7 +268,8 @@ constexpr int kSellC = 32;                       // rows per chunk (one warp)
 constexpr double kSellMaxPadding = 1.2;          // slots / entries
 constexpr double kSellStreamBytes = 128.0 * (1 << 20);  // CSR bytes beyond L2
 
-// Chunk layout: chunk c takes width_c x 32 slots, width_c its longest row
+// (With `origin`, offsets are j - origin[i]: a colour's rows, origin[i] their row
+// in A.)  Chunk layout: chunk c takes width_c x 32 slots, width_c its longest row
 // (explicit columns) or, for an offset chunk, the number of distinct column
 // offsets j - i over its rows.  A chunk is an offset chunk when that union is
 // at most its longest row + kOffsetSlack and at most 32 (stencil rows: the
@@ -284,7 +285,8 @@ struct SellLayout {
   int offset_chunks = 0, wmax = 0;
 };
 
-static bool sell_layout(const std::vector<int>& rp, const int* ci, int n, SellLayout& out) {
+static bool sell_layout(const std::vector<int>& rp, const int* ci, int n, const int* origin,
+                        SellLayout& out) {
   const int nc = (n + kSellC - 1) / kSellC;
   out.cptr.assign(nc + 1, 0);
   out.coff.assign(nc, -1);
@@ -300,7 +302,7 @@ static bool sell_layout(const std::vector<int>& rp, const int* ci, int n, SellLa
     for (int i = c * kSellC; i < std::min(n, (c + 1) * kSellC); ++i) {
       L = std::max(L, rp[i + 1] - rp[i]);
       for (int k = rp[i]; regular && k < rp[i + 1]; ++k) {
-        const int o = ci[k] - i;
+        const int o = ci[k] - (origin ? origin[i] : i);
         if (std::find(u.begin(), u.end(), o) == u.end()) {
           u.push_back(o);
           if ((int)u.size() > kOffsetMax) regular = false;
@@ -404,12 +406,13 @@ static bool lane_layout(const std::vector<int>& rp, int n, int K, LaneLayout& ou
 // The sliced-ELL arrays are filled on the device from the CSR arrays already
 // there (launch_to_sell, launch_to_lanes); only the chunk layout is computed
 // here.
-static void upload_sell(gs2_handle* h, DevCsr& M, const std::vector<int>& rp, const int* ci) {
+static void upload_sell(gs2_handle* h, DevCsr& M, const std::vector<int>& rp, const int* ci,
+                        const int* origin) {
   const int n = M.n;
   if (n == 0 || M.nnz == 0) return;
   SellLayout lay;
   const bool sliced = (M.mean_row <= kShortRowMean || 12.0 * M.nnz >= kSellStreamBytes) &&
-                      sell_layout(rp, ci, n, lay);
+                      sell_layout(rp, ci, n, origin, lay);
   LaneLayout lanes;
   if (!sliced) {
     // rows of uneven length, and long rows in a matrix that fits L2
@@ -462,7 +465,8 @@ static void upload_sell(gs2_handle* h, DevCsr& M, const std::vector<int>& rp, co
 }
 
 static void upload_csr(gs2_handle* h, DevCsr& M, int n, const std::vector<int>& rp,
-                       const int* ci, const double* va, int nnz) {
+                       const int* ci, const double* va, int nnz,
+                       const int* origin = nullptr) {
   M.n = n;
   M.nnz = nnz;
   M.mean_row = n ? (double)M.nnz / n : 0.0;
@@ -480,7 +484,7 @@ static void upload_csr(gs2_handle* h, DevCsr& M, int n, const std::vector<int>& 
   h->h2d(M.ci, ci, sizeof(int) * M.nnz);
   h->h2d(M.va, va, sizeof(double) * M.nnz);
   retile(h, M, rp, M.tpr, 1);
-  upload_sell(h, M, rp, ci);
+  upload_sell(h, M, rp, ci, origin);
 }
 
 // (Re)build the row tiles of M for K lanes per row and RPT rows per lane
@@ -783,23 +787,27 @@ void ensure_colors(gs2_handle* h) {
   for (int i = 0; i < n; ++i) rows[color[i]].push_back(i);
   for (int c = 0; c < nc; ++c) {
     const std::vector<int>& rr = rows[c];
-    std::vector<int> rp(rr.size() + 1, 0), ci;
-    std::vector<double> va;
-    for (size_t q = 0; q < rr.size(); ++q) {
-      const int i = rr[q];
-      for (int k = L.rp[i]; k < L.rp[i + 1]; ++k) {
-        ci.push_back(L.ci[k]);
-        va.push_back(L.va[k]);
+    std::vector<int> rp(rr.size() + 1, 0);
+    for (size_t q = 0; q < rr.size(); ++q)
+      rp[q + 1] = rp[q] + (L.rp[rr[q] + 1] - L.rp[rr[q]]) + (U.rp[rr[q] + 1] - U.rp[rr[q]]);
+    std::vector<int> ci(rp.back());
+    std::vector<double> va(rp.back());
+    parallel_ranges((int64_t)rr.size(), [&](int64_t q0, int64_t q1, int) {
+      for (int64_t q = q0; q < q1; ++q) {
+        const int i = rr[q];
+        int o = rp[q];
+        for (const HostTri* T : {&L, &U})
+          for (int k = T->rp[i]; k < T->rp[i + 1]; ++k, ++o) {
+            ci[o] = T->ci[k];
+            va[o] = T->va[k];
+          }
       }
-      for (int k = U.rp[i]; k < U.rp[i + 1]; ++k) {
-        ci.push_back(U.ci[k]);
-        va.push_back(U.va[k]);
-      }
-      rp[q + 1] = (int)ci.size();
-    }
-    upload_csr(h, h->colors[c], (int)rr.size(), rp, ci.data(), va.data(), (int)ci.size());
+    });
     h->color_rows[c] = (int*)h->dalloc(sizeof(int) * std::max<size_t>(rr.size(), 1));
     h->h2d(h->color_rows[c], rr.data(), sizeof(int) * rr.size());
+    h->colors[c].sell_origin = h->color_rows[c];
+    upload_csr(h, h->colors[c], (int)rr.size(), rp, ci.data(), va.data(), (int)ci.size(),
+               rr.data());
   }
   h->colors_ready = true;
 }

@@ -101,6 +101,7 @@ struct DevCsr {
   int* sell_coff = nullptr;    // sell_chunks: first offset, or -1
   int* sell_off = nullptr;     // the offset lists (chunks with equal lists share one)
   int sell_offset_chunks = 0;  // chunks without explicit columns
+  const int* sell_origin = nullptr;  // a colour's rows: offsets count from this row, not i
   int sell_wmax = 0;           // slots of the widest chunk
   int sell_ncols = 0;          // 1 + the largest column (the gathered vector's length)
   double* sell_va = nullptr;

@@ -31,13 +31,14 @@ namespace gs2 {
 // has 8 instead of 9, an undamped inner sweep of a 3-entry triangle 3 or 4
 // instead of 5; a few more roundings of the operand's size: sweeps are 2e-16 from
 // the 64-bit result where they were 1.6e-16).  kUnroll: the widest stencil row that takes the unrolled form
-// (k_stencil).
+// (k_stencil).  origin(i, pre): the row that row i's offsets count from.
 // ---------------------------------------------------------------------------
 
 // r = b - A x;  rhat = D^{-1} r   (Eq. 2 residual and Eq. 3 initial guess)
 struct EpiResid {
   static constexpr bool kSub = true;
   static constexpr int kUnroll = 6;
+  static constexpr bool kGuard = false;
   const double* __restrict__ x;
   const double* __restrict__ b;
   const double* __restrict__ dinv;
@@ -47,6 +48,7 @@ struct EpiResid {
   struct Pre {
     double b, d;
   };
+  __device__ int origin(int i, const Pre&) const { return i; }
   __device__ Pre pre(int i) const { return Pre{b[i], dinv[i]}; }
   __device__ double gather(int c) const { return __ldg(x + c); }
   __device__ double begin(const Pre& p) const { return p.b; }
@@ -61,9 +63,11 @@ struct EpiResid {
 struct EpiSpmv {
   static constexpr bool kSub = false;
   static constexpr int kUnroll = 8;
+  static constexpr bool kGuard = false;
   const double* __restrict__ x;
   double* __restrict__ y;
   struct Pre {};
+  __device__ int origin(int i, const Pre&) const { return i; }
   __device__ Pre pre(int) const { return Pre{}; }
   __device__ double gather(int c) const { return __ldg(x + c); }
   __device__ double begin(const Pre&) const { return 0.0; }
@@ -74,11 +78,13 @@ struct EpiSpmv {
 struct EpiSpmvAdd {
   static constexpr bool kSub = false;
   static constexpr int kUnroll = 8;
+  static constexpr bool kGuard = false;
   const double* __restrict__ x;
   double* __restrict__ y;
   struct Pre {
     double y;
   };
+  __device__ int origin(int i, const Pre&) const { return i; }
   __device__ Pre pre(int i) const { return Pre{y[i]}; }
   __device__ double gather(int c) const { return __ldg(x + c); }
   __device__ double begin(const Pre& p) const { return p.y; }
@@ -89,6 +95,7 @@ struct EpiSpmvAdd {
 struct EpiJr {
   static constexpr bool kSub = true;
   static constexpr int kUnroll = 8;
+  static constexpr bool kGuard = false;
   const double* __restrict__ x;
   const double* __restrict__ b;
   const double* __restrict__ dinv;
@@ -97,6 +104,7 @@ struct EpiJr {
   struct Pre {
     double x, b, d;
   };
+  __device__ int origin(int i, const Pre&) const { return i; }
   __device__ Pre pre(int i) const { return Pre{x[i], b[i], dinv[i]}; }
   __device__ double gather(int c) const { return __ldg(x + c); }
   __device__ double begin(const Pre& p) const { return p.b; }
@@ -119,6 +127,7 @@ template <typename GT, typename AT, InnerForm FORM, bool SCALED>
 struct EpiInner {
   static constexpr bool kSub = FORM == INNER_UNIT;
   static constexpr int kUnroll = 8;
+  static constexpr bool kGuard = false;
   const GT* __restrict__ g_in;
   const GT* __restrict__ rhat;
   GT* __restrict__ g_out;
@@ -133,6 +142,7 @@ struct EpiInner {
     double xi;
     float x32i;
   };
+  __device__ int origin(int i, const Pre&) const { return i; }
   __device__ Pre pre(int i) const {
     Pre p;
     p.rh = (AT)rhat[i];
@@ -181,6 +191,7 @@ template <bool SCALED>
 struct EpiResidSweep {
   static constexpr bool kSub = false;
   static constexpr int kUnroll = 4;
+  static constexpr bool kGuard = false;
   const float* __restrict__ bhat;
   const float* __restrict__ x32;
   const signed char* __restrict__ rowscale;
@@ -188,6 +199,7 @@ struct EpiResidSweep {
   struct Pre {
     float bx, sc;
   };
+  __device__ int origin(int i, const Pre&) const { return i; }
   __device__ Pre pre(int i) const {
     Pre p;
     p.bx = bhat[i] - x32[i];
@@ -207,6 +219,7 @@ struct EpiResidSweep {
 struct EpiCompact {
   static constexpr bool kSub = true;
   static constexpr int kUnroll = 8;
+  static constexpr bool kGuard = false;
   const double* __restrict__ x;
   const double* __restrict__ b;
   const double* __restrict__ dinv;
@@ -215,6 +228,7 @@ struct EpiCompact {
   struct Pre {
     double b, d;
   };
+  __device__ int origin(int i, const Pre&) const { return i; }
   __device__ Pre pre(int i) const { return Pre{b[i], dinv[i]}; }
   __device__ double gather(int c) const { return __ldg(x + c); }
   __device__ double begin(const Pre& p) const { return p.d * p.b; }
@@ -233,6 +247,7 @@ template <bool DAMPED>
 struct EpiColor {
   static constexpr bool kSub = true;
   static constexpr int kUnroll = 8;
+  static constexpr bool kGuard = true;
   const int* __restrict__ rows;
   const double* __restrict__ bhat;
   double* x;
@@ -241,6 +256,7 @@ struct EpiColor {
     int r;
     double bh, xr;
   };
+  __device__ int origin(int, const Pre& p) const { return p.r; }
   __device__ Pre pre(int i) const {
     Pre p;
     p.r = rows[i];
@@ -331,23 +347,25 @@ __device__ __forceinline__ void add_to(__half* p, __half v) {
 // Explicit chunk: slot k of row i goes to cptr[c] + 32 k + i % 32; value
 // slots past the row's end keep their zero, column slots repeat the row's
 // last column (column 0 for an empty row, whose slots stay zero).  Offset
-// chunk: the entry at column j goes to the slot of offset j - i in the
+// chunk: the entry at column j goes to the slot of offset j - i (with `origin`,
+// j - origin[i]) in the
 // chunk's offset list (added, so duplicate entries of an unvalidated matrix
 // sum as in an SpMV); the other slots keep their zero, and no column is
 // stored.
 template <typename T>
 __global__ void k_to_sell(int n, const int* __restrict__ rp, const int* __restrict__ ci,
                           const T* __restrict__ va, const int* __restrict__ cptr,
-                          const int* __restrict__ coff, const int* __restrict__ offs, int* sci,
-                          T* sva) {
+                          const int* __restrict__ coff, const int* __restrict__ offs,
+                          const int* __restrict__ origin, int* sci, T* sva) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     const int c = i >> 5, lane = i & 31;
     const int L = (cptr[c + 1] - cptr[c]) >> 5;
     const int a = rp[i], len = rp[i + 1] - a;
     const int ob = coff[c];
     if (ob >= 0) {
+      const int at = origin ? origin[i] : i;
       for (int k = 0; k < len; ++k) {
-        const int o = ci[a + k] - i;
+        const int o = ci[a + k] - at;
         int p = 0;
         while (p < L && offs[ob + p] != o) ++p;  // present by construction
         if (p < L) add_to(sva + cptr[c] + (p << 5) + lane, va[a + k]);
@@ -369,8 +387,8 @@ __global__ void k_to_sell(int n, const int* __restrict__ rp, const int* __restri
 template <typename T>
 static void to_sell(gs2_handle* h, const DevCsr& M, const T* va, T* sva, bool with_ci) {
   k_to_sell<T><<<vec_blocks(h, M.n), kVecThreads, 0, h->stream>>>(
-      M.n, M.rp, M.ci, va, M.sell_ptr, M.sell_coff, M.sell_off, with_ci ? M.sell_ci : nullptr,
-      sva);
+      M.n, M.rp, M.ci, va, M.sell_ptr, M.sell_coff, M.sell_off, M.sell_origin,
+      with_ci ? M.sell_ci : nullptr, sva);
   GS2_LAUNCH_CHECK();
 }
 void launch_to_sell(gs2_handle* h, const DevCsr& M, const double* va, double* sva, bool with_ci) {

@@ -68,6 +68,16 @@ __device__ __forceinline__ AT row_fma(AT a, AT x, AT s) {
   return fma(Epi::kSub ? -a : a, x, s);
 }
 
+// The gathered x of an offset chunk's slot, or with Epi::kGuard 0 in a slot of
+// value 0: an infinity or NaN at a column that the row does not have cannot
+// reach it.  (+0.0 by its bits: a comparison would issue on the FP64 pipe.)
+__device__ __forceinline__ bool zero_bits(double a) { return __double_as_longlong(a) == 0; }
+__device__ __forceinline__ bool zero_bits(float a) { return __float_as_int(a) == 0; }
+template <class Epi, typename AT>
+__device__ __forceinline__ AT guarded(AT a, AT x) {
+  return Epi::kGuard && zero_bits(a) ? AT(0) : x;
+}
+
 // ---------------------------------------------------------------------------
 // TMA bulk copies and mbarriers (inline PTX, sm_90+ / sm_103a)
 // ---------------------------------------------------------------------------
@@ -362,8 +372,8 @@ __device__ __forceinline__ bool sell_pair(int n, int c, const int* __restrict__ 
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     if (k < L) {
-      const int ca = min(max(r0 + __ldg(o0 + k), 0), cmax);
-      const int cb = min(max(r1 + __ldg(o1 + k), 0), cmax);
+      const int ca = min(max(epi.origin(r0, p0) + __ldg(o0 + k), 0), cmax);
+      const int cb = min(max(epi.origin(r1, p1) + __ldg(o1 + k), 0), cmax);
       const AT a = stream_val<VT>(v0 + 32 * k), b = stream_val<VT>(v1 + 32 * k);
       const AT xa = (AT)epi.gather(ca), xb = (AT)epi.gather(cb);
       s0 = row_fma<Epi>(a, xa, s0);
@@ -407,34 +417,35 @@ k_sell(int n, int nchunks, const int* __restrict__ cptr, const int* __restrict__
       // columns row + o, clamped into [0, ncols) for the zero slots of rows
       // at a boundary (and the rows past n of the last chunk)
       const int* oo = offs + ob;
+      const int at = epi.origin(row, pv);
       for (; k + 4 <= L; k += 4, vv += 128) {
-        const int c0 = min(max(row + __ldg(oo + k), 0), cmax);
-        const int c1 = min(max(row + __ldg(oo + k + 1), 0), cmax);
-        const int c2 = min(max(row + __ldg(oo + k + 2), 0), cmax);
-        const int c3 = min(max(row + __ldg(oo + k + 3), 0), cmax);
+        const int c0 = min(max(at + __ldg(oo + k), 0), cmax);
+        const int c1 = min(max(at + __ldg(oo + k + 1), 0), cmax);
+        const int c2 = min(max(at + __ldg(oo + k + 2), 0), cmax);
+        const int c3 = min(max(at + __ldg(oo + k + 3), 0), cmax);
         const AT a0 = stream_val<VT>(vv), a1 = stream_val<VT>(vv + 32);
         const AT a2 = stream_val<VT>(vv + 64), a3 = stream_val<VT>(vv + 96);
         const AT x0 = (AT)epi.gather(c0), x1 = (AT)epi.gather(c1);
         const AT x2 = (AT)epi.gather(c2), x3 = (AT)epi.gather(c3);
-        s = row_fma<Epi>(a0, x0, s);
-        s = row_fma<Epi>(a1, x1, s);
-        s = row_fma<Epi>(a2, x2, s);
-        s = row_fma<Epi>(a3, x3, s);
+        s = row_fma<Epi>(a0, guarded<Epi>(a0, x0), s);
+        s = row_fma<Epi>(a1, guarded<Epi>(a1, x1), s);
+        s = row_fma<Epi>(a2, guarded<Epi>(a2, x2), s);
+        s = row_fma<Epi>(a3, guarded<Epi>(a3, x3), s);
       }
       const int rem = L - k;
       if (rem > 0) {
-        const int c0 = min(max(row + __ldg(oo + k), 0), cmax);
-        const int c1 = rem > 1 ? min(max(row + __ldg(oo + k + 1), 0), cmax) : c0;
-        const int c2 = rem > 2 ? min(max(row + __ldg(oo + k + 2), 0), cmax) : c0;
+        const int c0 = min(max(at + __ldg(oo + k), 0), cmax);
+        const int c1 = rem > 1 ? min(max(at + __ldg(oo + k + 1), 0), cmax) : c0;
+        const int c2 = rem > 2 ? min(max(at + __ldg(oo + k + 2), 0), cmax) : c0;
         const AT a0 = stream_val<VT>(vv);
         const AT a1 = rem > 1 ? stream_val<VT>(vv + 32) : AT(0);
         const AT a2 = rem > 2 ? stream_val<VT>(vv + 64) : AT(0);
         const AT x0 = (AT)epi.gather(c0);
         const AT x1 = rem > 1 ? (AT)epi.gather(c1) : AT(0);
         const AT x2 = rem > 2 ? (AT)epi.gather(c2) : AT(0);
-        s = row_fma<Epi>(a0, x0, s);
-        if (rem > 1) s = row_fma<Epi>(a1, x1, s);
-        if (rem > 2) s = row_fma<Epi>(a2, x2, s);
+        s = row_fma<Epi>(a0, guarded<Epi>(a0, x0), s);
+        if (rem > 1) s = row_fma<Epi>(a1, guarded<Epi>(a1, x1), s);
+        if (rem > 2) s = row_fma<Epi>(a2, guarded<Epi>(a2, x2), s);
       }
       if (row < n) epi.finish(row, s, pv);
       continue;
@@ -506,48 +517,49 @@ k_sell(int n, int nchunks, const int* __restrict__ cptr, const int* __restrict__
 // The row sum of an offset row of exactly W slots: every slot's value and
 // gather is issued before the first product, so a row costs one round trip
 // to memory (in groups of four, a 5- or 7-slot row costs two).  Columns are
+// offsets from `at` (the row itself; the row of A for a colour's rows),
 // clamped into [0, cmax] for the zero slots of rows at a boundary (and the
 // rows past n of the last chunk).
 template <int W, typename VT, class Epi, typename AT>
-__device__ __forceinline__ AT stencil_row(AT s, int row, const int* __restrict__ oo,
+__device__ __forceinline__ AT stencil_row(AT s, int at, const int* __restrict__ oo,
                                           const VT* __restrict__ vv, const Epi& epi, int cmax) {
   AT a[W], x[W];
   int c[W];
 #pragma unroll
   for (int k = 0; k < W; ++k) a[k] = stream_val<VT>(vv + 32 * k);
 #pragma unroll
-  for (int k = 0; k < W; ++k) c[k] = min(max(row + __ldg(oo + k), 0), cmax);
+  for (int k = 0; k < W; ++k) c[k] = min(max(at + __ldg(oo + k), 0), cmax);
 #pragma unroll
   for (int k = 0; k < W; ++k) x[k] = (AT)epi.gather(c[k]);
 #pragma unroll
-  for (int k = 0; k < W; ++k) s = row_fma<Epi>(a[k], x[k], s);
+  for (int k = 0; k < W; ++k) s = row_fma<Epi>(a[k], guarded<Epi>(a[k], x[k]), s);
   return s;
 }
 
 // ... of L <= WM slots: L is the same for the whole warp, so the switch is a
 // uniform branch
 template <int WM, typename VT, class Epi, typename AT>
-__device__ __forceinline__ AT stencil_rows(AT s, int L, int row, const int* __restrict__ oo,
+__device__ __forceinline__ AT stencil_rows(AT s, int L, int at, const int* __restrict__ oo,
                                            const VT* __restrict__ vv, const Epi& epi, int cmax) {
   if (WM >= 7) {
     switch (L) {
-      case 8: return stencil_row<8, VT>(s, row, oo, vv, epi, cmax);
-      case 7: return stencil_row<7, VT>(s, row, oo, vv, epi, cmax);
+      case 8: return stencil_row<8, VT>(s, at, oo, vv, epi, cmax);
+      case 7: return stencil_row<7, VT>(s, at, oo, vv, epi, cmax);
       default: break;
     }
   }
   if (WM >= 5) {
     switch (L) {
-      case 6: return stencil_row<6, VT>(s, row, oo, vv, epi, cmax);
-      case 5: return stencil_row<5, VT>(s, row, oo, vv, epi, cmax);
+      case 6: return stencil_row<6, VT>(s, at, oo, vv, epi, cmax);
+      case 5: return stencil_row<5, VT>(s, at, oo, vv, epi, cmax);
       default: break;
     }
   }
   switch (L) {
-    case 4: return stencil_row<4, VT>(s, row, oo, vv, epi, cmax);
-    case 3: return stencil_row<3, VT>(s, row, oo, vv, epi, cmax);
-    case 2: return stencil_row<2, VT>(s, row, oo, vv, epi, cmax);
-    case 1: return stencil_row<1, VT>(s, row, oo, vv, epi, cmax);
+    case 4: return stencil_row<4, VT>(s, at, oo, vv, epi, cmax);
+    case 3: return stencil_row<3, VT>(s, at, oo, vv, epi, cmax);
+    case 2: return stencil_row<2, VT>(s, at, oo, vv, epi, cmax);
+    case 1: return stencil_row<1, VT>(s, at, oo, vv, epi, cmax);
     default: return s;
   }
 }
@@ -595,7 +607,7 @@ k_stencil(int n, int nchunks, const int* __restrict__ cptr, const int* __restric
       const int L = (end - base) >> 5;
       const VT* vv = va + base + lane;
       auto s = epi.begin(pv);
-      s = stencil_rows<WM, VT>(s, L, row, offs + ob, vv, epi, cmax);
+      s = stencil_rows<WM, VT>(s, L, epi.origin(row, pv), offs + ob, vv, epi, cmax);
       if (row < n) epi.finish(row, s, pv);
     }
     if (cn >= nchunks) return;

@@ -166,3 +166,33 @@ def test_lane_slices_infinity(g):  # noqa: F811
     one = np.zeros(n, int)
     np.add.at(one, rows[np.isin(A[1], [0, 777])], 1)
     assert np.isinf(got[one == 1]).all()
+
+
+# colours of stencils of every width (offsets count from a colour row's row in A), odd sizes and a
+# chunk at each end, and an infinity that may reach only the rows that hold its column
+@pytest.mark.parametrize("width", [3, 5, 7, 9])
+def test_colour_rows_infinity(g, width):  # noqa: F811
+    n = 1003
+    A = band_matrix(n, width, width)
+    h = g.gs2_setup(A)
+    b, x0 = rhs_and_x0(A, 51)
+    x = dev(x0)
+    g.mtgs_apply(h, dev(b), x, 2, 0.9, g.FORWARD)
+    assert rel(host(x), oracle.mtgs(A, b, x0, 2, 0.9, oracle.FORWARD)) <= TOL
+    # b = inf at the last row of the last colour: x there, and nowhere else, in one forward sweep
+    color = oracle.coloring(A)
+    color = np.asarray(color[0] if isinstance(color, tuple) else color)
+    last = int(np.flatnonzero(color == color.max())[-1])
+    b2 = b.copy()
+    b2[last] = np.inf
+    x = dev(x0)
+    g.mtgs_apply(h, dev(b2), x, 1, 1.0, g.FORWARD)
+    got = host(x)
+    assert np.isinf(got[last]) and np.isfinite(np.delete(got, last)).all()
+    # x = inf at row 0: every row of a colour that holds column 0 and is updated before row 0's
+    # own colour takes it; row 0 is in the first colour, so it is overwritten first
+    x1 = x0.copy()
+    x1[0] = np.inf
+    x = dev(x1)
+    g.mtgs_apply(h, dev(b), x, 1, 1.0, g.FORWARD)
+    assert np.isfinite(host(x)).all()
