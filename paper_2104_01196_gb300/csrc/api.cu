@@ -1261,13 +1261,16 @@ gs2_handle* gs2::setup_handle(int64_t n, int64_t nnz, const int64_t* rowptr,
   U.ci.resize(U.rp[n]);
   U.va.resize(U.rp[n]);
   std::vector<double> dinv(n);
+  std::atomic<bool> parted{true};
   parallel_ranges(n, [&](int64_t i0, int64_t i1, int) {
     for (int64_t i = i0; i < i1; ++i) {
       const double di = 1.0 / diag[i];
       dinv[i] = di;
       int ql = L.rp[i], qu = U.rp[i];
+      if (CI[RP[i] + (L.rp[i + 1] - ql)] != i) parted = false;
       for (int64_t k = RP[i]; k < RP[i + 1]; ++k) {
         const int j = CI[k];
+        if (j < i && qu > U.rp[i]) parted = false;
         if (j < i) {
           L.ci[ql] = j;
           L.va[ql++] = VA[k] * di;
@@ -1288,6 +1291,7 @@ gs2_handle* gs2::setup_handle(int64_t n, int64_t nnz, const int64_t* rowptr,
   h->stream = stream;
   h->async_alloc = async_alloc;
   h->for_pack = for_pack;
+  h->parted = parted;
   h->n = n;
   h->nnz = nnz;
   upload_csr(h, h->A, (int)n, rp32, CI, VA, (int)nnz);

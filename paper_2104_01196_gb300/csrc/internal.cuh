@@ -256,6 +256,7 @@ struct gs2_handle {
   double* persist_part = nullptr;   // its partial sums
   bool stall_barrier = false;       // test hook: next one-launch solve's barrier never opens
   int cl_wa = -1, cl_wl = -1, cl_wu = -1;  // longest rows of A, L, U (longest_rows)
+  bool parted = false;  // every row's entries left of the diagonal come first, it next
   void* cl_sys = nullptr;  // a pack in clusters: its per-system table (device)
   int cl_sys_cap = 0;
   // one-launch solve of a pack: per-system argument table, block -> system
@@ -441,6 +442,10 @@ bool precond_wants_rhat(const gs2_params* p);
 // the relaxation of p's kind (GS2, JR, exact GS, multicolour GS), global or
 // in the hybrid form, from x
 void gs2_relax(gs2_handle* h, const double* b, double* x, const gs2_params* p);
+// the GS2 sweeps of p on a small stencil system as one launch (small.cu)
+bool small_sweeps_eligible(gs2_handle* h, const gs2_params* p);
+int small_rows_per_cta(int64_t n);
+void launch_small_sweeps(gs2_handle* h, const double* b, double* x, const gs2_params* p);
 void gs_relax(gs2_handle* h, const double* b, double* x, int sweeps,
               double omega, int direction);
 void jr_relax(gs2_handle* h, const double* b, double* x, int sweeps,

@@ -229,6 +229,10 @@ void gs2_relax(gs2_handle* h, const double* b, double* x, const gs2_params* p) {
     sweep32_relax(h, p, b, x, false, global_sweeps(p), nullptr);
     return;
   }
+  if (small_sweeps_eligible(h, p)) {
+    launch_small_sweeps(h, b, x, p);
+    return;
+  }
   for (int s = 0; s < global_sweeps(p); ++s) {
     if (p->direction == GS2_FORWARD || p->direction == GS2_SYMMETRIC)
       gs2_half(h, p, h->L, h->U, b, x, false, nullptr);

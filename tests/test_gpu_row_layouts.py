@@ -196,3 +196,57 @@ def test_colour_rows_infinity(g, width):  # noqa: F811
     x = dev(x1)
     g.mtgs_apply(h, dev(b), x, 1, 1.0, g.FORWARD)
     assert np.isfinite(host(x)).all()
+
+
+# small stencil systems in one launch: one row, one and several CTAs with a last one short, both
+# size lines and one row beyond, more neighbours than it takes (row kernels), unsorted rows (row
+# kernels), every direction, damping, no inner sweep, several sweeps
+SMALL = {
+    "n1": (np.array([0, 1]), np.array([0], np.int32), np.array([3.0])),
+    "band_64": band_matrix(64, 3, 61),
+    "band_65": band_matrix(65, 7, 62),
+    "grid_4096": P.poisson2d_matrix(64),
+    "grid_4225": P.poisson2d_matrix(65),
+    "grid3d_8000": P.poisson3d_matrix(20),
+    "grid_8281": P.poisson2d_matrix(91),
+    "band_9_wide": band_matrix(300, 9, 63),
+    "unsorted": P.random_csr(300, 64, mean_offdiag=2.0),
+}
+
+
+@pytest.mark.parametrize("name", list(SMALL))
+@pytest.mark.parametrize("direction", [0, 1, 2])
+def test_small_sweeps(g, name, direction):  # noqa: F811
+    A = SMALL[name]
+    b, x0 = rhs_and_x0(A, 71)
+    h = g.gs2_setup(A)
+    for outer, inner, omega, gamma in ((1, 1, 1.0, 1.0), (2, 2, 0.9, 1.0), (1, 0, 0.8, 1.0),
+                                       (1, 3, 1.0, 1.0), (2, 3, 0.9, 0.7)):
+        x = dev(x0)
+        g.gs2_apply_ex(h, dev(b), x, g.params("gs2", outer=outer, inner=inner, omega=omega,
+                                              gamma=gamma, direction=direction))
+        ref = oracle.gs2(A, b, x0, outer, inner, omega, gamma, direction)
+        assert rel(host(x), ref) <= TOL, (outer, inner, omega, gamma)
+
+
+# the same call through the row kernels (which a profiled handle takes): the same bits, also where
+# b and x hold infinities and NaN
+@pytest.mark.parametrize("name", ["grid_4096", "band_65", "grid3d_8000"])
+def test_small_sweeps_equal_row_kernels(g, name):  # noqa: F811
+    A = SMALL[name]
+    b, x0 = rhs_and_x0(A, 72)
+    h = g.gs2_setup(A)
+    for special in (False, True):
+        if special:
+            b[3], x0[40], x0[50] = np.inf, np.nan, -np.inf
+        out = []
+        for profiled in (False, True):
+            h.profile(profiled)
+            x = dev(x0)
+            g.gs2_apply_ex(h, dev(b), x, g.params("gs2", inner=3, direction="symmetric"))
+            out.append(host(x))
+        h.profile(False)
+        fine = np.isfinite(out[1])
+        if special:  # (the row kernels' zero slots may turn more rows into NaN)
+            assert np.isfinite(out[0][fine]).all() and (~np.isfinite(out[0])).any()
+        assert np.array_equal(out[0][fine], out[1][fine])
