@@ -256,14 +256,15 @@ void retile(gs2_handle* h, DevCsr& M, const std::vector<int>& rp, int K, int RPT
 // elasticity the residual went from 2.8 to 5.0 TB/s against the best
 // row-tile shape, 8 lanes per row).  Long rows of smaller matrices (coarse
 // multigrid levels) are latency-bound: K lanes per row shorten each row's
-// chain of dependent gathers.  Their FP64 values, and those of matrices of
-// uneven rows, get lane slices, which reduce a row in K segments as the row
+// chain of dependent gathers.  They, and matrices of uneven rows, get lane
+// slices, which reduce a row in K segments as the row
 // tiles do without staging it through shared memory (the stages limit a tile
 // kernel to 2 to 3 blocks per SM, and its barriers idle the short rows'
 // lanes): symmetric FP64 sweep on 300,007 uneven rows 115 -> 70 us, on Q1
-// elasticity with 28^3 nodes 105 -> 58.  FP32 and FP16 values, half the bytes
-// through the same stages, stay in the row tiles (inner sweep on the uneven
-// rows 7.1 us against 10.5 in lane slices, on 40^3 nodes 15.4 against 19.8).
+// elasticity with 28^3 nodes 105 -> 58.  FP32 and FP16 values follow where the
+// slices have the row tiles' lanes, whose rounding they keep (inner sweep on
+// 40^3 nodes 16.9 -> 13.8 us, on 28^3 8.5 -> 6.8; whole-sweep residual there
+// 13.0 -> 10.5), and stay in the row tiles elsewhere.
 constexpr int kSellC = 32;                       // rows per chunk (one warp)
 constexpr double kSellMaxPadding = 1.2;          // slots / entries
 constexpr double kSellStreamBytes = 128.0 * (1 << 20);  // CSR bytes beyond L2
@@ -335,6 +336,7 @@ static bool sell_layout(const std::vector<int>& rp, const int* ci, int n, const 
 constexpr int kLaneWindow = 1024;    // rows sorted together
 constexpr int kLaneWarpsPerSm = 16;  // warps that a matrix should give each SM
 constexpr int kLaneMaxSlots = 128;   // of one chunk: longer rows need a whole block
+constexpr int kSellWarpsPerSm = 32;  // resident warps of k_sell on long rows
 
 // Lanes per row: at most 24 entries a lane on average; with fewer than 16
 // warps per SM more lanes, down to 4 entries each (a warp's groups of four
@@ -411,20 +413,24 @@ static void upload_sell(gs2_handle* h, DevCsr& M, const std::vector<int>& rp, co
   const int n = M.n;
   if (n == 0 || M.nnz == 0) return;
   SellLayout lay;
-  const bool sliced = (M.mean_row <= kShortRowMean || 12.0 * M.nnz >= kSellStreamBytes) &&
-                      sell_layout(rp, ci, n, origin, lay);
+  int longest = 0;
+  for (int i = 0; i < n; ++i) longest = std::max(longest, rp[i + 1] - rp[i]);
+  const bool short_rows = M.mean_row <= kShortRowMean;
+  const bool streams = 12.0 * M.nnz >= kSellStreamBytes;
   LaneLayout lanes;
-  if (!sliced) {
-    // rows of uneven length, and long rows in a matrix that fits L2
-    int longest = 0;
-    for (int i = 0; i < n; ++i) longest = std::max(longest, rp[i + 1] - rp[i]);
-    const int K = lane_count(h, n, M.mean_row, longest);
-    M.sell_lanes = K;
-    if (longest > kLaneMaxSlots * K || !lane_layout(rp, n, K, lanes)) {
-      M.sell_lanes = 0;
-      return;  // row tiles
-    }
-  }
+  auto try_lanes = [&](int K) {
+    M.sell_lanes = longest <= kLaneMaxSlots * K && lane_layout(rp, n, K, lanes) ? K : 0;
+    return M.sell_lanes > 0;
+  };
+  // a long-row A of less than two waves of warps: one lane a row, but a warp
+  // per chunk instead of a persistent grid whose last wave is nearly empty
+  // (Q1 elasticity on 40^3 nodes, residual 39.5 -> 34.8 us; no gain on 50^3,
+  // 3% lost on 64^3)
+  const bool few = &M == &h->A && !short_rows && streams &&
+                   n < 2 * 32 * (int64_t)kSellWarpsPerSm * h->nsm && try_lanes(1);
+  const bool sliced = !few && (short_rows || streams) && sell_layout(rp, ci, n, origin, lay);
+  // rows of uneven length, and long rows in a matrix that fits L2
+  if (!few && !sliced && !try_lanes(lane_count(h, n, M.mean_row, longest))) return;  // row tiles
   const std::vector<int>& cptr = sliced ? lay.cptr : lanes.cptr;
   const size_t slots = std::max(cptr.back(), 1);
   std::vector<int> top(kHostThreads, 0);
@@ -451,7 +457,7 @@ static void upload_sell(gs2_handle* h, DevCsr& M, const std::vector<int>& rp, co
       M.sell_row = (int*)h->dalloc(sizeof(int) * n);
       h->h2d(M.sell_row, lanes.row.data(), sizeof(int) * n);
     }
-    launch_to_lanes(h, M);
+    launch_to_sell(h, M, M.va, M.sell_va, true);
     return;
   }
   M.sell_wmax = lay.wmax;
@@ -522,7 +528,8 @@ static void prepare_lowprec(gs2_handle* h, DevCsr& M, const HostTri&, int prec) 
     M.va32 = (float*)h->dalloc(sizeof(float) * nz);
     launch_values_to_fp32(h, M, (int64_t)nz);
     // the layout exists (the autotuner may turn it off and on)
-    if (M.sell_chunks > 0 && !M.sell_lanes) {
+    // (lane slices with other lanes than the row tiles would round otherwise)
+    if (M.sell_chunks > 0 && (!M.sell_lanes || M.sell_lanes == choose_lanes(M.mean_row))) {
       const size_t slots = M.sell_slots;
       M.sell_va32 = (float*)h->dalloc(sizeof(float) * slots);
       h->dzero(M.sell_va32, sizeof(float) * slots);
@@ -540,7 +547,8 @@ static void prepare_lowprec(gs2_handle* h, DevCsr& M, const HostTri&, int prec) 
     h->dzero(M.va16, sizeof(__half) * nz);
     launch_values_to_fp16(h, M);
     // the layout exists (the autotuner may turn it off and on)
-    if (M.sell_chunks > 0 && !M.sell_lanes) {
+    // (lane slices with other lanes than the row tiles would round otherwise)
+    if (M.sell_chunks > 0 && (!M.sell_lanes || M.sell_lanes == choose_lanes(M.mean_row))) {
       const size_t slots = M.sell_slots;
       M.sell_va16 = (__half*)h->dalloc(sizeof(__half) * slots);
       h->dzero(M.sell_va16, sizeof(__half) * slots);

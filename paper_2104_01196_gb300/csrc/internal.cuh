@@ -107,8 +107,8 @@ struct DevCsr {
   double* sell_va = nullptr;
   float* sell_va32 = nullptr;
   __half* sell_va16 = nullptr;
-  // Lane slices (sell_lanes = K > 0, FP64 values only), for matrices that the
-  // layout above does not suit: K lanes per row as in the row tiles, so a chunk holds 32 / K
+  // Lane slices (sell_lanes = K > 0), for matrices that the layout above does
+  // not suit: K lanes per row as in the row tiles, so a chunk holds 32 / K
   // rows; lane l of a row takes its l-th K-th part (ceil(length / K)
   // consecutive entries), slot k of the warp's lanes side by side at
   // sell_ptr[c] + 32 k + lane; padding slots have column -1.  Rows of uneven
@@ -415,9 +415,6 @@ void launch_color(gs2_handle* h, const DevCsr& C, const int* rows, const double*
 void launch_to_sell(gs2_handle* h, const DevCsr& M, const double* va, double* sva, bool with_ci);
 void launch_to_sell(gs2_handle* h, const DevCsr& M, const float* va, float* sva, bool with_ci);
 void launch_to_sell(gs2_handle* h, const DevCsr& M, const __half* va, __half* sva, bool with_ci);
-
-// ... and columns into lane slices (M.sell_lanes > 0; columns preset to -1)
-void launch_to_lanes(gs2_handle* h, const DevCsr& M);
 
 // y = M x (accumulate: y += M x) for any tiled matrix M whose columns index x
 void launch_spmv_matrix(gs2_handle* h, const DevCsr& M, const double* x, double* y,

@@ -384,8 +384,39 @@ __global__ void k_to_sell(int n, const int* __restrict__ rp, const int* __restri
   }
 }
 
+// CSR rows into lane slices (DevCsr::sell_lanes), one thread per lane of a row
+template <typename T>
+__global__ void k_to_lanes(int n, int K, const int* __restrict__ rp, const int* __restrict__ ci,
+                           const T* __restrict__ va, const int* __restrict__ cptr,
+                           const int* __restrict__ perm, int* sci, T* sva) {
+  const int64_t total = (int64_t)n * K;
+  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
+       t += (int64_t)gridDim.x * blockDim.x) {
+    const int p = (int)(t / K), l = (int)(t % K);
+    const int row = perm ? perm[p] : p;
+    const int a = rp[row], len = rp[row + 1] - a, seg = (len + K - 1) / K;
+    const int base = cptr[t >> 5] + (int)(t & 31);
+    for (int k = 0; k < seg && l * seg + k < len; ++k) {
+      sva[base + 32 * k] = va[a + l * seg + k];
+      if (sci) sci[base + 32 * k] = ci[a + l * seg + k];
+    }
+  }
+}
+
+template <typename T>
+static void to_lanes(gs2_handle* h, const DevCsr& M, const T* va, T* sva, bool with_ci) {
+  k_to_lanes<T><<<vec_blocks(h, (int64_t)M.n * M.sell_lanes), kVecThreads, 0, h->stream>>>(
+      M.n, M.sell_lanes, M.rp, M.ci, va, M.sell_ptr, M.sell_row, with_ci ? M.sell_ci : nullptr,
+      sva);
+  GS2_LAUNCH_CHECK();
+}
+
 template <typename T>
 static void to_sell(gs2_handle* h, const DevCsr& M, const T* va, T* sva, bool with_ci) {
+  if (M.sell_lanes) {
+    to_lanes(h, M, va, sva, with_ci);
+    return;
+  }
   k_to_sell<T><<<vec_blocks(h, M.n), kVecThreads, 0, h->stream>>>(
       M.n, M.rp, M.ci, va, M.sell_ptr, M.sell_coff, M.sell_off, M.sell_origin,
       with_ci ? M.sell_ci : nullptr, sva);
@@ -399,30 +430,6 @@ void launch_to_sell(gs2_handle* h, const DevCsr& M, const float* va, float* sva,
 }
 void launch_to_sell(gs2_handle* h, const DevCsr& M, const __half* va, __half* sva, bool with_ci) {
   to_sell(h, M, va, sva, with_ci);
-}
-
-// CSR rows into lane slices (DevCsr::sell_lanes), one thread per lane of a row
-__global__ void k_to_lanes(int n, int K, const int* __restrict__ rp, const int* __restrict__ ci,
-                           const double* __restrict__ va, const int* __restrict__ cptr,
-                           const int* __restrict__ perm, int* sci, double* sva) {
-  const int64_t total = (int64_t)n * K;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int p = (int)(t / K), l = (int)(t % K);
-    const int row = perm ? perm[p] : p;
-    const int a = rp[row], len = rp[row + 1] - a, seg = (len + K - 1) / K;
-    const int base = cptr[t >> 5] + (int)(t & 31);
-    for (int k = 0; k < seg && l * seg + k < len; ++k) {
-      sva[base + 32 * k] = va[a + l * seg + k];
-      sci[base + 32 * k] = ci[a + l * seg + k];
-    }
-  }
-}
-
-void launch_to_lanes(gs2_handle* h, const DevCsr& M) {
-  k_to_lanes<<<vec_blocks(h, (int64_t)M.n * M.sell_lanes), kVecThreads, 0, h->stream>>>(
-      M.n, M.sell_lanes, M.rp, M.ci, M.va, M.sell_ptr, M.sell_row, M.sell_ci, M.sell_va);
-  GS2_LAUNCH_CHECK();
 }
 
 // Autotuner probe: milliseconds per launch of M's most frequent kernel with

@@ -629,11 +629,12 @@ k_stencil(int n, int nchunks, const int* __restrict__ cptr, const int* __restric
 // infinity elsewhere cannot reach the row.
 // (Five resident blocks: at the 66 registers ptxas takes unasked, three fit
 // and the uneven rows' sweep takes 91 instead of 70 us; at eight it takes 101.)
-template <int K, class Epi>
+template <int K, typename VT, class Epi>
 __global__ void __launch_bounds__(kRowThreads, 5)
 k_lanes(int n, int nchunks, const int* __restrict__ cptr, const int* __restrict__ ci,
-        const double* __restrict__ va, Epi epi, const int* skip, const int* __restrict__ live,
+        const VT* __restrict__ va, Epi epi, const int* skip, const int* __restrict__ live,
         const int* __restrict__ perm) {
+  using AT = typename ValTraits<VT>::AT;
   pdl_wait();
   if (skip && *skip) return;
   const int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -646,41 +647,41 @@ k_lanes(int n, int nchunks, const int* __restrict__ cptr, const int* __restrict_
   const bool own = p < n;
   const int row = own ? (perm ? __ldg(perm + p) : p) : 0;
   const int* cc = ci + base + lane;
-  const double* vv = va + base + lane;
+  const VT* vv = va + base + lane;
   int c0 = -1, c1 = -1, c2 = -1, c3 = -1;
-  double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+  AT a0 = AT(0), a1 = AT(0), a2 = AT(0), a3 = AT(0);
   auto load = [&](int k) {
     c0 = c1 = c2 = c3 = -1;
-    a0 = a1 = a2 = a3 = 0.0;
-    if (k < L) { c0 = __ldcs(cc); a0 = __ldcs(vv); }
-    if (k + 1 < L) { c1 = __ldcs(cc + 32); a1 = __ldcs(vv + 32); }
-    if (k + 2 < L) { c2 = __ldcs(cc + 64); a2 = __ldcs(vv + 64); }
-    if (k + 3 < L) { c3 = __ldcs(cc + 96); a3 = __ldcs(vv + 96); }
+    a0 = a1 = a2 = a3 = AT(0);
+    if (k < L) { c0 = __ldcs(cc); a0 = stream_val<VT>(vv); }
+    if (k + 1 < L) { c1 = __ldcs(cc + 32); a1 = stream_val<VT>(vv + 32); }
+    if (k + 2 < L) { c2 = __ldcs(cc + 64); a2 = stream_val<VT>(vv + 64); }
+    if (k + 3 < L) { c3 = __ldcs(cc + 96); a3 = stream_val<VT>(vv + 96); }
     cc += 128;
     vv += 128;
   };
   load(0);
   typename Epi::Pre pv{};
   if (own) pv = epi.pre(row);
-  double s = l == 0 ? epi.begin(pv) : 0.0;
+  AT s = l == 0 ? epi.begin(pv) : AT(0);
   for (int k = 0; k < L; k += 4) {
-    const double x0 = c0 >= 0 ? epi.gather(c0) : 0.0;
-    const double x1 = c1 >= 0 ? epi.gather(c1) : 0.0;
-    const double x2 = c2 >= 0 ? epi.gather(c2) : 0.0;
-    const double x3 = c3 >= 0 ? epi.gather(c3) : 0.0;
-    const double b0 = a0, b1 = a1, b2 = a2, b3 = a3;
+    const AT x0 = c0 >= 0 ? (AT)epi.gather(c0) : AT(0);
+    const AT x1 = c1 >= 0 ? (AT)epi.gather(c1) : AT(0);
+    const AT x2 = c2 >= 0 ? (AT)epi.gather(c2) : AT(0);
+    const AT x3 = c3 >= 0 ? (AT)epi.gather(c3) : AT(0);
+    const AT b0 = a0, b1 = a1, b2 = a2, b3 = a3;
     load(k + 4);
     s = row_fma<Epi>(b0, x0, s);
     if (k + 1 < L) s = row_fma<Epi>(b1, x1, s);
     if (k + 2 < L) s = row_fma<Epi>(b2, x2, s);
     if (k + 3 < L) s = row_fma<Epi>(b3, x3, s);
   }
-  if (K > 1) s = group_sum<K, double>(s);
+  if (K > 1) s = group_sum<K, AT>(s);
   if (own && l == 0) epi.finish(row, s, pv);
 }
 
 inline const double* sell_values(const DevCsr& M, const double*) { return M.sell_va; }
-// (lane slices hold FP64 values only: sell_va32 and sell_va16 are null there)
+// (null where the layout holds no copy in that precision: row tiles)
 inline const float* sell_values(const DevCsr& M, const float*) { return M.sell_va32; }
 inline const __half* sell_values(const DevCsr& M, const __half*) { return M.sell_va16; }
 
@@ -720,14 +721,14 @@ inline const int* live_rows(const gs2_handle* h, const DevCsr& M) {
   return (h->row_live && (&M == &h->A || &M == &h->L || &M == &h->U)) ? h->row_live : nullptr;
 }
 
-template <class Epi>
-inline void launch_lanes(gs2_handle* h, const DevCsr& M, const double* sv, const Epi& epi,
+template <typename VT, class Epi>
+inline void launch_lanes(gs2_handle* h, const DevCsr& M, const VT* sv, const Epi& epi,
                          const int* skip) {
-  auto fn = M.sell_lanes == 1   ? k_lanes<1, Epi>
-            : M.sell_lanes == 2 ? k_lanes<2, Epi>
-            : M.sell_lanes == 4 ? k_lanes<4, Epi>
-            : M.sell_lanes == 8 ? k_lanes<8, Epi>
-                                : k_lanes<16, Epi>;
+  auto fn = M.sell_lanes == 1   ? k_lanes<1, VT, Epi>
+            : M.sell_lanes == 2 ? k_lanes<2, VT, Epi>
+            : M.sell_lanes == 4 ? k_lanes<4, VT, Epi>
+            : M.sell_lanes == 8 ? k_lanes<8, VT, Epi>
+                                : k_lanes<16, VT, Epi>;
   const int warps = kRowThreads / 32;
   const int grid = (M.sell_chunks + warps - 1) / warps;
   launch_pdl(fn, grid, kRowThreads, 0, h->stream, M.n, M.sell_chunks, (const int*)M.sell_ptr,
@@ -783,11 +784,9 @@ inline void dispatch(gs2_handle* h, const DevCsr& M, const VT* va, const Epi& ep
                      const int* skip) {
   const VT* sv = M.sell ? sell_values(M, va) : nullptr;
   if (sv) {
-    if constexpr (sizeof(VT) == sizeof(double)) {
-      if (M.sell_lanes) {
-        launch_lanes<Epi>(h, M, sv, epi, skip);
-        return;
-      }
+    if (M.sell_lanes) {
+      launch_lanes<VT, Epi>(h, M, sv, epi, skip);
+      return;
     }
     launch_sell<VT, Epi>(h, M, sv, epi, skip);
     return;
