@@ -267,6 +267,7 @@ void retile(gs2_handle* h, DevCsr& M, const std::vector<int>& rp, int K, int RPT
 // 13.0 -> 10.5), and stay in the row tiles elsewhere.
 constexpr int kSellC = 32;                       // rows per chunk (one warp)
 constexpr double kSellMaxPadding = 1.2;          // slots / entries
+constexpr int kSellSmall = 1 << 18;  // entries up to which lane slices may pad to double
 constexpr double kSellStreamBytes = 128.0 * (1 << 20);  // CSR bytes beyond L2
 
 // (With `origin`, offsets are j - origin[i]: a colour's rows, origin[i] their row
@@ -365,13 +366,17 @@ struct LaneLayout {
 
 static bool lane_layout(const std::vector<int>& rp, int n, int K, LaneLayout& out) {
   const int per = 32 / K;
+  // (in a matrix of a few MB of long rows padding costs no time to speak of:
+  // the 2,386 rows of a third multigrid level, 33 entries in a triangle)
+  const bool small = rp[n] <= kSellSmall && rp[n] > kShortRowMean * n;
+  const double padding = small ? 2.0 : kSellMaxPadding;
   std::vector<int> width(n);
   for (int i = 0; i < n; ++i) width[i] = (rp[i + 1] - rp[i] + K - 1) / K;
   auto chunks = [&](const std::vector<int>& row) {
     out.cptr.assign((n + per - 1) / per + 1, 0);
     int64_t total = 0;
     for (size_t c = 0; c + 1 < out.cptr.size(); ++c) {
-      if (total > kSellMaxPadding * rp[n]) return false;
+      if (total > padding * rp[n]) return false;
       int w = 0;
       for (int p = (int)c * per; p < std::min(n, ((int)c + 1) * per); ++p)
         w = std::max(w, width[row.empty() ? p : row[p]]);
@@ -379,7 +384,7 @@ static bool lane_layout(const std::vector<int>& rp, int n, int K, LaneLayout& ou
       if (total > INT32_MAX) return false;
       out.cptr[c + 1] = (int)total;
     }
-    return total <= kSellMaxPadding * rp[n];
+    return total <= padding * rp[n];
   };
   out.row.clear();
   if (chunks(out.row)) return true;
@@ -428,9 +433,18 @@ static void upload_sell(gs2_handle* h, DevCsr& M, const std::vector<int>& rp, co
   // 3% lost on 64^3)
   const bool few = &M == &h->A && !short_rows && streams &&
                    n < 2 * 32 * (int64_t)kSellWarpsPerSm * h->nsm && try_lanes(1);
-  const bool sliced = !few && (short_rows || streams) && sell_layout(rp, ci, n, origin, lay);
+  bool sliced = !few && (short_rows || streams) && sell_layout(rp, ci, n, origin, lay);
+  // rows with explicit columns, too few for the SMs' warps at one lane each
+  // (the 64,560 rows of a second multigrid level, 15 entries in a triangle:
+  // inner sweep 12.6 -> 8.6 us with two lanes)
+  if (sliced && lay.offset_chunks == 0 && !h->for_pack &&
+      lane_count(h, n, M.mean_row, longest) > 1 &&
+      try_lanes(lane_count(h, n, M.mean_row, longest)))
+    sliced = false;
   // rows of uneven length, and long rows in a matrix that fits L2
-  if (!few && !sliced && !try_lanes(lane_count(h, n, M.mean_row, longest))) return;  // row tiles
+  if (!few && !sliced && M.sell_lanes == 0 &&
+      !try_lanes(lane_count(h, n, M.mean_row, longest)))
+    return;  // row tiles
   const std::vector<int>& cptr = sliced ? lay.cptr : lanes.cptr;
   const size_t slots = std::max(cptr.back(), 1);
   std::vector<int> top(kHostThreads, 0);

@@ -65,10 +65,12 @@ struct Group {
 };
 
 // Bytes of the sliced-ELL copy of a matrix with this many entries (at most
-// 1.2 slots per entry, else no copy is made) holding vbytes-byte values, with
+// 1.2 slots per entry, 2 in a small matrix, else no copy is made) holding
+// vbytes-byte values, with
 // its chunk offsets and row order (lane slices: up to a chunk per two rows).
 static int64_t sell_bytes(int64_t entries, int64_t n, int vbytes) {
-  return (entries * 6 / 5 + 1) * (4 + vbytes) + 4 * (n / 2 + 2) + 4 * n;
+  const int64_t slots = entries <= (1 << 18) ? 2 * entries + 1 : entries * 6 / 5 + 1;
+  return slots * (4 + vbytes) + 4 * (n / 2 + 2) + 4 * n;
 }
 
 // Device bytes a request of this size holds once admitted: the matrix, its
