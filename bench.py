@@ -608,7 +608,7 @@ def run_ours(args):
             if not args.no_profile:
                 tab, _ = profiled(h, torch, stream, sp, 0, hbm, n, nnz)
                 row["kernels"] = {k: v for k, v in tab.items()
-                                  if k.startswith(("inner", "resid", "spmv", "rhat", "to32"))}
+                                  if k.startswith(("inner", "resid", "spmv", "rhat", "sweep32"))}
             res[prec] = row
         out["precision"] = res
     h.close()

@@ -498,8 +498,17 @@ static void cycle(AmgHierarchy* H, size_t l, const gs2_params& sp, const double*
   AmgLevel& C = H->lv[l + 1];
   precond_apply(hl, &pre, b, x, rhat_ready, skip);           // x = S_pre(b) from zero
   launch_resid(hl, b, x, L.r, nullptr, nullptr, skip);       // r = b - A x
-  launch_spmv_matrix(hl, L.R, L.r, C.b, false, skip);        // b_c = R r
-  cycle(H, l + 1, sp, C.b, C.x, false, skip);                // x_c
+  // b_c = R r, and with it the D^{-1} b_c that the coarse smoother starts from
+  // (a launch of its own otherwise, 3 us a level)
+  gs2_handle* hc = C.h;
+  const void* rb = l + 2 < H->lv.size() ? precond_rhat_buffer(hc, &pre) : nullptr;
+  const bool ready = rb != nullptr;
+  if (ready)
+    launch_restrict(hl, L.R, L.r, C.b, hc->dinv, rb == hc->rhat ? hc->rhat : nullptr,
+                    rb == hc->rhat32 ? hc->rhat32 : nullptr, skip);
+  else
+    launch_spmv_matrix(hl, L.R, L.r, C.b, false, skip);
+  cycle(H, l + 1, sp, C.b, C.x, ready, skip);                // x_c
   launch_spmv_matrix(hl, L.P, C.x, x, true, skip);           // x += P x_c
   smooth_sweeps(hl, &post, b, x, skip);                      // x = S_post(b, x)
 }

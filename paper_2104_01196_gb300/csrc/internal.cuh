@@ -377,11 +377,11 @@ void launch_rhat_update(gs2_handle* h, int prec, const void* rhat, double* x,
 // GS2_FP16_ROWSCALED): rhat32 = fl32(D^{-1} b) - x32 - O x32 in FP32 (bhat32
 // and x32 of the handle, O = D^{-1}(L + U)); the update of a sweep with no
 // inner sweep, x32 / x from rhat (mode: one of the x32 InnerModes); and the
-// conversion x32 = fl32(x).
+// start of a call, x32 = fl32(x) and bhat32 = fl32(D^{-1} b).
 void launch_resid_sweep(gs2_handle* h, int vprec, const int* skip);
 void launch_rhat_update32(gs2_handle* h, const float* rhat, double* x, double omega, int mode,
                           const int* skip);
-void launch_to32(gs2_handle* h, const double* x, float* x32, const int* skip);
+void launch_sweep32_begin(gs2_handle* h, const double* b, const double* x, const int* skip);
 // M's FP64 values (the nz entries of va, padding included) to M.va32; to
 // M.va16 with the per-row power-of-two scale exponents M.scale16 (the FP16
 // row-scaled precision)
@@ -419,6 +419,9 @@ void launch_to_sell(gs2_handle* h, const DevCsr& M, const __half* va, __half* sv
 // y = M x (accumulate: y += M x) for any tiled matrix M whose columns index x
 void launch_spmv_matrix(gs2_handle* h, const DevCsr& M, const double* x, double* y,
                         bool accumulate, const int* skip);
+// y = M x and rhat = dinv y in the sweep precision (whichever is non-null)
+void launch_restrict(gs2_handle* h, const DevCsr& M, const double* x, double* y,
+                     const double* dinv, double* rhat64, float* rhat32, const int* skip);
 
 void launch_axpy(gs2_handle* h, double* y, double a, const double* x,
                  const int* skip);

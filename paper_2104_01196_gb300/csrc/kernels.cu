@@ -74,6 +74,31 @@ struct EpiSpmv {
   __device__ void finish(int i, double s, const Pre&) const { y[i] = s; }
 };
 
+// y = M x and rhat = D^{-1} y with another matrix's diagonal (multigrid
+// restriction: the coarse level's smoother starts from D^{-1} b_c)
+struct EpiRestrict {
+  static constexpr bool kSub = false;
+  static constexpr int kUnroll = 8;
+  static constexpr bool kGuard = false;
+  const double* __restrict__ x;
+  const double* __restrict__ dinv;
+  double* __restrict__ y;
+  double* __restrict__ rhat64;
+  float* __restrict__ rhat32;
+  struct Pre {
+    double d;
+  };
+  __device__ int origin(int i, const Pre&) const { return i; }
+  __device__ Pre pre(int i) const { return Pre{dinv[i]}; }
+  __device__ double gather(int c) const { return __ldg(x + c); }
+  __device__ double begin(const Pre&) const { return 0.0; }
+  __device__ void finish(int i, double s, const Pre& p) const {
+    y[i] = s;
+    if (rhat64) rhat64[i] = p.d * s;
+    if (rhat32) rhat32[i] = (float)(p.d * s);
+  }
+};
+
 // y += M x (multigrid prolongation)
 struct EpiSpmvAdd {
   static constexpr bool kSub = false;
@@ -335,6 +360,14 @@ void launch_spmv_matrix(gs2_handle* h, const DevCsr& M, const double* x, double*
     EpiSpmv e{x, y};
     dispatch<double>(h, M, M.va, e, skip);
   }
+}
+
+void launch_restrict(gs2_handle* h, const DevCsr& M, const double* x, double* y,
+                     const double* dinv, double* rhat64, float* rhat32, const int* skip) {
+  KernelTimer tm(h, "amg_restrict",
+                 bytes_csr(M, 8) + 24.0 * M.n + (rhat64 ? 8.0 : 4.0) * M.n);
+  EpiRestrict e{x, dinv, y, rhat64, rhat32};
+  dispatch<double>(h, M, M.va, e, skip);
 }
 
 __device__ __forceinline__ void add_to(double* p, double v) { *p += v; }
@@ -605,11 +638,16 @@ __global__ void k_rhat_update32(int n, const float* __restrict__ rhat, float* x3
   }
 }
 
-__global__ void k_to32(int n, const double* __restrict__ x, float* x32, const int* skip) {
+// start of a whole-sweep-precision call: x32 = fl32(x), bhat32 = fl32(D^{-1} b)
+__global__ void k_sweep32_begin(int n, const double* __restrict__ x, const double* __restrict__ b,
+                                const double* __restrict__ dinv, float* __restrict__ x32,
+                                float* __restrict__ bhat32, const int* skip) {
   pdl_wait();
   if (skip && *skip) return;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     x32[i] = (float)x[i];
+    bhat32[i] = (float)(dinv[i] * b[i]);
+  }
 }
 
 __global__ void k_values_to_fp32(int64_t nz, const double* __restrict__ va, float* va32) {
@@ -699,10 +737,11 @@ void launch_values_to_fp16(gs2_handle* h, const DevCsr& M) {
   GS2_LAUNCH_CHECK();
 }
 
-void launch_to32(gs2_handle* h, const double* x, float* x32, const int* skip) {
+void launch_sweep32_begin(gs2_handle* h, const double* b, const double* x, const int* skip) {
   if (h->n == 0) return;
-  KernelTimer tm(h, "to32", 12.0 * h->n);
-  launch_pdl(k_to32, vec_blocks(h, h->n), kVecThreads, 0, h->stream, (int)h->n, x, x32, skip);
+  KernelTimer tm(h, "sweep32_begin", 32.0 * h->n);
+  launch_pdl(k_sweep32_begin, vec_blocks(h, h->n), kVecThreads, 0, h->stream, (int)h->n, x, b,
+             h->dinv, h->x32, h->bhat32, skip);
   GS2_LAUNCH_CHECK();
 }
 

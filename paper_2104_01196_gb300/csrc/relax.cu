@@ -127,8 +127,7 @@ static void gs2_half_sweep32(gs2_handle* h, const gs2_params* p, const DevCsr& T
 static void sweep32_relax(gs2_handle* h, const gs2_params* p, const double* b, double* x,
                           bool x_zero, int sweeps, const int* skip) {
   if (!x_zero) {
-    launch_to32(h, x, h->x32, skip);
-    launch_prep_rhat(h, b, nullptr, h->bhat32, skip);
+    launch_sweep32_begin(h, b, x, skip);
   }
   const bool fwd = p->direction == GS2_FORWARD || p->direction == GS2_SYMMETRIC;
   const bool bwd = p->direction == GS2_BACKWARD || p->direction == GS2_SYMMETRIC;
