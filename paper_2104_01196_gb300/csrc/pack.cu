@@ -60,7 +60,7 @@ struct Pack {
   int gb = 1, gs = 1;
   int m = 0;                       // restart the arrays below are sized for
   double *H = nullptr, *hbuf = nullptr, *gvec = nullptr, *cs = nullptr, *sn = nullptr,
-         *y = nullptr, *part = nullptr;
+         *y = nullptr, *part = nullptr, *part2 = nullptr;
   // captured Arnoldi steps of one cycle
   cudaGraphExec_t gexec = nullptr;
   std::vector<double> gkey;
@@ -104,13 +104,15 @@ k_pdots(int ld, const int4* __restrict__ blk, const int* __restrict__ items,
   }
 }
 
-// w -= V h (h of the item's system); then p = V^T w or p = w^T w
+// w -= V h (h of the item's system, summed from the pass before's partials
+// cpart of its blocks; its first block writes them to column j of H, mode 0,
+// or adds them, mode 1); then p = V^T w or p = w^T w
 template <int JC, bool NORM>
 __global__ void __launch_bounds__(kVecThreads)
 k_pupdate(int ld, const int4* __restrict__ blk, const int* __restrict__ items,
           const int* __restrict__ nitems, const KrylovState* st, const double* __restrict__ V,
-          const double* __restrict__ hbuf, int hb_stride, double* __restrict__ w, double* part,
-          int nb) {
+          const double* __restrict__ cpart, const int* __restrict__ seg_blk, double* H,
+          size_t hstride, size_t hcol, int mode, double* __restrict__ w, double* part, int nb) {
   pdl_wait();
   __shared__ double hneg[JC];
   const int nq = *nitems;
@@ -118,9 +120,8 @@ k_pupdate(int ld, const int4* __restrict__ blk, const int* __restrict__ items,
     const int e = items[q];
     const int4 b = blk[e];
     if (st[b.x].stop) continue;
-    for (int k = threadIdx.x; k < JC; k += blockDim.x)
-      hneg[k] = -hbuf[(size_t)b.x * hb_stride + k];
-    __syncthreads();
+    sum_columns<JC>(cpart, nb, seg_blk[b.x], seg_blk[b.x + 1], hneg,
+                    b.w ? H + b.x * hstride + hcol : nullptr, mode);
     constexpr int NA = NORM ? 1 : JC;
     double acc[NA];
 #pragma unroll
@@ -603,6 +604,7 @@ static void ensure_pack_krylov(gs2_handle* h, int m) {
   P->sn = (double*)h->dalloc(sizeof(double) * S * P->vstride());
   P->y = (double*)h->dalloc(sizeof(double) * S * P->vstride());
   P->part = (double*)h->dalloc(sizeof(double) * (size_t)(m + 2) * std::max(1, P->nb));
+  P->part2 = (double*)h->dalloc(sizeof(double) * (size_t)(m + 2) * std::max(1, P->nb));
   h->dzero(P->H, sizeof(double) * S * P->hstride());
 }
 
@@ -774,49 +776,55 @@ struct PackRun {
     launch_cycle();
   }
 
-  int launch_dots(int jc) {
+  int launch_dots(int jc, double* part) {
     KernelTimer tm(h, "cgs2_dots", 8.0 * h->n * (jc + 1));
     const int N = (int)h->n;
     switch (jc) {
 #define GS2_PDOTS_CASE(J)                                                               \
   case J:                                                                               \
     launch_pdl(k_pdots<J>, P->gb, kVecThreads, 0, h->stream, N, P->blk, P->items, P->cnt, P->st, h->V,  \
-               h->w, P->part, P->nb);                                                               \
+               h->w, part, P->nb);                                                               \
     break;
       GS2_PJC_CASES(GS2_PDOTS_CASE)
 #undef GS2_PDOTS_CASE
       default:
         launch_pdl(k_pdots_rt<64>, P->gb, kVecThreads, 0, h->stream, N, P->blk, P->items, P->cnt, P->st,
-                   h->V, jc, h->w, P->part, P->nb);
+                   h->V, jc, h->w, part, P->nb);
         break;
     }
     GS2_LAUNCH_CHECK();
     return P->nb;
   }
 
+  // the update pass of step j: the coefficients from the partials cpart of the
+  // pass before (more than 32 of them: reduced into hbuf by launch_reduce)
   template <bool NORM>
-  void launch_update(int jc) {
+  void launch_update(int j, const double* cpart, double* part) {
+    const int jc = j + 1, mode = NORM ? 1 : 0;
+    if (jc > 32) launch_reduce(j, jc, mode, cpart);
     KernelTimer tm(h, NORM ? "cgs2_upd_norm" : "cgs2_upd_dots", 8.0 * h->n * (jc + 2));
     const int N = (int)h->n, hs = (int)P->vstride();
+    const size_t hcol = (size_t)j * ldh();
     switch (jc) {
-#define GS2_PUPD_CASE(J)                                                                \
-  case J:                                                                               \
-    launch_pdl(k_pupdate<J, NORM>, P->gb, kVecThreads, 0, h->stream, N, P->blk, P->items, P->cnt,     \
-               P->st, h->V, P->hbuf, hs, h->w, P->part, P->nb);                                        \
+#define GS2_PUPD_CASE(J)                                                                         \
+  case J:                                                                                        \
+    launch_pdl(k_pupdate<J, NORM>, P->gb, kVecThreads, 0, h->stream, N, P->blk, P->items,        \
+               P->cnt, P->st, h->V, cpart, P->seg_blk, P->H, P->hstride(), hcol, mode, h->w,     \
+               part, P->nb);                                                                     \
     break;
       GS2_PJC_CASES(GS2_PUPD_CASE)
 #undef GS2_PUPD_CASE
       default:
-        launch_pdl(k_pupdate_rt<64, NORM>, P->gb, kVecThreads, 0, h->stream, N, P->blk, P->items, P->cnt,
-                   P->st, h->V, jc, P->hbuf, hs, h->w, P->part, P->nb);
+        launch_pdl(k_pupdate_rt<64, NORM>, P->gb, kVecThreads, 0, h->stream, N, P->blk, P->items,
+                   P->cnt, P->st, h->V, jc, P->hbuf, hs, h->w, part, P->nb);
         break;
     }
     GS2_LAUNCH_CHECK();
   }
 
-  void launch_reduce(int j, int jc, int mode) {
+  void launch_reduce(int j, int jc, int mode, const double* part) {
     KernelTimer tm(h, "reduce_cols", 8.0 * jc * P->nb);
-    launch_pdl(k_preduce, P->gs, 256, 0, h->stream, P->part, P->nb, P->seg_blk, P->sys, P->cnt + 1, P->st,
+    launch_pdl(k_preduce, P->gs, 256, 0, h->stream, part, P->nb, P->seg_blk, P->sys, P->cnt + 1, P->st,
                P->H, P->hstride(), ldh(), j, P->hbuf, (int)P->vstride(), mode, jc);
     GS2_LAUNCH_CHECK();
   }
@@ -835,12 +843,10 @@ struct PackRun {
     LiveRows lr(h, P->live_run);
     precond_apply(h, pc, h->V + (size_t)j * N, h->z, wants, skip);
     launch_spmv(h, h->z, h->w, skip);
-    const int jc = j + 1;
-    launch_dots(jc);
-    launch_reduce(j, jc, 0);
-    launch_update<false>(jc);
-    launch_reduce(j, jc, 1);
-    launch_update<true>(jc);
+    // (the passes alternate between two partial-sum buffers)
+    launch_dots(j + 1, P->part);
+    launch_update<false>(j, P->part, P->part2);
+    launch_update<true>(j, P->part2, P->part);
     {
       KernelTimer tm(h, "givens", 8.0 * P->nb + 8.0 * 4 * (j + 2) * P->count);
       launch_pdl(k_pgivens, P->gs, 128, 0, h->stream, P->part, P->seg_blk, P->sys, P->cnt + 1, P->st, P->H,

@@ -160,4 +160,33 @@ __device__ __forceinline__ void block_partials(const double (&acc)[NV], int nv, 
   block_partials<NV>(acc, nv, part, nblk, (int)blockIdx.x);
 }
 
+// Column sums of a kernel's partials by every block of the kernel that needs
+// them: hneg[v] = -sum_{b0 <= b < b1} part[v * ld + b] for v < JC, and with
+// `col` non-null (one block) H's column: col[v] = the sum (mode 0) or += it
+// (mode 1).  Eight lanes a coefficient, 32 coefficients at a time in a block
+// of 256 threads: a fixed order that depends on b1 - b0 only.  For the few
+// dozen partials of a pack's system this replaces a kernel of its own (48
+// systems, 56.3 -> 52.4 us an Arnoldi step); for the 152 partials a column of
+// a single system of 185,193 rows it cost more than the kernel (61.8 -> 63.9).
+// Ends in a block barrier.
+template <int JC>
+__device__ __forceinline__ void sum_columns(const double* __restrict__ part, int ld, int b0,
+                                            int b1, double* hneg, double* col, int mode) {
+  const int lane8 = threadIdx.x & 7;
+  for (int v = threadIdx.x >> 3; v < (JC + 3) / 4 * 4; v += kVecThreads / 8) {
+    double s = 0.0;
+    if (v < JC) {
+#pragma unroll 4
+      for (int b = b0 + lane8; b < b1; b += 8) s += part[(size_t)v * ld + b];
+    }
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (v < JC && lane8 == 0) {
+      hneg[v] = -s;
+      if (col) col[v] = mode == 0 ? s : col[v] + s;
+    }
+  }
+  __syncthreads();
+}
+
 }  // namespace gs2
