@@ -434,10 +434,12 @@ static void upload_sell(gs2_handle* h, DevCsr& M, const std::vector<int>& rp, co
   const bool few = &M == &h->A && !short_rows && streams &&
                    n < 2 * 32 * (int64_t)kSellWarpsPerSm * h->nsm && try_lanes(1);
   bool sliced = !few && (short_rows || streams) && sell_layout(rp, ci, n, origin, lay);
-  // rows with explicit columns, too few for the SMs' warps at one lane each
-  // (the 64,560 rows of a second multigrid level, 15 entries in a triangle:
-  // inner sweep 12.6 -> 8.6 us with two lanes)
-  if (sliced && lay.offset_chunks == 0 && !h->for_pack &&
+  // short rows with explicit columns, too few for the SMs' warps at one lane
+  // each (the 64,560 rows of a second multigrid level, 15 entries in a
+  // triangle: inner sweep 12.6 -> 8.6 us with two lanes); long rows here
+  // stream and keep one lane (Q1 elasticity on 64^3 nodes, residual 126 us
+  // against 150 with four)
+  if (sliced && short_rows && lay.offset_chunks == 0 && !h->for_pack &&
       lane_count(h, n, M.mean_row, longest) > 1 &&
       try_lanes(lane_count(h, n, M.mean_row, longest)))
     sliced = false;
