@@ -741,27 +741,32 @@ static void find_levels(const HostTri& T, int n, bool lower, HostLevels& out) {
   for (int p = 0; p < n; ++p) out.rp[p + 1] += out.rp[p];
 }
 
-// both triangles of one splitting, found side by side
+// both triangles of one splitting, found side by side when they are large
 static void build_levels(gs2_handle* h, const HostTri& L, const HostTri& U, const DevCsr& dL,
                          const DevCsr& dU, TriSolve& tL, TriSolve& tU) {
   const int n = (int)h->n;
   HostLevels hl[2];
-  std::exception_ptr failed;
-  std::thread other([&] {
-    try {
-      find_levels(L, n, true, hl[0]);
-    } catch (...) {
-      failed = std::current_exception();
-    }
-  });
-  try {
+  if (n < 32768) {  // (sooner done than a thread is started)
+    find_levels(L, n, true, hl[0]);
     find_levels(U, n, false, hl[1]);
-  } catch (...) {
+  } else {
+    std::exception_ptr failed;
+    std::thread other([&] {
+      try {
+        find_levels(L, n, true, hl[0]);
+      } catch (...) {
+        failed = std::current_exception();
+      }
+    });
+    try {
+      find_levels(U, n, false, hl[1]);
+    } catch (...) {
+      other.join();
+      throw;
+    }
     other.join();
-    throw;
+    if (failed) std::rethrow_exception(failed);
   }
-  other.join();
-  if (failed) std::rethrow_exception(failed);
   tL.levels = hl[0].levels;
   tU.levels = hl[1].levels;
   tri_upload(h, dL, hl[0].rows, hl[0].rp, tL);

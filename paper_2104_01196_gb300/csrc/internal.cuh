@@ -271,7 +271,7 @@ struct gs2_handle {
   cudaStream_t gstream = nullptr;
   cudaEvent_t gev_in = nullptr, gev_out = nullptr;
   cudaGraphExec_t gexec = nullptr;
-  std::vector<double> gkey;
+  std::vector<double> gkey, gseen;  // gseen: the shape of a cycle run without a graph
   // CG: a chunk of iterations as one graph (same stream and events)
   cudaGraphExec_t cg_gexec = nullptr;
   std::vector<double> cg_gkey;
@@ -643,8 +643,9 @@ int vec_blocks(gs2_handle* h, int64_t n);
 constexpr int kVecThreads = 256;
 constexpr int kRowThreads = 256;
 // Mean row length up to which one lane per row is the natural width: such
-// matrices always get a sliced-ELL copy (when it pads little), longer rows
-// only when they stream from HBM, and then take the pipelined instantiation.
+// matrices get a sliced-ELL copy (when it pads little), longer rows when they
+// stream from HBM, and then take the pipelined instantiation; the others get
+// lane slices (upload_sell).
 constexpr double kShortRowMean = 24.0;
 constexpr int kMaxRestart = 64;
 

@@ -13,7 +13,8 @@
 // spend more FP64 issue slots on the tree than on the products.  Rows are
 // therefore reduced sequentially by one thread (or by K contiguous segments
 // for long rows), with each tile's row pointers, columns and values staged
-// into shared memory by TMA bulk copies (tiles.cuh).  x-gathers go through
+// into shared memory by TMA bulk copies, or laid out as slices that a warp
+// reads straight from memory (tiles.cuh).  x-gathers go through
 // the read-only path and stay L2-resident.  (Fusing the SpMV with the first
 // Gram-Schmidt dot pass of an Arnoldi step was measured: the fused kernel
 // reached only ~0.65 of both the HBM and the FP64 rate, 3% faster than the

@@ -26,6 +26,10 @@
 // Laplacian (298 levels) 2908 -> 512 us, 0.8 us a level; 500^2 Laplacian (999
 // levels) 6508 -> 1099; 40^2 426 -> 75; Q1 elasticity on 20^3 nodes 5931 ->
 // 900.  One, two and four blocks per SM differ by 3%.
+#include <algorithm>
+#include <cstring>
+#include <vector>
+
 #include "tiles.cuh"
 
 namespace gs2 {
@@ -173,16 +177,27 @@ void tri_upload(gs2_handle* h, const DevCsr& M, const std::vector<int>& rows,
     for (int p = T.levels[v]; p < T.levels[v + 1]; p += per)
       chunk.push_back(make_int2(p, std::min(per, T.levels[v + 1] - p)));
   T.nchunks = (int)chunk.size();
-  T.rows = (int*)h->dalloc(sizeof(int) * n);
-  T.rp = (int*)h->dalloc(sizeof(int) * (n + 1));
-  T.ci = (int*)h->dalloc(sizeof(int) * std::max(M.nnz, 1));
-  T.va = (double*)h->dalloc(sizeof(double) * std::max(M.nnz, 1));
-  T.chunk = (int2*)h->dalloc(sizeof(int2) * chunk.size());
-  T.g = (unsigned long long*)h->dalloc(sizeof(double) * n);
-  T.ticket = (int*)h->dalloc(sizeof(int));
-  h->h2d(T.rows, rows.data(), sizeof(int) * n);
-  h->h2d(T.rp, rp.data(), sizeof(int) * (n + 1));
-  h->h2d(T.chunk, chunk.data(), sizeof(int2) * chunk.size());
+  // one allocation, and one upload of rows, entry places and chunks
+  const size_t head = sizeof(int) * (2 * (size_t)n + 2) + sizeof(int2) * chunk.size();
+  auto up = [](size_t x) { return (x + 255) / 256 * 256; };
+  char* base = (char*)h->dalloc(up(head) + up(sizeof(int) * M.nnz) + up(sizeof(double) * M.nnz) +
+                                up(sizeof(double) * n) + sizeof(int));
+  std::vector<int> host(head / sizeof(int));
+  std::copy(rows.begin(), rows.end(), host.begin());
+  std::copy(rp.begin(), rp.end(), host.begin() + n);
+  std::memcpy(host.data() + 2 * (size_t)n + 2, chunk.data(), sizeof(int2) * chunk.size());
+  h->h2d(base, host.data(), head);
+  T.rows = (int*)base;
+  T.rp = T.rows + n;
+  T.chunk = (int2*)(T.rows + 2 * (size_t)n + 2);
+  base += up(head);
+  T.ci = (int*)base;
+  base += up(sizeof(int) * M.nnz);
+  T.va = (double*)base;
+  base += up(sizeof(double) * M.nnz);
+  T.g = (unsigned long long*)base;
+  base += up(sizeof(double) * n);
+  T.ticket = (int*)base;
   // the column -> place map is needed only here: it lies in g until the
   // first solve
   int* place = (int*)T.g;
