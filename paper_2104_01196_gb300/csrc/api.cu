@@ -303,8 +303,9 @@ static bool sell_layout(const std::vector<int>& rp, const int* ci, int n, const 
     bool regular = true;
     for (int i = c * kSellC; i < std::min(n, (c + 1) * kSellC); ++i) {
       L = std::max(L, rp[i + 1] - rp[i]);
+      const int at = origin ? origin[i] : i;
       for (int k = rp[i]; regular && k < rp[i + 1]; ++k) {
-        const int o = ci[k] - (origin ? origin[i] : i);
+        const int o = ci[k] - at;
         if (std::find(u.begin(), u.end(), o) == u.end()) {
           u.push_back(o);
           if ((int)u.size() > kOffsetMax) regular = false;

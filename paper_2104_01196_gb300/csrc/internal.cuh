@@ -271,7 +271,8 @@ struct gs2_handle {
   cudaStream_t gstream = nullptr;
   cudaEvent_t gev_in = nullptr, gev_out = nullptr;
   cudaGraphExec_t gexec = nullptr;
-  std::vector<double> gkey, gseen;  // gseen: the shape of a cycle run without a graph
+  std::vector<double> gkey, gseen;  // gseen: the shape of the last cycles without a graph,
+  int gseen_cycles = 0;             // and how many they were
   // CG: a chunk of iterations as one graph (same stream and events)
   cudaGraphExec_t cg_gexec = nullptr;
   std::vector<double> cg_gkey;

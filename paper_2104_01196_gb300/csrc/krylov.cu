@@ -621,17 +621,20 @@ struct GmresRun {
     return key;
   }
 
-  // Automatic mode: the first cycle of a shape on a handle runs as separate
-  // launches, a graph is captured when a second one comes -- capture and
-  // instantiation cost about 1 ms, more than the launch gaps of one cycle (a
-  // new system of 185,193 rows, 23 iterations: 2.5 -> 1.8 ms).
-  bool first_cycle() {
+  // Automatic mode: the first cycles of a shape on a handle run as separate
+  // launches; a graph is captured once a few have.  Capture and instantiation
+  // cost 1 ms (with a V-cycle in each step 3.5), a replay saves 3% to 6% of a
+  // cycle (a new system of 185,193 rows, 23 iterations: 2.5 -> 1.8 ms).
+  static constexpr int kEagerCycles = 4;
+  bool eager_cycle() {
     if (h->graph_mode != 0 || profiling_active(h)) return false;
     std::vector<double> key = graph_key();
     if (h->gexec && h->gkey == key) return false;
-    if (h->gseen == key) return false;
-    h->gseen = std::move(key);
-    return true;
+    if (h->gseen != key) {
+      h->gseen = std::move(key);
+      h->gseen_cycles = 0;
+    }
+    return h->gseen_cycles++ < kEagerCycles;
   }
 
   // Capture (once per cycle shape) without running anything: host work
@@ -686,7 +689,7 @@ struct GmresRun {
                r64, r32, h->gvec, m, h->st);
     GS2_LAUNCH_CHECK();
     cycle_ran = true;
-    if (use_graph() && !first_cycle()) {
+    if (use_graph() && !eager_cycle()) {
       graph_steps();
       graph_ran = true;
     } else {

@@ -752,7 +752,9 @@ inline void launch_sell(gs2_handle* h, const DevCsr& M, const VT* sv, const Epi&
   // to the width at which it is the faster one for the epilogue: for the FP64
   // residual 6 slots (its two more row operands and 7 slots need 56
   // registers, half the resident warps: 58 against 53 us on 7-point rows,
-  // n = 3.4M), for the whole-sweep residual 4.
+  // n = 3.4M), for the whole-sweep residual 4.  FP16 values (whose conversion
+  // and row scale cost it 46 registers) keep k_sell: inner sweep 19 against 23
+  // us at the same size.
   bool pair = false;
   auto fn = M.mean_row > kShortRowMean ? k_sell<VT, Epi, true, false> : k_sell<VT, Epi, false, false>;
   if constexpr (sizeof(VT) < sizeof(double)) {
@@ -762,7 +764,8 @@ inline void launch_sell(gs2_handle* h, const DevCsr& M, const VT* sv, const Epi&
     }
   }
   constexpr int WM = Epi::kUnroll;
-  if (M.sell_offset_chunks == M.sell_chunks && M.sell_wmax <= WM) {
+  if (sizeof(VT) > sizeof(__half) && M.sell_offset_chunks == M.sell_chunks &&
+      M.sell_wmax <= WM) {
     pair = false;
     fn = M.sell_wmax <= 4 ? k_stencil<VT, Epi, 4> : k_stencil<VT, Epi, WM>;
   }
