@@ -187,7 +187,8 @@ gs2_status gs2_autotune(gs2_handle* h);
  * rows fit its shared memory, else as one cooperative launch whose blocks
  * meet at bounded grid barriers (GMRES n <= 8,192, CG n <= 16,384) -- every restart cycle,
  * preconditioner application and Givens step included; otherwise as in
- * mode 1; 1 = each restart cycle's steps
+ * mode 1 from the fifth cycle of a shape on, as in mode 2 before (the same
+ * bits; capturing a graph costs more than it saves in a few cycles); 1 = each restart cycle's steps
  * as one replayed CUDA graph; 2 = as separate launches; 3 = the one-launch
  * solver, up to n = 65,536 (INVALID_ARG when the solve does not qualify);
  * 4 = the one-cluster solver: the whole GMRES solve inside one cluster of

@@ -591,8 +591,8 @@ struct GmresRun {
     }
   }
 
-  // Graphs by default at every size: even at n = 2.1M the launch gaps of
-  // separate launches cost ~6% of a solve.
+  // Graphs at every size (eager_cycle says from when): even at n = 2.1M the
+  // launch gaps of separate launches cost ~6% of a solve.
   bool use_graph() const { return h->graph_mode != 2; }
 
   // The m steps as one CUDA graph: captured once per cycle shape on the
