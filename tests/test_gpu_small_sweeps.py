@@ -1,0 +1,36 @@
+"""Sweeps without an inner sweep in the one-launch form: a half sweep's residual reads other rows'
+x right before the update writes it, with no inner sweep's barrier between them.
+
+The row kernels (which a profiled handle takes) separate the two by a launch, and reduce a row in
+the same order: the results are equal bit for bit, in every repetition.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2104_01196_gb300 import problems as P
+from test_gpu_parity import dev, g, host, rel, rhs_and_x0  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+# one CTA, a cluster of full warps, one whose last CTA is short, and the largest (16 x 512 rows)
+@pytest.mark.parametrize("name", ["poisson2d_8", "poisson2d_64", "poisson2d_61", "poisson3d_20"])
+@pytest.mark.parametrize("direction", [0, 1, 2])
+@pytest.mark.parametrize("omega", [1.0])
+def test_no_inner_sweep(g, name, direction, omega):  # noqa: F811
+    kind, size = name.split("_")
+    A = getattr(P, kind + "_matrix")(int(size))
+    b, x0 = rhs_and_x0(A, 81)
+    h = g.gs2_setup(A)
+    pc = g.params("gs2", outer=6, inner=0, omega=omega, direction=direction)
+    h.profile(True)
+    x = dev(x0)
+    g.gs2_apply_ex(h, dev(b), x, pc)
+    rows = host(x)
+    h.profile(False)
+    assert rel(rows, oracle.gs2(A, b, x0, 6, 0, omega, 1.0, direction)) <= 1e-12
+    for _ in range(50):
+        x = dev(x0)
+        g.gs2_apply_ex(h, dev(b), x, pc)
+        assert np.array_equal(host(x), rows)
