@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small_sweeps(SmallArgs a) {
       // every read of the old x ends before the first write of the new one: the
       // barriers of the inner sweeps lie between them, else one of its own
       if (a.inner == 0) sm_barrier();
-      x = unit ? x + g : x + a.omega * g;
+      x = fma(a.omega, g, x);
       if (own) vec[0][t] = x;
     }
   }

@@ -17,7 +17,7 @@ pytestmark = pytest.mark.gpu
 # one CTA, a cluster of full warps, one whose last CTA is short, and the largest (16 x 512 rows)
 @pytest.mark.parametrize("name", ["poisson2d_8", "poisson2d_64", "poisson2d_61", "poisson3d_20"])
 @pytest.mark.parametrize("direction", [0, 1, 2])
-@pytest.mark.parametrize("omega", [1.0])
+@pytest.mark.parametrize("omega", [1.0, 0.8])
 def test_no_inner_sweep(g, name, direction, omega):  # noqa: F811
     kind, size = name.split("_")
     A = getattr(P, kind + "_matrix")(int(size))
