@@ -132,6 +132,7 @@ struct KrylovState {
   double hn;       // last H(j+1, j)
   double inv_hn;
   double rz[2];    // CG: r.z before and after an iteration, by its parity
+  int arrived;     // CG: blocks of k_cg_xr that are done (0 between launches)
 };
 
 struct Profiler;

@@ -255,6 +255,7 @@ __global__ void k_state_init(KrylovState* st, double tol, int max_iters) {
   st->stop = 0;
   st->status = GS2_OK;
   st->k = 0;
+  st->arrived = 0;
   st->iters = 0;
   st->max_iters = max_iters;
   st->tol_abs = tol * st->bnorm;
@@ -944,8 +945,8 @@ gs2_status gmres_batch(gs2_handle* const* hs, const double* const* bs, double* c
 // An iteration is the row kernels of A p and of the preconditioner and four
 // vector kernels.  The scalars have no kernels of their own: each block of the
 // kernel that needs one sums the partials of the kernel before (sum_partials),
-// alpha in k_cg_xr, beta and the stopping test in k_cg_p.  The residual test
-// comes after the preconditioner, whose last application is then not used.
+// alpha in k_cg_xr, beta in k_cg_p; the stopping test runs in the last block of
+// k_cg_xr to finish, so that the preconditioner is not applied once it stops.
 
 // r.z of a (re)started search direction
 __global__ void k_cg_start(const double* __restrict__ part, int nblk, KrylovState* st) {
@@ -955,8 +956,12 @@ __global__ void k_cg_start(const double* __restrict__ part, int nblk, KrylovStat
 }
 
 // alpha = r.z / p.q from the partials of p.q (breakdown if that is 0);
-// x += alpha p ; r -= alpha q ; partials of r.r ; and the preconditioner's
-// D^{-1} r in its sweep precision (whichever of rhat64, rhat32 is non-null)
+// x += alpha p ; r -= alpha q ; partials of r.r ; the preconditioner's D^{-1} r
+// in its sweep precision (whichever of rhat64, rhat32 is non-null); and the
+// ||r|| test of the iteration.
+// The stop flag is set when every block has arrived: each thread of a block
+// reads it by itself, before barriers that all of the block's threads must
+// reach, so it must not change while a block may still start.
 __global__ void __launch_bounds__(kSumThreads, 2)
 k_cg_xr(int n, double* __restrict__ x, double* __restrict__ r, const double* __restrict__ p,
         const double* __restrict__ q, const double* __restrict__ part_pq, double* part_rr,
@@ -966,55 +971,59 @@ k_cg_xr(int n, double* __restrict__ x, double* __restrict__ r, const double* __r
   pdl_wait();
   if (skip && *skip) return;
   const double pq = sum_partials(part_pq, nblk);
-  if (pq == 0.0) {
-    // (every block sees it, or the flag)
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-      st->status = GS2_ERR_BREAKDOWN;
-      st->stop = 1;
-      *stop_host = 1;
-    }
-    return;
-  }
-  const double a = st->rz[parity] / pq;
+  const bool broken = pq == 0.0;  // (the same in every block)
   double s = 0.0;
+  if (!broken) {
+    const double a = st->rz[parity] / pq;
 #pragma unroll 2
-  for (int i = blockIdx.x * kSumThreads + threadIdx.x; i < n; i += gridDim.x * kSumThreads) {
-    x[i] = fma(a, p[i], x[i]);
-    const double ri = fma(-a, q[i], r[i]);
-    r[i] = ri;
-    s = fma(ri, ri, s);
-    if (rhat64) rhat64[i] = dinv[i] * ri;
-    if (rhat32) rhat32[i] = (float)(dinv[i] * ri);
+    for (int i = blockIdx.x * kSumThreads + threadIdx.x; i < n; i += gridDim.x * kSumThreads) {
+      x[i] = fma(a, p[i], x[i]);
+      const double ri = fma(-a, q[i], r[i]);
+      r[i] = ri;
+      s = fma(ri, ri, s);
+      if (rhat64) rhat64[i] = dinv[i] * ri;
+      if (rhat32) rhat32[i] = (float)(dinv[i] * ri);
+    }
   }
   s = block_total<kSumThreads>(s);
-  if (threadIdx.x == 0) part_rr[blockIdx.x] = s;
+  __shared__ bool last;
+  if (threadIdx.x == 0) {
+    part_rr[blockIdx.x] = s;
+    __threadfence();
+    last = atomicAdd(&st->arrived, 1) == (int)gridDim.x - 1;
+    __threadfence();
+  }
+  __syncthreads();
+  if (!last) return;
+  const double rn = sqrt(sum_partials(part_rr, nblk));
+  if (threadIdx.x != 0) return;
+  st->arrived = 0;
+  if (broken) {
+    st->status = GS2_ERR_BREAKDOWN;
+    st->stop = 1;
+  } else {
+    st->iters += 1;
+    st->beta = rn;
+    if (isnan(rn) || isinf(rn)) {
+      st->status = GS2_ERR_NAN;
+      st->stop = 1;
+    } else if (rn <= st->tol_abs || st->iters >= st->max_iters) {
+      st->stop = 1;
+    }
+  }
+  if (st->stop) *stop_host = 1;
 }
 
-// beta = r.z / (r.z before) ; p = z + beta p ; the ||r|| test of the iteration
-// (block 0; p is not used again once it stops the loop of launches)
+// beta = r.z / (r.z before) ; p = z + beta p
 __global__ void __launch_bounds__(kSumThreads, 2)
 k_cg_p(int n, double* __restrict__ p, const double* __restrict__ z,
-       const double* __restrict__ part_rr, const double* __restrict__ part_rz, int nblk,
-       KrylovState* st, int parity, volatile int* stop_host, const int* skip) {
+       const double* __restrict__ part_rz, int nblk, KrylovState* st, int parity,
+       const int* skip) {
   pdl_wait();
   if (skip && *skip) return;
   const double rz = sum_partials(part_rz, nblk);
   const double bt = rz / st->rz[parity];
-  if (blockIdx.x == 0) {
-    const double rn = sqrt(sum_partials(part_rr, nblk));
-    if (threadIdx.x == 0) {
-      st->rz[parity ^ 1] = rz;
-      st->iters += 1;
-      st->beta = rn;
-      if (isnan(rn) || isinf(rn)) {
-        st->status = GS2_ERR_NAN;
-        st->stop = 1;
-      } else if (rn <= st->tol_abs || st->iters >= st->max_iters) {
-        st->stop = 1;
-      }
-      if (st->stop) *stop_host = 1;
-    }
-  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) st->rz[parity ^ 1] = rz;
 #pragma unroll 4
   for (int i = blockIdx.x * kSumThreads + threadIdx.x; i < n; i += gridDim.x * kSumThreads)
     p[i] = fma(bt, p[i], z[i]);
@@ -1088,8 +1097,7 @@ gs2_status cg_run(gs2_handle* h, const double* b, double* x, double tol, int max
                part_rz, skip);
     GS2_LAUNCH_CHECK();
     launch_pdl(k_cg_p, nb, kSumThreads, 0, h->stream, n, pv, (const double*)z,
-               (const double*)part_rr, (const double*)part_rz, nb, h->st, it & 1,
-               (volatile int*)h->stop_mapped_dev, skip);
+               (const double*)part_rz, nb, h->st, it & 1, skip);
     GS2_LAUNCH_CHECK();
   };
   constexpr int kCheckEvery = 16;

@@ -18,14 +18,24 @@ __device__ __forceinline__ double warp_sum(double s) {
 // sums them gets the same bits.  (Two blocks per SM that sum 304 partials out
 // of L2 spend about 1 us at their start; a kernel of its own between producer
 // and consumers costs 3 to 4.  Summed by all warps of eight blocks per SM the
-// FP64 adds alone took 5 us.)
-__device__ __forceinline__ double sum_partials(const double* __restrict__ part, int nblk) {
+// FP64 adds alone took 5 us.)  Read at L2: the partials may be those of other
+// blocks of the same launch.
+constexpr int kSumLoads = 10;  // 304 partials: one round trip to L2
+__device__ __forceinline__ double sum_partials(const double* part, int nblk) {
   __shared__ double total;
   __syncthreads();  // total may still be read from an earlier call
   if (threadIdx.x < 32) {
     double s = 0.0;
-#pragma unroll 4
-    for (int b = threadIdx.x; b < nblk; b += 32) s += part[b];
+    for (int b = 0; b < nblk; b += 32 * kSumLoads) {
+      double v[kSumLoads];
+#pragma unroll
+      for (int q = 0; q < kSumLoads; ++q) {
+        const int at = b + 32 * q + threadIdx.x;
+        v[q] = at < nblk ? __ldcg(part + at) : 0.0;
+      }
+#pragma unroll
+      for (int q = 0; q < kSumLoads; ++q) s += v[q];
+    }
     s = warp_sum(s);
     if (threadIdx.x == 0) total = s;
   }
