@@ -339,11 +339,17 @@ static void free_hierarchy(AmgHierarchy* H, gs2_handle* h) {
 void amg_free(gs2_handle* h) {
   if (!h->amg) return;
   if (h->stream) cudaStreamSynchronize(h->stream);
-  // a captured cycle may hold the hierarchy's buffers
+  // captured GMRES cycles and CG iterations may hold the hierarchy's buffers (a
+  // new one may lie at the old one's address, so that no key tells them apart)
   if (h->gexec) {
     cudaGraphExecDestroy(h->gexec);
     h->gexec = nullptr;
     h->gkey.clear();
+  }
+  if (h->cg_gexec) {
+    cudaGraphExecDestroy(h->cg_gexec);
+    h->cg_gexec = nullptr;
+    h->cg_gkey.clear();
   }
   free_hierarchy(h->amg, h);
   h->amg = nullptr;
