@@ -455,8 +455,10 @@ gs2_status gs2_check(gs2_handle* h);
  * small system sums its inner products in another order); with
  * pack_rows set, a packed request's result is the same, bit for bit, as that
  * request solved alone as a pack of one (a pack partitions each system by
- * its own size), and equal to gmres_solve's up to the rounding of the inner
- * products. */
+ * its own size, and sums a row in 1, 2, 4, 8 or 16 parts by the pack's mean
+ * row length -- up to 24, 48, 96, 192 entries or more -- so its systems must
+ * share one of these classes, as every stencil does), and equal to
+ * gmres_solve's up to the rounding of the inner products. */
 typedef struct gs2_server gs2_server;
 
 typedef struct {

@@ -422,7 +422,9 @@ static void upload_sell(gs2_handle* h, DevCsr& M, const std::vector<int>& rp, co
   int longest = 0;
   for (int i = 0; i < n; ++i) longest = std::max(longest, rp[i + 1] - rp[i]);
   const bool short_rows = M.mean_row <= kShortRowMean;
-  const bool streams = 12.0 * M.nnz >= kSellStreamBytes;
+  // (a pack's long rows keep the lanes of their length whatever its size, so that
+  // a system's result does not depend on the others)
+  const bool streams = !h->for_pack && 12.0 * M.nnz >= kSellStreamBytes;
   LaneLayout lanes;
   auto try_lanes = [&](int K) {
     M.sell_lanes = longest <= kLaneMaxSlots * K && lane_layout(rp, n, K, lanes) ? K : 0;
