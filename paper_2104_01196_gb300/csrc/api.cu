@@ -270,13 +270,15 @@ constexpr double kSellMaxPadding = 1.2;          // slots / entries
 constexpr int kSellSmall = 1 << 18;  // entries up to which lane slices may pad to double
 constexpr double kSellStreamBytes = 128.0 * (1 << 20);  // CSR bytes beyond L2
 
-// (With `origin`, offsets are j - origin[i]: a colour's rows, origin[i] their row
-// in A.)  Chunk layout: chunk c takes width_c x 32 slots, width_c its longest row
+// Chunk layout: chunk c takes width_c x 32 slots, width_c its longest row
 // (explicit columns) or, for an offset chunk, the number of distinct column
 // offsets j - i over its rows.  A chunk is an offset chunk when that union is
 // at most its longest row + kOffsetSlack and at most 32 (stencil rows: the
 // rows at a grid boundary miss some offsets and get zero slots there).
-// Consecutive chunks with the same offset list share one copy.  Returns
+// Consecutive chunks with the same offset list share one copy.  With `origin`
+// (a colour's rows, origin[i] their row in A) offsets are j - origin[i], and a
+// chunk that stores a zero keeps its columns: the kernel tells an empty slot by
+// its zero value, and a stored zero times an infinity or NaN is a NaN.  Returns
 // false when the layout pads too much or its slots would not fit 32-bit
 // offsets.
 constexpr int kOffsetSlack = 2;
@@ -287,8 +289,8 @@ struct SellLayout {
   int offset_chunks = 0, wmax = 0;
 };
 
-static bool sell_layout(const std::vector<int>& rp, const int* ci, int n, const int* origin,
-                        SellLayout& out) {
+static bool sell_layout(const std::vector<int>& rp, const int* ci, const double* va, int n,
+                        const int* origin, SellLayout& out) {
   const int nc = (n + kSellC - 1) / kSellC;
   out.cptr.assign(nc + 1, 0);
   out.coff.assign(nc, -1);
@@ -305,6 +307,7 @@ static bool sell_layout(const std::vector<int>& rp, const int* ci, int n, const 
       L = std::max(L, rp[i + 1] - rp[i]);
       const int at = origin ? origin[i] : i;
       for (int k = rp[i]; regular && k < rp[i + 1]; ++k) {
+        if (origin && va[k] == 0.0) regular = false;
         const int o = ci[k] - at;
         if (std::find(u.begin(), u.end(), o) == u.end()) {
           u.push_back(o);
@@ -415,7 +418,7 @@ static bool lane_layout(const std::vector<int>& rp, int n, int K, LaneLayout& ou
 // there (launch_to_sell, launch_to_lanes); only the chunk layout is computed
 // here.
 static void upload_sell(gs2_handle* h, DevCsr& M, const std::vector<int>& rp, const int* ci,
-                        const int* origin) {
+                        const double* va, const int* origin) {
   const int n = M.n;
   if (n == 0 || M.nnz == 0) return;
   SellLayout lay;
@@ -436,7 +439,7 @@ static void upload_sell(gs2_handle* h, DevCsr& M, const std::vector<int>& rp, co
   // 3% lost on 64^3)
   const bool few = &M == &h->A && !short_rows && streams &&
                    n < 2 * 32 * (int64_t)kSellWarpsPerSm * h->nsm && try_lanes(1);
-  bool sliced = !few && (short_rows || streams) && sell_layout(rp, ci, n, origin, lay);
+  bool sliced = !few && (short_rows || streams) && sell_layout(rp, ci, va, n, origin, lay);
   // short rows with explicit columns, too few for the SMs' warps at one lane
   // each (the 64,560 rows of a second multigrid level, 15 entries in a
   // triangle: inner sweep 12.6 -> 8.6 us with two lanes); long rows here
@@ -509,7 +512,7 @@ static void upload_csr(gs2_handle* h, DevCsr& M, int n, const std::vector<int>& 
   h->h2d(M.ci, ci, sizeof(int) * M.nnz);
   h->h2d(M.va, va, sizeof(double) * M.nnz);
   retile(h, M, rp, M.tpr, 1);
-  upload_sell(h, M, rp, ci, origin);
+  upload_sell(h, M, rp, ci, va, origin);
 }
 
 // (Re)build the row tiles of M for K lanes per row and RPT rows per lane
