@@ -25,19 +25,22 @@ namespace gs2 {
 
 // ---------------------------------------------------------------------------
 // epilogues: pre(i) loads the row's operands before the gathers, finish(i,
-// s, pre) consumes the row sum.  The FP64 pipe (2 FMA/clk/SM) bounds the FP64
-// row kernels, so an epilogue that only subtracts the row sum from an operand
-// lets the products do it (kSub): the sum starts at that operand and
-// subtracts each product, one FP64 operation a row fewer (a 7-point residual
-// has 8 instead of 9, an undamped inner sweep of a 3-entry triangle 3 or 4
-// instead of 5; a few more roundings of the operand's size: sweeps are 2e-16 from
-// the 64-bit result where they were 1.6e-16).  kUnroll: the widest stencil row that takes the unrolled form
-// (k_stencil).  origin(i, pre): the row that row i's offsets count from.
+// s, pre) consumes the row sum.  kUnroll: the widest stencil row that takes the
+// unrolled form (k_stencil).  origin(i, pre): the row that row i's offsets
+// count from.
+//
+// A row's sum starts at zero and meets its operand (b, rhat, y) once, at the
+// end.  Starting it at the operand would save one of the 5 to 9 operations a
+// row spends on the FP64 pipe (2 FMA/clk/SM), which bounds these kernels
+// (symmetric sweep on the 150^3 convection-diffusion matrix 161 instead of 192
+// us), but rounds every product at the operand's size: over stencils, Q1
+// elasticity and uneven rows the distance from the exact sweep grew by 7% to
+// 65% (multicolour GS 0.93e-16 -> 1.43e-16, a forward sweep with two inner
+// ones 1.15e-16 -> 1.89e-16).
 // ---------------------------------------------------------------------------
 
 // r = b - A x;  rhat = D^{-1} r   (Eq. 2 residual and Eq. 3 initial guess)
 struct EpiResid {
-  static constexpr bool kSub = true;
   static constexpr int kUnroll = 6;
   static constexpr bool kGuard = false;
   const double* __restrict__ x;
@@ -52,8 +55,8 @@ struct EpiResid {
   __device__ int origin(int i, const Pre&) const { return i; }
   __device__ Pre pre(int i) const { return Pre{b[i], dinv[i]}; }
   __device__ double gather(int c) const { return __ldg(x + c); }
-  __device__ double begin(const Pre& p) const { return p.b; }
-  __device__ void finish(int i, double ri, const Pre& p) const {
+  __device__ void finish(int i, double s, const Pre& p) const {
+    const double ri = p.b - s;
     const double rh = p.d * ri;
     if (r) r[i] = ri;
     if (rhat64) rhat64[i] = rh;
@@ -62,7 +65,6 @@ struct EpiResid {
 };
 
 struct EpiSpmv {
-  static constexpr bool kSub = false;
   static constexpr int kUnroll = 8;
   static constexpr bool kGuard = false;
   const double* __restrict__ x;
@@ -71,14 +73,12 @@ struct EpiSpmv {
   __device__ int origin(int i, const Pre&) const { return i; }
   __device__ Pre pre(int) const { return Pre{}; }
   __device__ double gather(int c) const { return __ldg(x + c); }
-  __device__ double begin(const Pre&) const { return 0.0; }
   __device__ void finish(int i, double s, const Pre&) const { y[i] = s; }
 };
 
 // y = M x and rhat = D^{-1} y with another matrix's diagonal (multigrid
 // restriction: the coarse level's smoother starts from D^{-1} b_c)
 struct EpiRestrict {
-  static constexpr bool kSub = false;
   static constexpr int kUnroll = 8;
   static constexpr bool kGuard = false;
   const double* __restrict__ x;
@@ -92,7 +92,6 @@ struct EpiRestrict {
   __device__ int origin(int i, const Pre&) const { return i; }
   __device__ Pre pre(int i) const { return Pre{dinv[i]}; }
   __device__ double gather(int c) const { return __ldg(x + c); }
-  __device__ double begin(const Pre&) const { return 0.0; }
   __device__ void finish(int i, double s, const Pre& p) const {
     y[i] = s;
     if (rhat64) rhat64[i] = p.d * s;
@@ -102,7 +101,6 @@ struct EpiRestrict {
 
 // y += M x (multigrid prolongation)
 struct EpiSpmvAdd {
-  static constexpr bool kSub = false;
   static constexpr int kUnroll = 8;
   static constexpr bool kGuard = false;
   const double* __restrict__ x;
@@ -113,13 +111,11 @@ struct EpiSpmvAdd {
   __device__ int origin(int i, const Pre&) const { return i; }
   __device__ Pre pre(int i) const { return Pre{y[i]}; }
   __device__ double gather(int c) const { return __ldg(x + c); }
-  __device__ double begin(const Pre& p) const { return p.y; }
-  __device__ void finish(int i, double s, const Pre&) const { y[i] = s; }
+  __device__ void finish(int i, double s, const Pre& p) const { y[i] = p.y + s; }
 };
 
 // x_out = x_in + omega D^{-1} (b - A x_in)   (damped JR, ping-pong buffers)
 struct EpiJr {
-  static constexpr bool kSub = true;
   static constexpr int kUnroll = 8;
   static constexpr bool kGuard = false;
   const double* __restrict__ x;
@@ -133,9 +129,8 @@ struct EpiJr {
   __device__ int origin(int i, const Pre&) const { return i; }
   __device__ Pre pre(int i) const { return Pre{x[i], b[i], dinv[i]}; }
   __device__ double gather(int c) const { return __ldg(x + c); }
-  __device__ double begin(const Pre& p) const { return p.b; }
-  __device__ void finish(int i, double r, const Pre& p) const {
-    x_out[i] = p.x + omega * (p.d * r);
+  __device__ void finish(int i, double s, const Pre& p) const {
+    x_out[i] = p.x + omega * (p.d * (p.b - s));
   }
 };
 
@@ -144,14 +139,11 @@ struct EpiJr {
 // The form and SCALED (FP16 triangles with a per-row scale) are compile-time:
 // a runtime flag on a uniform kernel argument is predicated, and its FP64
 // instructions would then issue on every row.  UNIT (FP64, omega = gamma = 1,
-// Eq. (4)-(5) as printed): g' is the row sum itself and the update adds or
-// stores it, without the products by omega.  The lower precisions keep the
-// general form, so that their rounding does not depend on omega.
+// Eq. (4)-(5) as printed): without the products by omega, the same bits.
 enum InnerForm { INNER_PLAIN, INNER_DAMPED, INNER_UNIT };
 
 template <typename GT, typename AT, InnerForm FORM, bool SCALED>
 struct EpiInner {
-  static constexpr bool kSub = FORM == INNER_UNIT;
   static constexpr int kUnroll = 8;
   static constexpr bool kGuard = false;
   const GT* __restrict__ g_in;
@@ -179,13 +171,13 @@ struct EpiInner {
     return p;
   }
   __device__ AT gather(int c) const { return (AT)__ldg(g_in + c); }
-  __device__ AT begin(const Pre& p) const { return FORM == INNER_UNIT ? p.rh : AT(0); }
   __device__ void finish(int i, AT s, const Pre& p) const {
     if (FORM == INNER_UNIT) {
+      const AT go = p.rh - s;
       if (mode == INNER_MID) {
-        g_out[i] = (GT)s;
+        g_out[i] = (GT)go;
       } else {
-        double v = (double)s;
+        double v = (double)go;
         if (mode == INNER_LAST_ADD) v += p.xi;
         x[i] = v;
       }
@@ -215,7 +207,6 @@ struct EpiInner {
 //   rhat32 = (fl32(D^{-1} b) - x32) - O x32
 template <bool SCALED>
 struct EpiResidSweep {
-  static constexpr bool kSub = false;
   static constexpr int kUnroll = 4;
   static constexpr bool kGuard = false;
   const float* __restrict__ bhat;
@@ -233,7 +224,6 @@ struct EpiResidSweep {
     return p;
   }
   __device__ float gather(int c) const { return __ldg(x32 + c); }
-  __device__ float begin(const Pre&) const { return 0.f; }
   __device__ void finish(int i, float s, const Pre& p) const {
     if (SCALED) s *= p.sc;
     rhat32[i] = p.bx - s;
@@ -243,7 +233,6 @@ struct EpiResidSweep {
 // compact right-hand side of Eq. (9) on the other prescaled triangle
 // T' = D^{-1} U (forward) or D^{-1} L (backward):  rhat = D^{-1} b - T' x
 struct EpiCompact {
-  static constexpr bool kSub = true;
   static constexpr int kUnroll = 8;
   static constexpr bool kGuard = false;
   const double* __restrict__ x;
@@ -257,8 +246,8 @@ struct EpiCompact {
   __device__ int origin(int i, const Pre&) const { return i; }
   __device__ Pre pre(int i) const { return Pre{b[i], dinv[i]}; }
   __device__ double gather(int c) const { return __ldg(x + c); }
-  __device__ double begin(const Pre& p) const { return p.d * p.b; }
-  __device__ void finish(int i, double rh, const Pre&) const {
+  __device__ void finish(int i, double s, const Pre& p) const {
+    const double rh = p.d * p.b - s;
     if (rhat64) rhat64[i] = rh;
     if (rhat32) rhat32[i] = (float)rh;
   }
@@ -271,7 +260,6 @@ struct EpiCompact {
 //   x_r = (1 - omega) x_r + omega (bhat_r - sum_j (a_rj / a_rr) x_j)
 template <bool DAMPED>
 struct EpiColor {
-  static constexpr bool kSub = true;
   static constexpr int kUnroll = 8;
   static constexpr bool kGuard = true;
   const int* __restrict__ rows;
@@ -291,8 +279,8 @@ struct EpiColor {
     return p;
   }
   __device__ double gather(int c) const { return __ldg(x + c); }
-  __device__ double begin(const Pre& p) const { return p.bh; }
-  __device__ void finish(int, double gs, const Pre& p) const {
+  __device__ void finish(int, double s, const Pre& p) const {
+    const double gs = p.bh - s;
     x[p.r] = DAMPED ? p.xr + omega * (gs - p.xr) : gs;
   }
 };

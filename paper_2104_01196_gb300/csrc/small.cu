@@ -109,43 +109,38 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small_sweeps(SmallArgs a) {
   }
   // the warp's longest rows: slots beyond them issue nothing on the FP64 pipe
   const int wl = __reduce_max_sync(0xffffffffu, nl), wu = __reduce_max_sync(0xffffffffu, nu);
-  // s -+ sum of one side's values times vector v
+  // s + sum of one side's values times vector v
   auto side = [&](double s, const double (&val)[kSmSide], const unsigned (&adr)[kSmSide], int cnt,
-                  int most, int v, bool sub) {
+                  int most, int v) {
     double g[kSmSide];
 #pragma unroll
     for (int k = 0; k < kSmSide; ++k) g[k] = k < cnt ? sm_load(adr[k] + (unsigned)v * kStep) : 0.0;
 #pragma unroll
     for (int k = 0; k < kSmSide; ++k)
       if (k < most) {
-        if (k < cnt) s = fma(sub ? -val[k] : val[k], g[k], s);
+        if (k < cnt) s = fma(val[k], g[k], s);
       }
     return s;
   };
-  const bool unit = a.omega == 1.0 && a.gamma == 1.0, damped = a.gamma != 1.0;
+  const bool damped = a.gamma != 1.0;
   for (int s = 0; s < a.sweeps; ++s) {
     for (int half = 0; half < 2; ++half) {
       const bool fwd = half == 0;
       if (a.dir == (fwd ? GS2_BACKWARD : GS2_FORWARD)) continue;
       sm_barrier();  // x complete
       // rhat = D^{-1} (b - A x), the inner iterate g_0
-      double r = side(b, al, pl, nl, wl, 0, true);
-      r = fma(-ad, x, r);
-      r = side(r, au, pu, nu, wu, 0, true);
-      const double rh = d * r;
+      double r = side(0.0, al, pl, nl, wl, 0);
+      r = fma(ad, x, r);
+      r = side(r, au, pu, nu, wu, 0);
+      const double rh = d * (b - r);
       double g = rh;
       int cur = 1;
       for (int j = 0; j < a.inner; ++j) {
         if (own) vec[cur][t] = g;
         sm_barrier();  // g complete
-        if (unit) {
-          g = fwd ? side(rh, tl, pl, nl, wl, cur, true) : side(rh, tu, pu, nu, wu, cur, true);
-        } else {
-          const double sum = fwd ? side(0.0, tl, pl, nl, wl, cur, false)
-                                 : side(0.0, tu, pu, nu, wu, cur, false);
-          const double go = rh - a.omega * sum;
-          g = damped ? (1.0 - a.gamma) * g + a.gamma * go : go;
-        }
+        const double sum = fwd ? side(0.0, tl, pl, nl, wl, cur) : side(0.0, tu, pu, nu, wu, cur);
+        const double go = rh - a.omega * sum;
+        g = damped ? (1.0 - a.gamma) * g + a.gamma * go : go;
         cur ^= 3;
       }
       // every read of the old x ends before the first write of the new one: the

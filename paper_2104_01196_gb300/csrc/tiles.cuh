@@ -61,13 +61,6 @@ struct ValTraits<__half> {
   __device__ static float get(const __half* p, int k) { return __half2float(p[k]); }
 };
 
-// An epilogue's row sum: begin(pre) + sum_k a_k x_k, or with Epi::kSub
-// begin(pre) - sum_k a_k x_k (begin = 0 for a plain sum).
-template <class Epi, typename AT>
-__device__ __forceinline__ AT row_fma(AT a, AT x, AT s) {
-  return fma(Epi::kSub ? -a : a, x, s);
-}
-
 // The gathered x of an offset chunk's slot, or with Epi::kGuard 0 in a slot of
 // value 0: an infinity or NaN at a column that the row does not have cannot
 // reach it.  (+0.0 by its bits: a comparison would issue on the FP64 pipe.)
@@ -173,8 +166,8 @@ struct StageLayout {
   }
 };
 
-// Engine: for every row i, acc_i = begin +- sum_k va[k] * epi.gather(ci[k]),
-// then epi.finish(i, acc_i).  Double-buffered: while the block reduces tile t
+// Engine: for every row i, acc_i = sum_k va[k] * epi.gather(ci[k]), then
+// epi.finish(i, acc_i).  Double-buffered: while the block reduces tile t
 // from one shared-memory stage, one thread has TMA fill the other stage
 // with tile t + grid (its rowptr slice, columns and values), completion
 // tracked by one mbarrier per stage.  Rows are reduced by one thread each
@@ -252,9 +245,9 @@ k_tiles(TileMat<VT> M, Epi epi, const int* skip) {
       // one long row: whole block, straight from global memory
       const int a = -1 - d.z;
       const typename Epi::Pre pv = epi.pre(d.x);
-      AT s = threadIdx.x == 0 ? epi.begin(pv) : AT(0);
+      AT s = AT(0);
       for (int k = a + threadIdx.x; k < d.w; k += blockDim.x)
-        s = row_fma<Epi>((AT)ValTraits<VT>::get(M.va, k), (AT)epi.gather(M.ci[k]), s);
+        s = fma((AT)ValTraits<VT>::get(M.va, k), (AT)epi.gather(M.ci[k]), s);
       s = block_sum<AT>(s, red);
       if (threadIdx.x == 0) epi.finish(d.x, s, pv);
       __syncthreads();
@@ -272,7 +265,6 @@ k_tiles(TileMat<VT> M, Epi epi, const int* skip) {
       typename Epi::Pre pv{};
       if (row < d.y) {
         pv = epi.pre(row);
-        if (l == 0) s = epi.begin(pv);
         const int rs = s_rp[row - rpb] - d.z, re = s_rp[row + 1 - rpb] - d.z;
         int ks = rs, ke = re;
         if (K > 1) {
@@ -285,19 +277,19 @@ k_tiles(TileMat<VT> M, Epi epi, const int* skip) {
         for (; k + 4 <= ke; k += 4) {
           const AT x0 = (AT)epi.gather(s_ci[k]), x1 = (AT)epi.gather(s_ci[k + 1]);
           const AT x2 = (AT)epi.gather(s_ci[k + 2]), x3 = (AT)epi.gather(s_ci[k + 3]);
-          s = row_fma<Epi>((AT)ValTraits<VT>::get(s_va, k), x0, s);
-          s = row_fma<Epi>((AT)ValTraits<VT>::get(s_va, k + 1), x1, s);
-          s = row_fma<Epi>((AT)ValTraits<VT>::get(s_va, k + 2), x2, s);
-          s = row_fma<Epi>((AT)ValTraits<VT>::get(s_va, k + 3), x3, s);
+          s = fma((AT)ValTraits<VT>::get(s_va, k), x0, s);
+          s = fma((AT)ValTraits<VT>::get(s_va, k + 1), x1, s);
+          s = fma((AT)ValTraits<VT>::get(s_va, k + 2), x2, s);
+          s = fma((AT)ValTraits<VT>::get(s_va, k + 3), x3, s);
         }
         const int rem = ke - k;
         if (rem > 0) {
           const AT x0 = (AT)epi.gather(s_ci[k]);
           const AT x1 = rem > 1 ? (AT)epi.gather(s_ci[k + 1]) : AT(0);
           const AT x2 = rem > 2 ? (AT)epi.gather(s_ci[k + 2]) : AT(0);
-          s = row_fma<Epi>((AT)ValTraits<VT>::get(s_va, k), x0, s);
-          if (rem > 1) s = row_fma<Epi>((AT)ValTraits<VT>::get(s_va, k + 1), x1, s);
-          if (rem > 2) s = row_fma<Epi>((AT)ValTraits<VT>::get(s_va, k + 2), x2, s);
+          s = fma((AT)ValTraits<VT>::get(s_va, k), x0, s);
+          if (rem > 1) s = fma((AT)ValTraits<VT>::get(s_va, k + 1), x1, s);
+          if (rem > 2) s = fma((AT)ValTraits<VT>::get(s_va, k + 2), x2, s);
         }
       }
       if (K > 1) s = group_sum<K, AT>(s);
@@ -368,7 +360,7 @@ __device__ __forceinline__ bool sell_pair(int n, int c, const int* __restrict__ 
   const VT* v1 = va + b1 + lane;
   const int* o0 = offs + ob0;
   const int* o1 = offs + ob1;
-  AT s0 = epi.begin(p0), s1 = epi.begin(p1);
+  AT s0 = AT(0), s1 = AT(0);
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     if (k < L) {
@@ -376,8 +368,8 @@ __device__ __forceinline__ bool sell_pair(int n, int c, const int* __restrict__ 
       const int cb = min(max(epi.origin(r1, p1) + __ldg(o1 + k), 0), cmax);
       const AT a = stream_val<VT>(v0 + 32 * k), b = stream_val<VT>(v1 + 32 * k);
       const AT xa = (AT)epi.gather(ca), xb = (AT)epi.gather(cb);
-      s0 = row_fma<Epi>(a, xa, s0);
-      s1 = row_fma<Epi>(b, xb, s1);
+      s0 = fma(a, xa, s0);
+      s1 = fma(b, xb, s1);
     }
   }
   if (r0 < n) epi.finish(r0, s0, p0);
@@ -410,7 +402,7 @@ k_sell(int n, int nchunks, const int* __restrict__ cptr, const int* __restrict__
     typename Epi::Pre pv{};
     if (row < n) pv = epi.pre(row);
     const VT* vv = va + base + lane;
-    AT s = epi.begin(pv);
+    AT s = AT(0);
     int k = 0;
     const int ob = __ldg(coff + c);
     if (ob >= 0) {
@@ -427,10 +419,10 @@ k_sell(int n, int nchunks, const int* __restrict__ cptr, const int* __restrict__
         const AT a2 = stream_val<VT>(vv + 64), a3 = stream_val<VT>(vv + 96);
         const AT x0 = (AT)epi.gather(c0), x1 = (AT)epi.gather(c1);
         const AT x2 = (AT)epi.gather(c2), x3 = (AT)epi.gather(c3);
-        s = row_fma<Epi>(a0, guarded<Epi>(a0, x0), s);
-        s = row_fma<Epi>(a1, guarded<Epi>(a1, x1), s);
-        s = row_fma<Epi>(a2, guarded<Epi>(a2, x2), s);
-        s = row_fma<Epi>(a3, guarded<Epi>(a3, x3), s);
+        s = fma(a0, guarded<Epi>(a0, x0), s);
+        s = fma(a1, guarded<Epi>(a1, x1), s);
+        s = fma(a2, guarded<Epi>(a2, x2), s);
+        s = fma(a3, guarded<Epi>(a3, x3), s);
       }
       const int rem = L - k;
       if (rem > 0) {
@@ -443,9 +435,9 @@ k_sell(int n, int nchunks, const int* __restrict__ cptr, const int* __restrict__
         const AT x0 = (AT)epi.gather(c0);
         const AT x1 = rem > 1 ? (AT)epi.gather(c1) : AT(0);
         const AT x2 = rem > 2 ? (AT)epi.gather(c2) : AT(0);
-        s = row_fma<Epi>(a0, guarded<Epi>(a0, x0), s);
-        if (rem > 1) s = row_fma<Epi>(a1, guarded<Epi>(a1, x1), s);
-        if (rem > 2) s = row_fma<Epi>(a2, guarded<Epi>(a2, x2), s);
+        s = fma(a0, guarded<Epi>(a0, x0), s);
+        if (rem > 1) s = fma(a1, guarded<Epi>(a1, x1), s);
+        if (rem > 2) s = fma(a2, guarded<Epi>(a2, x2), s);
       }
       if (row < n) epi.finish(row, s, pv);
       continue;
@@ -463,20 +455,20 @@ k_sell(int n, int nchunks, const int* __restrict__ cptr, const int* __restrict__
         const int n0 = __ldcs(cc), n1 = __ldcs(cc + 32), n2 = __ldcs(cc + 64), n3 = __ldcs(cc + 96);
         const AT b0 = stream_val<VT>(vv), b1 = stream_val<VT>(vv + 32);
         const AT b2 = stream_val<VT>(vv + 64), b3 = stream_val<VT>(vv + 96);
-        s = row_fma<Epi>(a0, x0, s);
-        s = row_fma<Epi>(a1, x1, s);
-        s = row_fma<Epi>(a2, x2, s);
-        s = row_fma<Epi>(a3, x3, s);
+        s = fma(a0, x0, s);
+        s = fma(a1, x1, s);
+        s = fma(a2, x2, s);
+        s = fma(a3, x3, s);
         c0 = n0; c1 = n1; c2 = n2; c3 = n3;
         a0 = b0; a1 = b1; a2 = b2; a3 = b3;
       }
       // the last preloaded group
       const AT x0 = (AT)epi.gather(c0), x1 = (AT)epi.gather(c1);
       const AT x2 = (AT)epi.gather(c2), x3 = (AT)epi.gather(c3);
-      s = row_fma<Epi>(a0, x0, s);
-      s = row_fma<Epi>(a1, x1, s);
-      s = row_fma<Epi>(a2, x2, s);
-      s = row_fma<Epi>(a3, x3, s);
+      s = fma(a0, x0, s);
+      s = fma(a1, x1, s);
+      s = fma(a2, x2, s);
+      s = fma(a3, x3, s);
       k += 4;
       cc += 128;
       vv += 128;
@@ -488,10 +480,10 @@ k_sell(int n, int nchunks, const int* __restrict__ cptr, const int* __restrict__
       const AT a2 = stream_val<VT>(vv + 64), a3 = stream_val<VT>(vv + 96);
       const AT x0 = (AT)epi.gather(c0), x1 = (AT)epi.gather(c1);
       const AT x2 = (AT)epi.gather(c2), x3 = (AT)epi.gather(c3);
-      s = row_fma<Epi>(a0, x0, s);
-      s = row_fma<Epi>(a1, x1, s);
-      s = row_fma<Epi>(a2, x2, s);
-      s = row_fma<Epi>(a3, x3, s);
+      s = fma(a0, x0, s);
+      s = fma(a1, x1, s);
+      s = fma(a2, x2, s);
+      s = fma(a3, x3, s);
     }
     // the last one to three slots, also issued together
     const int rem = L - k;
@@ -505,9 +497,9 @@ k_sell(int n, int nchunks, const int* __restrict__ cptr, const int* __restrict__
       const AT x0 = (AT)epi.gather(c0);
       const AT x1 = rem > 1 ? (AT)epi.gather(c1) : AT(0);
       const AT x2 = rem > 2 ? (AT)epi.gather(c2) : AT(0);
-      s = row_fma<Epi>(a0, x0, s);
-      if (rem > 1) s = row_fma<Epi>(a1, x1, s);
-      if (rem > 2) s = row_fma<Epi>(a2, x2, s);
+      s = fma(a0, x0, s);
+      if (rem > 1) s = fma(a1, x1, s);
+      if (rem > 2) s = fma(a2, x2, s);
     }
     if (row < n) epi.finish(row, s, pv);
   }
@@ -532,7 +524,7 @@ __device__ __forceinline__ AT stencil_row(AT s, int at, const int* __restrict__ 
 #pragma unroll
   for (int k = 0; k < W; ++k) x[k] = (AT)epi.gather(c[k]);
 #pragma unroll
-  for (int k = 0; k < W; ++k) s = row_fma<Epi>(a[k], guarded<Epi>(a[k], x[k]), s);
+  for (int k = 0; k < W; ++k) s = fma(a[k], guarded<Epi>(a[k], x[k]), s);
   return s;
 }
 
@@ -606,8 +598,8 @@ k_stencil(int n, int nchunks, const int* __restrict__ cptr, const int* __restric
       if (row < n) pv = epi.pre(row);
       const int L = (end - base) >> 5;
       const VT* vv = va + base + lane;
-      auto s = epi.begin(pv);
-      s = stencil_rows<WM, VT>(s, L, epi.origin(row, pv), offs + ob, vv, epi, cmax);
+      using AT = typename ValTraits<VT>::AT;
+      const AT s = stencil_rows<WM, VT>(AT(0), L, epi.origin(row, pv), offs + ob, vv, epi, cmax);
       if (row < n) epi.finish(row, s, pv);
     }
     if (cn >= nchunks) return;
@@ -663,7 +655,7 @@ k_lanes(int n, int nchunks, const int* __restrict__ cptr, const int* __restrict_
   load(0);
   typename Epi::Pre pv{};
   if (own) pv = epi.pre(row);
-  AT s = l == 0 ? epi.begin(pv) : AT(0);
+  AT s = AT(0);
   for (int k = 0; k < L; k += 4) {
     const AT x0 = c0 >= 0 ? (AT)epi.gather(c0) : AT(0);
     const AT x1 = c1 >= 0 ? (AT)epi.gather(c1) : AT(0);
@@ -671,10 +663,10 @@ k_lanes(int n, int nchunks, const int* __restrict__ cptr, const int* __restrict_
     const AT x3 = c3 >= 0 ? (AT)epi.gather(c3) : AT(0);
     const AT b0 = a0, b1 = a1, b2 = a2, b3 = a3;
     load(k + 4);
-    s = row_fma<Epi>(b0, x0, s);
-    if (k + 1 < L) s = row_fma<Epi>(b1, x1, s);
-    if (k + 2 < L) s = row_fma<Epi>(b2, x2, s);
-    if (k + 3 < L) s = row_fma<Epi>(b3, x3, s);
+    s = fma(b0, x0, s);
+    if (k + 1 < L) s = fma(b1, x1, s);
+    if (k + 2 < L) s = fma(b2, x2, s);
+    if (k + 3 < L) s = fma(b3, x3, s);
   }
   if (K > 1) s = group_sum<K, AT>(s);
   if (own && l == 0) epi.finish(row, s, pv);
