@@ -351,6 +351,12 @@ constexpr int kSellWarpsPerSm = 32;  // resident warps of k_sell on long rows
 // a symmetric sweep 79 -> 70 us).  With more than 16 warps per SM further
 // lanes only add shuffles and FP64 adds (elasticity on 28^3 nodes: 58 us with
 // 4 lanes, 98 with 16).  A pack's lanes do not depend on its size.
+//
+// Where A has more lanes than its row tiles, a row's last entry is held back
+// until the lanes' parts are added up (sell_held): in rows that store the
+// diagonal last the parts are small, and their total meets it in one rounding.
+// Summed with the others in its lane it was rounded again as the parts came
+// together (uneven rows, distance from the exact sweep 17% to 20% larger).
 static int lane_count(const gs2_handle* h, int64_t n, double mean, int longest) {
   int K = choose_lanes(mean);
   if (h->for_pack) return K;
@@ -474,6 +480,7 @@ static void upload_sell(gs2_handle* h, DevCsr& M, const std::vector<int>& rp, co
   h->h2d(M.sell_ptr, cptr.data(), sizeof(int) * cptr.size());
   M.sell = true;
   if (!sliced) {
+    M.sell_held = M.diagonal && M.sell_lanes > choose_lanes(M.mean_row);
     GS2_CUDA(cudaMemsetAsync(M.sell_ci, 0xff, sizeof(int) * slots, h->stream));
     if (!lanes.row.empty()) {
       M.sell_row = (int*)h->dalloc(sizeof(int) * n);
@@ -909,6 +916,7 @@ Hybrid* ensure_hybrid(gs2_handle* h, const gs2_params* p) {
     y = new Hybrid();
     y->parts = P;
     h->hybrids.push_back(y);
+    y->Aloc.diagonal = true;
     upload_matrix(h, y->Aloc, n, lrp, lci, lva);
     upload_matrix(h, y->E, n, erp, eci, eva);
     upload_matrix(h, y->Lloc, n, tris.first.rp, tris.first.ci, tris.first.va);
@@ -1329,6 +1337,7 @@ gs2_handle* gs2::setup_handle(int64_t n, int64_t nnz, const int64_t* rowptr,
   h->parted = parted;
   h->n = n;
   h->nnz = nnz;
+  h->A.diagonal = true;
   upload_csr(h, h->A, (int)n, rp32, CI, VA, (int)nnz);
   hs->Arp = rp32;
   upload_csr(h, h->L, (int)n, L.rp, L.ci.data(), L.va.data(), (int)L.ci.size());

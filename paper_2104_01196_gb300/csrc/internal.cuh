@@ -114,7 +114,12 @@ struct DevCsr {
   // sell_ptr[c] + 32 k + lane; padding slots have column -1.  Rows of uneven
   // length are sorted by it inside windows: sell_row[p] is the row at place p
   // (null: in order).
+  // sell_held (more lanes than the row tiles, `diagonal`): the row's last entry
+  // is in the chunk's last slot of its first lane, the lanes' parts hold the
+  // others.
+  bool diagonal = false;  // the rows hold their diagonal entries (set before the upload)
   int sell_lanes = 0;
+  bool sell_held = false;
   int* sell_row = nullptr;
 };
 

@@ -408,7 +408,7 @@ __global__ void k_to_sell(int n, const int* __restrict__ rp, const int* __restri
 
 // CSR rows into lane slices (DevCsr::sell_lanes), one thread per lane of a row
 template <typename T>
-__global__ void k_to_lanes(int n, int K, const int* __restrict__ rp, const int* __restrict__ ci,
+__global__ void k_to_lanes(int n, int K, bool held, const int* __restrict__ rp, const int* __restrict__ ci,
                            const T* __restrict__ va, const int* __restrict__ cptr,
                            const int* __restrict__ perm, int* sci, T* sva) {
   const int64_t total = (int64_t)n * K;
@@ -418,9 +418,18 @@ __global__ void k_to_lanes(int n, int K, const int* __restrict__ rp, const int* 
     const int row = perm ? perm[p] : p;
     const int a = rp[row], len = rp[row + 1] - a, seg = (len + K - 1) / K;
     const int base = cptr[t >> 5] + (int)(t & 31);
-    for (int k = 0; k < seg && l * seg + k < len; ++k) {
-      sva[base + 32 * k] = va[a + l * seg + k];
-      if (sci) sci[base + 32 * k] = ci[a + l * seg + k];
+    // lane l takes seg entries in its slots 0 .. seg - 1; held: lane 0 one
+    // fewer, and the last entry in the chunk's last slot
+    const int e0 = held && l > 0 ? l * seg - 1 : l * seg;
+    const int e1 = min(held ? (l + 1) * seg - 1 : (l + 1) * seg, held ? len - 1 : len);
+    for (int e = e0; e < e1; ++e) {
+      sva[base + 32 * (e - e0)] = va[a + e];
+      if (sci) sci[base + 32 * (e - e0)] = ci[a + e];
+    }
+    if (held && l == 0 && len > 0) {
+      const int last = cptr[(t >> 5) + 1] - 32 + (int)(t & 31);
+      sva[last] = va[a + len - 1];
+      if (sci) sci[last] = ci[a + len - 1];
     }
   }
 }
@@ -428,8 +437,8 @@ __global__ void k_to_lanes(int n, int K, const int* __restrict__ rp, const int* 
 template <typename T>
 static void to_lanes(gs2_handle* h, const DevCsr& M, const T* va, T* sva, bool with_ci) {
   k_to_lanes<T><<<vec_blocks(h, (int64_t)M.n * M.sell_lanes), kVecThreads, 0, h->stream>>>(
-      M.n, M.sell_lanes, M.rp, M.ci, va, M.sell_ptr, M.sell_row, with_ci ? M.sell_ci : nullptr,
-      sva);
+      M.n, M.sell_lanes, M.sell_held, M.rp, M.ci, va, M.sell_ptr, M.sell_row,
+      with_ci ? M.sell_ci : nullptr, sva);
   GS2_LAUNCH_CHECK();
 }
 

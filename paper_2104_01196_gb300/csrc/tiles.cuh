@@ -618,10 +618,12 @@ k_stencil(int n, int nchunks, const int* __restrict__ cptr, const int* __restric
 // window start early and the hardware's block scheduler fills in the short
 // ones.  The next group's four slots are loaded while the current group's
 // gathers are in flight; padding slots (column -1) gather nothing, so an
-// infinity elsewhere cannot reach the row.
+// infinity elsewhere cannot reach the row.  HELD (DevCsr::sell_held): the last
+// slot of a row's first lane is its last entry, which joins the sum after the
+// lanes' parts.
 // (Five resident blocks: at the 66 registers ptxas takes unasked, three fit
 // and the uneven rows' sweep takes 91 instead of 70 us; at eight it takes 101.)
-template <int K, typename VT, class Epi>
+template <int K, bool HELD, typename VT, class Epi>
 __global__ void __launch_bounds__(kRowThreads, 5)
 k_lanes(int n, int nchunks, const int* __restrict__ cptr, const int* __restrict__ ci,
         const VT* __restrict__ va, Epi epi, const int* skip, const int* __restrict__ live,
@@ -656,7 +658,8 @@ k_lanes(int n, int nchunks, const int* __restrict__ cptr, const int* __restrict_
   typename Epi::Pre pv{};
   if (own) pv = epi.pre(row);
   AT s = AT(0);
-  for (int k = 0; k < L; k += 4) {
+  int k = 0;
+  for (; k + 4 < L; k += 4) {
     const AT x0 = c0 >= 0 ? (AT)epi.gather(c0) : AT(0);
     const AT x1 = c1 >= 0 ? (AT)epi.gather(c1) : AT(0);
     const AT x2 = c2 >= 0 ? (AT)epi.gather(c2) : AT(0);
@@ -664,11 +667,34 @@ k_lanes(int n, int nchunks, const int* __restrict__ cptr, const int* __restrict_
     const AT b0 = a0, b1 = a1, b2 = a2, b3 = a3;
     load(k + 4);
     s = fma(b0, x0, s);
-    if (k + 1 < L) s = fma(b1, x1, s);
-    if (k + 2 < L) s = fma(b2, x2, s);
-    if (k + 3 < L) s = fma(b3, x3, s);
+    s = fma(b1, x1, s);
+    s = fma(b2, x2, s);
+    s = fma(b3, x3, s);
   }
+  // the last group: one to four slots (none in a chunk of empty rows)
+  const int rem = L - k;
+  AT x0 = c0 >= 0 ? (AT)epi.gather(c0) : AT(0);
+  const AT x1 = c1 >= 0 ? (AT)epi.gather(c1) : AT(0);
+  const AT x2 = c2 >= 0 ? (AT)epi.gather(c2) : AT(0);
+  const AT x3 = c3 >= 0 ? (AT)epi.gather(c3) : AT(0);
+  if (rem > 1) {
+    s = fma(a0, x0, s);
+    a0 = a1;
+    x0 = x1;
+  }
+  if (rem > 2) {
+    s = fma(a0, x0, s);
+    a0 = a2;
+    x0 = x2;
+  }
+  if (rem > 3) {
+    s = fma(a0, x0, s);
+    a0 = a3;
+    x0 = x3;
+  }
+  if (rem > 0 && !(HELD && l == 0)) s = fma(a0, x0, s);
   if (K > 1) s = group_sum<K, AT>(s);
+  if (HELD) s = fma(a0, x0, s);
   if (own && l == 0) epi.finish(row, s, pv);
 }
 
@@ -716,11 +742,19 @@ inline const int* live_rows(const gs2_handle* h, const DevCsr& M) {
 template <typename VT, class Epi>
 inline void launch_lanes(gs2_handle* h, const DevCsr& M, const VT* sv, const Epi& epi,
                          const int* skip) {
-  auto fn = M.sell_lanes == 1   ? k_lanes<1, VT, Epi>
-            : M.sell_lanes == 2 ? k_lanes<2, VT, Epi>
-            : M.sell_lanes == 4 ? k_lanes<4, VT, Epi>
-            : M.sell_lanes == 8 ? k_lanes<8, VT, Epi>
-                                : k_lanes<16, VT, Epi>;
+  auto fn = M.sell_lanes == 1   ? k_lanes<1, false, VT, Epi>
+            : M.sell_lanes == 2 ? k_lanes<2, false, VT, Epi>
+            : M.sell_lanes == 4 ? k_lanes<4, false, VT, Epi>
+            : M.sell_lanes == 8 ? k_lanes<8, false, VT, Epi>
+                                : k_lanes<16, false, VT, Epi>;
+  // (lower precisions have slices only with the row tiles' lanes)
+  if constexpr (sizeof(VT) == sizeof(double)) {
+    if (M.sell_held)
+      fn = M.sell_lanes == 2   ? k_lanes<2, true, VT, Epi>
+           : M.sell_lanes == 4 ? k_lanes<4, true, VT, Epi>
+           : M.sell_lanes == 8 ? k_lanes<8, true, VT, Epi>
+                               : k_lanes<16, true, VT, Epi>;
+  }
   const int warps = kRowThreads / 32;
   const int grid = (M.sell_chunks + warps - 1) / warps;
   launch_pdl(fn, grid, kRowThreads, 0, h->stream, M.n, M.sell_chunks, (const int*)M.sell_ptr,

@@ -106,3 +106,41 @@ def test_exact_and_multicolour_sweeps(g, name):  # noqa: F811
     x = dev(x0)
     g.mtgs_apply(h, dev(b), x, 1, 1.0, g.FORWARD)
     assert np.array_equal(host(x), want)
+
+
+# a row's total meets its last entry in one rounding also where the row is summed on several lanes:
+# an even number of ones, then a last entry of 2^53, is exact that way; a one added to 2^53 on its own
+# is lost
+@pytest.mark.parametrize("n,mean", [(3000, 11), (20000, 11), (120000, 14), (900, 60)])
+def test_last_entry(g, n, mean):  # noqa: F811
+    rng = np.random.RandomState(n)
+    count = 2 * np.clip((mean / 2.0 * np.exp(0.6 * rng.randn(n))).astype(int), 0, 60)
+    rp = np.concatenate([[0], np.cumsum(count + 1)]).astype(np.int64)
+    row = np.repeat(np.arange(n), count + 1)
+    k = np.arange(len(row)) - rp[row]
+    ci = np.where(k == count[row], row, (row + 1 + k) % n).astype(np.int32)
+    va = np.where(k == count[row], 2.0 ** 53, 1.0)
+    h = g.gs2_setup((rp, ci, va))
+    y = dev(np.zeros(n))
+    g.gs2_spmv(h, dev(np.ones(n)), y)
+    assert np.array_equal(host(y), 2.0 ** 53 + count)
+
+
+# ... and in the local blocks of the hybrid form
+@pytest.mark.parametrize("n,mean", [(3000, 11), (20000, 11)])
+def test_last_entry_hybrid(g, n, mean):  # noqa: F811
+    rng = np.random.RandomState(n + 1)
+    count = 2 * np.clip((mean / 2.0 * np.exp(0.6 * rng.randn(n))).astype(int), 0, 60)
+    rp = np.concatenate([[0], np.cumsum(count + 1)]).astype(np.int64)
+    row = np.repeat(np.arange(n), count + 1)
+    k = np.arange(len(row)) - rp[row]
+    half = n // 2  # two blocks, each row's columns inside its own
+    lo, size = np.where(row < half, 0, half), np.where(row < half, half, n - half)
+    ci = np.where(k == count[row], row, lo + (row - lo + 1 + k) % size).astype(np.int32)
+    va = np.where(k == count[row], 2.0 ** 53, 1.0)
+    h = g.gs2_setup((rp, ci, va))
+    # one sweep without an inner one from x = 1, b = 0: x - (2^53 + count) / 2^53
+    x = dev(np.ones(n))
+    g.relax_apply(h, dev(np.zeros(n)), x, g.params("gs2", inner=0, parts=2))
+    want = 1.0 - (2.0 ** 53 + count) * 2.0 ** -53
+    assert np.array_equal(host(x), want)
