@@ -1,6 +1,6 @@
 // The triangular solve of exact Gauss-Seidel / SOR, (D + omega T) g = r by
 // D^{-1}:  g_i = rhat_i - omega sum_k T_ik g_k, then x_i += omega g_i, in one
-// launch for the whole triangle.
+// launch for the whole triangle (or one per level where there are few: by_level).
 //
 // What bounds it is the chain of levels: a 100^3 stencil has 298 of them,
 // each a dependent step, against 24 us of memory traffic for the sweep.  One
@@ -141,6 +141,41 @@ k_trisolve(TriView T, const double* __restrict__ rhat, double* x, double omega, 
   }
 }
 
+// One level: rows p0 .. p1 of the level order, g of the earlier levels final.
+// The arithmetic of a row is that of k_trisolve.
+template <int K>
+__global__ void __launch_bounds__(kTriThreads)
+k_level(int p0, int p1, TriView T, const double* __restrict__ rhat, double* x, double omega,
+        int x_zero, const int* skip) {
+  pdl_wait();
+  if (skip && *skip) return;
+  double* g = (double*)T.g;
+  const int q = threadIdx.x / K, l = threadIdx.x % K;
+  constexpr int R = kTriThreads / K;
+  for (int base = p0 + blockIdx.x * R; base < p1; base += gridDim.x * R) {
+    const int p = base + q;
+    const bool own = p < p1;
+    double s = 0.0, rh = 0.0, xi = 0.0;
+    int row = 0;
+    if (own) {
+      if (l == 0) {
+        row = __ldg(T.rows + p);
+        rh = rhat[row];
+        if (!x_zero) xi = x[row];
+      }
+      const int e = __ldg(T.rp + p + 1);
+      for (int k = __ldg(T.rp + p) + l; k < e; k += K)
+        s = fma(__ldg(T.va + k), g[__ldg(T.ci + k)], s);
+    }
+    if (K > 1) s = group_sum<K, double>(s);
+    if (own && l == 0) {
+      const double gi = rh - omega * s;
+      g[p] = gi;
+      x[row] = xi + omega * gi;
+    }
+  }
+}
+
 // entries of the rows in level order (rp: their places): the place of each
 // entry's column, and its value
 __global__ void k_tri_place(int n, const int* __restrict__ rows, int* place) {
@@ -209,13 +244,41 @@ void tri_upload(gs2_handle* h, const DevCsr& M, const std::vector<int>& rows,
   GS2_LAUNCH_CHECK();
 }
 
+// Few levels of many rows are cheaper as a launch per level: a level then costs
+// 3 to 4 us, but its rows stream without the fill of g, the counter and the
+// polls, which cost about 20 us per million rows.  The line is where the two
+// cross on 7-point rows in 1 to 33 levels, half sweeps in us, residual included
+// (launch per level / one launch):
+//                 1 level       3            5            9            17           33
+//     4,096 rows  5.7 / 7.2     9.1 / 8.3    12.5 / 9.4   19 / 12      35 / 18      63 / 28
+//    32,768       5.8 / 7.3     9.3 / 9.2    13.6 / 10.7  22 / 15      34 / 20      67 / 32
+//   262,144       6.3 / 14.2    14.9 / 19.4  20.2 / 20.7  27 / 22      44 / 30      75 / 44
+// 2,097,152       32 / 73       81 / 126     86 / 128     95 / 128     118 / 131    155 / 131
+// (Longer rows in so few levels favour the launches more.)  Both forms give the
+// same bits.
+static bool by_level(const TriSolve& T, int n) {
+  return (int64_t)T.levels.size() - 1 <= 2 + n / 100000;
+}
+
 void launch_trisolve(gs2_handle* h, const TriSolve& T, const double* rhat, double* x,
                      double omega, bool x_zero, const int* skip) {
   if (h->n == 0) return;
   const int n = (int)h->n;
+  const TriView v{T.nchunks, T.chunk, T.rows, T.rp, T.ci, T.va, T.g, T.ticket};
+  if (by_level(T, n)) {
+    auto fn = T.lanes == 16 ? k_level<16> : T.lanes == 4 ? k_level<4> : k_level<1>;
+    const int R = kTriThreads / T.lanes;
+    for (size_t q = 0; q + 1 < T.levels.size(); ++q) {
+      const int p0 = T.levels[q], p1 = T.levels[q + 1];
+      const int grid = std::max(1, std::min((p1 - p0 + R - 1) / R, 8 * h->nsm));
+      launch_pdl(fn, grid, kTriThreads, 0, h->stream, p0, p1, v, rhat, x, omega, x_zero ? 1 : 0,
+                 skip);
+      GS2_LAUNCH_CHECK();
+    }
+    return;
+  }
   launch_pdl(k_tri_begin, vec_blocks(h, n), kVecThreads, 0, h->stream, n, T.g, T.ticket, skip);
   GS2_LAUNCH_CHECK();
-  const TriView v{T.nchunks, T.chunk, T.rows, T.rp, T.ci, T.va, T.g, T.ticket};
   const int warps = kTriThreads / 32;
   const int grid = std::max(1, std::min((T.nchunks + warps - 1) / warps,
                                         kTriBlocksPerSm * h->nsm));
