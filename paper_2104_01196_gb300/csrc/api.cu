@@ -276,9 +276,10 @@ constexpr double kSellStreamBytes = 128.0 * (1 << 20);  // CSR bytes beyond L2
 // at most its longest row + kOffsetSlack and at most 32 (stencil rows: the
 // rows at a grid boundary miss some offsets and get zero slots there).
 // Consecutive chunks with the same offset list share one copy.  With `origin`
-// (a colour's rows, origin[i] their row in A) offsets are j - origin[i], and a
-// chunk that stores a zero keeps its columns: the kernel tells an empty slot by
-// its zero value, and a stored zero times an infinity or NaN is a NaN.  Returns
+// (a colour's rows, origin[i] their row in A) offsets are j - origin[i], and
+// with `zeros` (the rows store zeros) every chunk keeps its columns: the kernel
+// tells an empty slot by its zero value, and a stored zero times an infinity or
+// NaN is a NaN.  Returns
 // false when the layout pads too much or its slots would not fit 32-bit
 // offsets.
 constexpr int kOffsetSlack = 2;
@@ -289,8 +290,8 @@ struct SellLayout {
   int offset_chunks = 0, wmax = 0;
 };
 
-static bool sell_layout(const std::vector<int>& rp, const int* ci, const double* va, int n,
-                        const int* origin, SellLayout& out) {
+static bool sell_layout(const std::vector<int>& rp, const int* ci, int n, const int* origin,
+                        bool zeros, SellLayout& out) {
   const int nc = (n + kSellC - 1) / kSellC;
   out.cptr.assign(nc + 1, 0);
   out.coff.assign(nc, -1);
@@ -302,12 +303,11 @@ static bool sell_layout(const std::vector<int>& rp, const int* ci, const double*
   for (int c = 0; c < nc; ++c) {
     int L = 0;
     u.clear();
-    bool regular = true;
+    bool regular = !zeros;
     for (int i = c * kSellC; i < std::min(n, (c + 1) * kSellC); ++i) {
       L = std::max(L, rp[i + 1] - rp[i]);
       const int at = origin ? origin[i] : i;
       for (int k = rp[i]; regular && k < rp[i + 1]; ++k) {
-        if (origin && va[k] == 0.0) regular = false;
         const int o = ci[k] - at;
         if (std::find(u.begin(), u.end(), o) == u.end()) {
           u.push_back(o);
@@ -424,7 +424,7 @@ static bool lane_layout(const std::vector<int>& rp, int n, int K, LaneLayout& ou
 // there (launch_to_sell, launch_to_lanes); only the chunk layout is computed
 // here.
 static void upload_sell(gs2_handle* h, DevCsr& M, const std::vector<int>& rp, const int* ci,
-                        const double* va, const int* origin) {
+                        const int* origin, bool zeros) {
   const int n = M.n;
   if (n == 0 || M.nnz == 0) return;
   SellLayout lay;
@@ -445,7 +445,7 @@ static void upload_sell(gs2_handle* h, DevCsr& M, const std::vector<int>& rp, co
   // 3% lost on 64^3)
   const bool few = &M == &h->A && !short_rows && streams &&
                    n < 2 * 32 * (int64_t)kSellWarpsPerSm * h->nsm && try_lanes(1);
-  bool sliced = !few && (short_rows || streams) && sell_layout(rp, ci, va, n, origin, lay);
+  bool sliced = !few && (short_rows || streams) && sell_layout(rp, ci, n, origin, zeros, lay);
   // short rows with explicit columns, too few for the SMs' warps at one lane
   // each (the 64,560 rows of a second multigrid level, 15 entries in a
   // triangle: inner sweep 12.6 -> 8.6 us with two lanes); long rows here
@@ -501,7 +501,7 @@ static void upload_sell(gs2_handle* h, DevCsr& M, const std::vector<int>& rp, co
 
 static void upload_csr(gs2_handle* h, DevCsr& M, int n, const std::vector<int>& rp,
                        const int* ci, const double* va, int nnz,
-                       const int* origin = nullptr) {
+                       const int* origin = nullptr, bool zeros = false) {
   M.n = n;
   M.nnz = nnz;
   M.mean_row = n ? (double)M.nnz / n : 0.0;
@@ -519,7 +519,7 @@ static void upload_csr(gs2_handle* h, DevCsr& M, int n, const std::vector<int>& 
   h->h2d(M.ci, ci, sizeof(int) * M.nnz);
   h->h2d(M.va, va, sizeof(double) * M.nnz);
   retile(h, M, rp, M.tpr, 1);
-  upload_sell(h, M, rp, ci, va, origin);
+  upload_sell(h, M, rp, ci, origin, zeros);
 }
 
 // (Re)build the row tiles of M for K lanes per row and RPT rows per lane
@@ -834,7 +834,9 @@ void ensure_colors(gs2_handle* h) {
       rp[q + 1] = rp[q] + (L.rp[rr[q] + 1] - L.rp[rr[q]]) + (U.rp[rr[q] + 1] - U.rp[rr[q]]);
     std::vector<int> ci(rp.back());
     std::vector<double> va(rp.back());
+    std::atomic<bool> zeros{false};
     parallel_ranges((int64_t)rr.size(), [&](int64_t q0, int64_t q1, int) {
+      bool zero = false;
       for (int64_t q = q0; q < q1; ++q) {
         const int i = rr[q];
         int o = rp[q];
@@ -842,14 +844,16 @@ void ensure_colors(gs2_handle* h) {
           for (int k = T->rp[i]; k < T->rp[i + 1]; ++k, ++o) {
             ci[o] = T->ci[k];
             va[o] = T->va[k];
+            zero |= va[o] == 0.0;
           }
       }
+      if (zero) zeros = true;
     });
     h->color_rows[c] = (int*)h->dalloc(sizeof(int) * std::max<size_t>(rr.size(), 1));
     h->h2d(h->color_rows[c], rr.data(), sizeof(int) * rr.size());
     h->colors[c].sell_origin = h->color_rows[c];
     upload_csr(h, h->colors[c], (int)rr.size(), rp, ci.data(), va.data(), (int)ci.size(),
-               rr.data());
+               rr.data(), zeros);
   }
   h->colors_ready = true;
 }
