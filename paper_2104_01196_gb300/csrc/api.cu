@@ -368,8 +368,8 @@ static int lane_count(const gs2_handle* h, int64_t n, double mean, int longest) 
 // Lane-slice layout: K lanes per row, rows sorted by their number of slots
 // inside windows of kLaneWindow rows where the padding calls for it (the sort
 // is stable and local, so neighbouring rows' gathers stay near one another).
-// Returns false when the slots would not fit 32-bit offsets.
-
+// Returns false when that pads too much or its slots would not fit 32-bit
+// offsets.
 struct LaneLayout {
   std::vector<int> cptr, row;  // row empty: in order
 };
@@ -380,21 +380,31 @@ static bool lane_layout(const std::vector<int>& rp, int n, int K, LaneLayout& ou
   // the 2,386 rows of a third multigrid level, 33 entries in a triangle)
   const bool small = rp[n] <= kSellSmall && rp[n] > kShortRowMean * n;
   const double padding = small ? 2.0 : kSellMaxPadding;
+  int shift = 0;
+  while (1 << shift < K) ++shift;
   std::vector<int> width(n);
-  for (int i = 0; i < n; ++i) width[i] = (rp[i + 1] - rp[i] + K - 1) / K;
+  parallel_ranges(n, [&](int64_t i0, int64_t i1, int) {
+    for (int64_t i = i0; i < i1; ++i) width[i] = (rp[i + 1] - rp[i] + K - 1) >> shift;
+  });
   auto chunks = [&](const std::vector<int>& row) {
     out.cptr.assign((n + per - 1) / per + 1, 0);
+    // each chunk's width (chunks that start in a thread's range are its), then
+    // the places
+    parallel_ranges(n, [&](int64_t i0, int64_t i1, int) {
+      for (int c = (int)((i0 + per - 1) / per); (int64_t)c * per < i1; ++c) {
+        int w = 0;
+        for (int p = c * per; p < std::min(n, (c + 1) * per); ++p)
+          w = std::max(w, width[row.empty() ? p : row[p]]);
+        out.cptr[c + 1] = w;
+      }
+    });
     int64_t total = 0;
     for (size_t c = 0; c + 1 < out.cptr.size(); ++c) {
-      if (total > padding * rp[n]) return false;
-      int w = 0;
-      for (int p = (int)c * per; p < std::min(n, ((int)c + 1) * per); ++p)
-        w = std::max(w, width[row.empty() ? p : row[p]]);
-      total += 32 * (int64_t)w;
-      if (total > INT32_MAX) return false;
+      total += 32 * (int64_t)out.cptr[c + 1];
+      if (total > INT32_MAX || total > padding * rp[n]) return false;
       out.cptr[c + 1] = (int)total;
     }
-    return total <= padding * rp[n];
+    return true;
   };
   out.row.clear();
   if (chunks(out.row)) return true;
@@ -461,6 +471,32 @@ static void upload_sell(gs2_handle* h, DevCsr& M, const std::vector<int>& rp, co
     return;  // row tiles
   const std::vector<int>& cptr = sliced ? lay.cptr : lanes.cptr;
   const size_t slots = std::max(cptr.back(), 1);
+  M.sell_chunks = (int)cptr.size() - 1;
+  M.sell_slots = (int)slots;
+  M.sell = true;
+  if (!sliced) {
+    // one allocation (they take a good part of a small matrix's setup)
+    auto up = [](size_t x) { return (x + 255) / 256 * 256; };
+    const size_t rows = lanes.row.empty() ? 0 : sizeof(int) * n;
+    char* base = (char*)h->dalloc(up(sizeof(double) * slots) + up(sizeof(int) * slots) +
+                                  up(sizeof(int) * cptr.size()) + rows);
+    M.sell_va = (double*)base;
+    base += up(sizeof(double) * slots);
+    M.sell_ci = (int*)base;
+    base += up(sizeof(int) * slots);
+    M.sell_ptr = (int*)base;
+    base += up(sizeof(int) * cptr.size());
+    h->dzero(M.sell_va, sizeof(double) * slots);
+    h->h2d(M.sell_ptr, cptr.data(), sizeof(int) * cptr.size());
+    M.sell_held = M.diagonal && M.sell_lanes > choose_lanes(M.mean_row);
+    GS2_CUDA(cudaMemsetAsync(M.sell_ci, 0xff, sizeof(int) * slots, h->stream));
+    if (rows) {
+      M.sell_row = (int*)base;
+      h->h2d(M.sell_row, lanes.row.data(), sizeof(int) * n);
+    }
+    launch_to_sell(h, M, M.va, M.sell_va, true);
+    return;
+  }
   std::vector<int> top(kHostThreads, 0);
   auto largest = [&](int64_t k0, int64_t k1, int t) {
     int v = 0;
@@ -469,26 +505,12 @@ static void upload_sell(gs2_handle* h, DevCsr& M, const std::vector<int>& rp, co
   };
   if (M.nnz < (1 << 22)) largest(0, M.nnz, 0);  // (sooner done than threads are started)
   else parallel_ranges(M.nnz, largest);
-  const int ncols = 1 + *std::max_element(top.begin(), top.end());
-  M.sell_chunks = (int)cptr.size() - 1;
-  M.sell_slots = (int)slots;
-  M.sell_ncols = ncols;
+  M.sell_ncols = 1 + *std::max_element(top.begin(), top.end());
   M.sell_ptr = (int*)h->dalloc(sizeof(int) * cptr.size());
   M.sell_ci = (int*)h->dalloc(sizeof(int) * slots);
   M.sell_va = (double*)h->dalloc(sizeof(double) * slots);
   h->dzero(M.sell_va, sizeof(double) * slots);
   h->h2d(M.sell_ptr, cptr.data(), sizeof(int) * cptr.size());
-  M.sell = true;
-  if (!sliced) {
-    M.sell_held = M.diagonal && M.sell_lanes > choose_lanes(M.mean_row);
-    GS2_CUDA(cudaMemsetAsync(M.sell_ci, 0xff, sizeof(int) * slots, h->stream));
-    if (!lanes.row.empty()) {
-      M.sell_row = (int*)h->dalloc(sizeof(int) * n);
-      h->h2d(M.sell_row, lanes.row.data(), sizeof(int) * n);
-    }
-    launch_to_sell(h, M, M.va, M.sell_va, true);
-    return;
-  }
   M.sell_wmax = lay.wmax;
   M.sell_offset_chunks = lay.offset_chunks;
   M.sell_coff = (int*)h->dalloc(sizeof(int) * std::max<size_t>(lay.coff.size(), 1));
