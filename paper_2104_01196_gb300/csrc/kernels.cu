@@ -233,7 +233,7 @@ struct EpiResidSweep {
 // compact right-hand side of Eq. (9) on the other prescaled triangle
 // T' = D^{-1} U (forward) or D^{-1} L (backward):  rhat = D^{-1} b - T' x
 struct EpiCompact {
-  static constexpr int kUnroll = 8;
+  static constexpr int kUnroll = 2;
   static constexpr bool kGuard = false;
   const double* __restrict__ x;
   const double* __restrict__ b;

@@ -778,9 +778,12 @@ inline void launch_sell(gs2_handle* h, const DevCsr& M, const VT* sv, const Epi&
   // to the width at which it is the faster one for the epilogue: for the FP64
   // residual 6 slots (its two more row operands and 7 slots need 56
   // registers, half the resident warps: 58 against 53 us on 7-point rows,
-  // n = 3.4M), for the whole-sweep residual 4.  FP16 values (whose conversion
-  // and row scale cost it 46 registers) keep k_sell: inner sweep 19 against 23
-  // us at the same size.
+  // n = 3.4M), for the compact right-hand side 2 (a compact symmetric sweep on
+  // the 100^3 convection-diffusion matrix, 3-entry triangles, 47.0 against 42.7
+  // us; on the 1000^2 Laplacian, 2 entries, 37.8 against 41.6), for the
+  // whole-sweep residual 4.  FP16 values (whose conversion and row scale cost it
+  // 46 registers) keep k_sell: inner sweep 19 against 23 us on 7-point rows'
+  // triangles, n = 3.4M.
   bool pair = false;
   auto fn = M.mean_row > kShortRowMean ? k_sell<VT, Epi, true, false> : k_sell<VT, Epi, false, false>;
   if constexpr (sizeof(VT) < sizeof(double)) {
