@@ -24,15 +24,20 @@ constexpr int kSmCtas = 16;
 constexpr int kSmThreads = 512;
 constexpr int kSmSide = 4;  // entries of a row to either side of the diagonal
 
-// The sizes it takes: up to 4,096 rows always, up to 8,192 (512 rows an SM,
-// whose FP64 pipe then sets the time of a phase) from six row kernels on.
-// Back-to-back calls, us, row kernels and one launch:
-//                          400 rows   4,096      8,100
-//   forward (2 kernels)    5.4  3.9   5.5  4.8   5.4  6.3
-//   symmetric (4)          8.9  5.6   9.1  6.8   9.2  9.5
-//   symmetric, 3 inner (8) 16.2 7.8   17.2 9.5   17.3 13.6
-constexpr int64_t kSmallRows = 4096, kSmallRowsMany = 8192;
-constexpr int64_t kSmallMany = 6;
+// The sizes it takes, by the row kernels that it replaces: the launches saved
+// grow with them, and beyond 256 rows an SM its FP64 pipe sets the time of a
+// phase.  The lines are where the two cross on 7-point rows (5-point rows cross
+// later, at 5,500 and 6,500 rows); back-to-back calls, us, row kernels / one
+// launch:
+//                          400 rows    4,096       5,832       6,859       8,000
+//   forward (2 kernels)    5.3  4.2    5.3  5.3    5.5  6.0    5.3  6.3    5.3  6.8
+//   symmetric (4)          8.7  5.8    9.3  7.3    8.9  8.7    8.9  9.5    8.8 10.1
+//   symmetric, 2 inner (6) 12.1 7.0    13.4 9.0    13.6 10.8   13.8 11.8   13.3 12.7
+//   symmetric, 3 inner (8) 15.7 8.4    17.5 10.8   17.8 13.1   17.9 14.4   17.6 15.5
+// (400 rows of a 5-point stencil.)
+static int64_t small_rows(int64_t kernels) {
+  return kernels >= 6 ? 8192 : kernels >= 4 ? 6000 : 4096;
+}
 
 struct SmallArgs {
   int n, R;  // rows, rows per CTA
@@ -160,8 +165,7 @@ __global__ void __launch_bounds__(kSmThreads, 1) k_small_sweeps(SmallArgs a) {
 bool small_sweeps_eligible(gs2_handle* h, const gs2_params* p) {
   const int64_t kernels = (p->direction == GS2_SYMMETRIC ? 2 : 1) * (int64_t)(1 + p->inner) *
                           p->outer * std::max(1, p->local_sweeps);
-  if (h->n < 1 || h->n > (kernels >= kSmallMany ? kSmallRowsMany : kSmallRows) || h->pack ||
-      !h->parted || profiling_active(h))
+  if (h->n < 1 || h->n > small_rows(kernels) || h->pack || !h->parted || profiling_active(h))
     return false;
   if (p->kind != GS2_PC_GS2 || p->precision != GS2_FP64 || p->form != GS2_NONCOMPACT ||
       p->parts > 1)
