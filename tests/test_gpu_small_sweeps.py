@@ -34,3 +34,22 @@ def test_no_inner_sweep(g, name, direction, omega):  # noqa: F811
         x = dev(x0)
         g.gs2_apply_ex(h, dev(b), x, pc)
         assert np.array_equal(host(x), rows)
+
+
+# inner sweeps, relaxed and damped: the same bits as the row kernels too
+@pytest.mark.parametrize("name", ["poisson2d_64", "poisson3d_17"])
+@pytest.mark.parametrize("outer,inner,omega,gamma", [
+    (2, 1, 0.9, 1.0), (1, 2, 1.0, 0.7), (2, 3, 0.9, 0.7), (1, 3, 1.1, 1.0)])
+def test_inner_sweeps(g, name, outer, inner, omega, gamma):  # noqa: F811
+    kind, size = name.split("_")
+    A = getattr(P, kind + "_matrix")(int(size))
+    b, x0 = rhs_and_x0(A, 82)
+    h = g.gs2_setup(A)
+    pc = g.params("gs2", outer=outer, inner=inner, omega=omega, gamma=gamma, direction="symmetric")
+    out = []
+    for profiled in (True, False):
+        h.profile(profiled)
+        x = dev(x0)
+        g.gs2_apply_ex(h, dev(b), x, pc)
+        out.append(host(x))
+    assert np.array_equal(out[0], out[1])
