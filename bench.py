@@ -1131,7 +1131,7 @@ def hybrid(gs2, torch, pr, stream, b):
     """The hybrid (block-Jacobi) preconditioners of the paper's distributed
     runs on the same workload, P row blocks standing in for P processes:
     the global JR(4,1), the local JR(1,4), hybrid SGS2(1,1) and hybrid exact
-    SGS (local triangular solves by level sets); GMRES(30)
+    SGS (local triangular solves); GMRES(30)
     iterations and device time per solve for each P (one untimed solve
     first, which also builds the blocks' matrices)."""
     res = {"workload": "GMRES(30) to 1e-8 on the 128^3 Laplacian, P contiguous row blocks"}

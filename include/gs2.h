@@ -4,8 +4,8 @@
  * Two-stage Gauss-Seidel (GS2) replaces the sparse triangular solve of a
  * Gauss-Seidel sweep by a fixed number of inner Jacobi-Richardson (JR)
  * sweeps (Sec. 4, Eq. (2)-(5)); it is used here as a relaxation and as the
- * preconditioner of restarted GMRES.  Exact GS through a level-scheduled
- * triangular solve and damped JR are provided beside it as baselines.
+ * preconditioner of restarted GMRES.  Exact GS through a triangular solve
+ * in level order and damped JR are provided beside it as baselines.
  *
  * Conventions shared by every call:
  *  - Status: every call returns a gs2_status and never throws across the
@@ -83,7 +83,7 @@ typedef enum {
   GS2_PC_NONE = 0, /* identity */
   GS2_PC_GS2 = 1,  /* two-stage GS, Eq. (2)-(5) with damping */
   GS2_PC_JR = 2,   /* damped Jacobi-Richardson, `outer` sweeps */
-  GS2_PC_GS = 3,   /* exact GS/SOR, level-scheduled, `outer` sweeps */
+  GS2_PC_GS = 3,   /* exact GS/SOR (triangular solves), `outer` sweeps */
   GS2_PC_MTGS = 4, /* multicolour GS/SOR, `outer` sweeps (Sec. 6.1.2) */
   GS2_PC_AMG = 5,  /* one AMG V-cycle, GS2 smoother (outer, inner, omega,
                       gamma, precision) on every level */
@@ -129,7 +129,7 @@ typedef struct {
 
 typedef struct {
   int64_t n, nnz, nnz_lower, nnz_upper;
-  int levels_lower, levels_upper; /* 0 until a level-scheduled call */
+  int levels_lower, levels_upper; /* 0 until a call of exact GS */
   int64_t device_bytes;           /* device memory held by the handle */
   int tpr_a, tpr_tri;             /* lanes per row of the tile kernels (A, D^-1 L) */
   int rpt_a, rpt_tri;             /* rows per lane group of the tile kernels */
@@ -273,9 +273,10 @@ gs2_status gs2_apply_noalloc(int64_t n, const int64_t* rowptr, const int32_t* co
                              int direction, void* stream);
 
 /* Exact GS / SOR baseline: x + omega (D + omega T)^{-1} (b - A x) per half
- * sweep (Sec. 4, "Damping factor"), the triangular solve scheduled by
- * level sets of T (Sec. 3, level-set scheduling).  Levels are computed on
- * the first call. x in/out. */
+ * sweep (Sec. 4, "Damping factor"), the triangular solve in the order of
+ * the level sets of T (Sec. 3): one launch in which a row waits for its own
+ * dependencies only, or a launch per level where there are few.  Levels are
+ * computed on the first call. x in/out. */
 gs2_status gs_apply(gs2_handle* h, const double* b, double* x, int sweeps,
                     double omega, int direction);
 
@@ -340,7 +341,7 @@ gs2_status gs2_amg_info(const gs2_handle* h, int* levels, int64_t* rows, int64_t
 gs2_status gs2_amg_vcycle(gs2_handle* h, const double* b, double* x, const gs2_params* p);
 
 /* The relaxation of p's kind from x (in/out): GS2 (as gs2_apply_ex), JR,
- * exact GS by level sets or multicolour GS, with `outer` sweeps; for GS2, JR
+ * exact GS or multicolour GS, with `outer` sweeps; for GS2, JR
  * and GS the hybrid (block-Jacobi) form when p->parts > 1, local exact GS
  * solving each block's triangle by its own level sets.  Errors: INVALID_ARG
  * for the other kinds and bad parameters, OOM, CUDA. */
@@ -391,7 +392,7 @@ gs2_status gs2_batch_solve(gs2_handle* const* hs, const double* const* bs,
  * A pack holds `count` independent systems A_s x_s = b_s as one handle
  * whose matrix is their block-diagonal concatenation diag(A_0, ..., A_{S-1})
  * (system s owns rows offsets[s] .. offsets[s+1]-1).  Every row kernel of a
- * sweep (residual, inner JR sweeps, SpMV, level-scheduled and multicolour
+ * sweep (residual, inner JR sweeps, SpMV, exact and multicolour
  * GS, JR) covers all systems in one launch: a row reads only its own
  * system's columns, so each system is relaxed exactly as it would be alone
  * (gs2_apply and the other relaxations work on a pack unchanged, vectors

@@ -1,8 +1,8 @@
 // Packs: many independent systems solved together as one block-diagonal
 // matrix diag(A_0, ..., A_{S-1}) held by a single handle.
 //
-// A GS2 sweep (and the residual, the SpMV, JR, level-scheduled and
-// multicolour GS) of a block-diagonal matrix is the sweep of every block on
+// A GS2 sweep (and the residual, the SpMV, JR, exact and multicolour
+// GS) of a block-diagonal matrix is the sweep of every block on
 // its own: a row reads only columns of its own system, the triangles of the
 // pack are the blocks' triangles, and its level sets and first-fit colours
 // are those of the blocks side by side.  So each row kernel covers all
@@ -693,8 +693,8 @@ struct PackRun {
     launch_pdl(k_pnorm_part, P->gb, kVecThreads, 0, h->stream, P->blk, P->items, P->cnt, v, P->part,
                P->nb);
     GS2_LAUNCH_CHECK();
-    launch_pdl(k_pnorm_final, P->gs, 256, 0, h->stream, P->part, P->seg_blk, P->sys, P->cnt + 1, P->st,
-               which);
+    launch_pdl(k_pnorm_final, P->gs, 256, 0, h->stream, P->part, P->seg_blk, P->sys, P->cnt + 1,
+               P->st, which);
     GS2_LAUNCH_CHECK();
   }
 
@@ -781,15 +781,15 @@ struct PackRun {
     const int N = (int)h->n;
     switch (jc) {
 #define GS2_PDOTS_CASE(J)                                                               \
-  case J:                                                                               \
-    launch_pdl(k_pdots<J>, P->gb, kVecThreads, 0, h->stream, N, P->blk, P->items, P->cnt, P->st, h->V,  \
-               h->w, part, P->nb);                                                               \
+  case J:                                                                                \
+    launch_pdl(k_pdots<J>, P->gb, kVecThreads, 0, h->stream, N, P->blk, P->items, P->cnt, \
+               P->st, h->V, h->w, part, P->nb);                                          \
     break;
       GS2_PJC_CASES(GS2_PDOTS_CASE)
 #undef GS2_PDOTS_CASE
       default:
-        launch_pdl(k_pdots_rt<64>, P->gb, kVecThreads, 0, h->stream, N, P->blk, P->items, P->cnt, P->st,
-                   h->V, jc, h->w, part, P->nb);
+        launch_pdl(k_pdots_rt<64>, P->gb, kVecThreads, 0, h->stream, N, P->blk, P->items, P->cnt,
+                   P->st, h->V, jc, h->w, part, P->nb);
         break;
     }
     GS2_LAUNCH_CHECK();
@@ -824,8 +824,8 @@ struct PackRun {
 
   void launch_reduce(int j, int jc, int mode, const double* part) {
     KernelTimer tm(h, "reduce_cols", 8.0 * jc * P->nb);
-    launch_pdl(k_preduce, P->gs, 256, 0, h->stream, part, P->nb, P->seg_blk, P->sys, P->cnt + 1, P->st,
-               P->H, P->hstride(), ldh(), j, P->hbuf, (int)P->vstride(), mode, jc);
+    launch_pdl(k_preduce, P->gs, 256, 0, h->stream, part, P->nb, P->seg_blk, P->sys, P->cnt + 1,
+               P->st, P->H, P->hstride(), ldh(), j, P->hbuf, (int)P->vstride(), mode, jc);
     GS2_LAUNCH_CHECK();
   }
 
@@ -849,16 +849,16 @@ struct PackRun {
     launch_update<true>(j, P->part2, P->part);
     {
       KernelTimer tm(h, "givens", 8.0 * P->nb + 8.0 * 4 * (j + 2) * P->count);
-      launch_pdl(k_pgivens, P->gs, 128, 0, h->stream, P->part, P->seg_blk, P->sys, P->cnt + 1, P->st, P->H,
-                 P->hstride(), ldh(), j, P->cs, P->sn, P->gvec, (int)P->vstride(), P->nactive, P->off_dev,
-                 P->live_run, h->st, h->stop_mapped_dev);
+      launch_pdl(k_pgivens, P->gs, 128, 0, h->stream, P->part, P->seg_blk, P->sys, P->cnt + 1,
+                 P->st, P->H, P->hstride(), ldh(), j, P->cs, P->sn, P->gvec, (int)P->vstride(),
+                 P->nactive, P->off_dev, P->live_run, h->st, h->stop_mapped_dev);
       GS2_LAUNCH_CHECK();
     }
     if (j + 1 < m) {
       KernelTimer tm(h, "scale_next",
                      16.0 * N + (r64 ? 16.0 * N : 0.0) + (r32 ? 12.0 * N : 0.0));
-      launch_pdl(k_pscale_next, P->gb, kVecThreads, 0, h->stream, P->blk, P->items, P->cnt, P->st, h->w,
-                 h->V + (size_t)(j + 1) * N, h->dinv, r64, r32);
+      launch_pdl(k_pscale_next, P->gb, kVecThreads, 0, h->stream, P->blk, P->items, P->cnt, P->st,
+                 h->w, h->V + (size_t)(j + 1) * N, h->dinv, r64, r32);
       GS2_LAUNCH_CHECK();
     }
   }
@@ -916,13 +916,14 @@ struct PackRun {
     *h->stop_mapped = 0;
     GS2_CUDA(cudaMemcpyAsync(P->active, P->active_host, sizeof(int) * P->count,
                              cudaMemcpyHostToDevice, h->stream));
-    launch_pdl(k_pcycle_reset, 1, 1024, 0, h->stream, P->st, P->active, P->count, P->nactive, h->st);
+    launch_pdl(k_pcycle_reset, 1, 1024, 0, h->stream, P->st, P->active, P->count, P->nactive,
+               h->st);
     GS2_LAUNCH_CHECK();
     launch_pdl(k_plive_init, (P->nchunks + 255) / 256, 256, 0, h->stream, P->nchunks, (int)h->n,
                P->off_dev, P->count, P->active, P->live_cycle, P->live_run);
     GS2_LAUNCH_CHECK();
-    launch_pdl(k_pcycle_start, P->gb, kVecThreads, 0, h->stream, P->blk, P->items, P->cnt, P->st, h->r,
-               h->V, h->dinv, r64, r32, P->gvec, (int)P->vstride(), m);
+    launch_pdl(k_pcycle_start, P->gb, kVecThreads, 0, h->stream, P->blk, P->items, P->cnt, P->st,
+               h->r, h->V, h->dinv, r64, r32, P->gvec, (int)P->vstride(), m);
     GS2_LAUNCH_CHECK();
     cycle_ran = true;
     if (use_graph()) {
@@ -950,9 +951,9 @@ struct PackRun {
       KernelTimer tm(h, "combine", 8.0 * h->n * (m + 1));
       const int N = (int)h->n;
       const int vs = (int)P->vstride();
-#define GS2_PCOMBINE(M)                                                                  \
-  launch_pdl(k_pcombine<M>, P->gb, kVecThreads, 0, h->stream, N, P->blk, P->items, P->cnt, P->st, h->V, \
-             P->y, vs, h->w, h->dinv, r64, r32)
+#define GS2_PCOMBINE(M)                                                                    \
+  launch_pdl(k_pcombine<M>, P->gb, kVecThreads, 0, h->stream, N, P->blk, P->items, P->cnt, \
+             P->st, h->V, P->y, vs, h->w, h->dinv, r64, r32)
       if (m <= 8) GS2_PCOMBINE(8);
       else if (m <= 16) GS2_PCOMBINE(16);
       else if (m <= 32) GS2_PCOMBINE(32);

@@ -5,7 +5,7 @@
 // microseconds of launch and drain however little work it holds.  Here the
 // whole solve -- every restart cycle, the GS2 or JR preconditioner, the CGS2
 // Arnoldi steps, the Givens rotations and the true-residual checks -- runs in
-// one launch of at most 64 co-resident blocks (cooperative launch).  Rows are
+// one launch of at most 128 co-resident blocks (cooperative launch).  Rows are
 // owned by threads for the whole solve, so a phase that only touches its own
 // rows needs no synchronisation; a phase that gathers other rows' values
 // waits at a grid barrier first.  Inner products are block partial sums

@@ -182,7 +182,7 @@ static void hybrid_apply(gs2_handle* h, const gs2_params* p, const Hybrid& Y, co
         continue;
       }
       if (p->kind == GS2_PC_GS) {
-        // local exact GS / SOR: the local triangular solves by level sets
+        // local exact GS / SOR: the local triangular solves
         if (p->direction == GS2_FORWARD || p->direction == GS2_SYMMETRIC) {
           gs_half(h, Y.Lloc, Y.triL, Y.Aloc, c, x, p->omega, zero, skip);
           zero = false;

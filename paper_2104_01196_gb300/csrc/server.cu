@@ -66,11 +66,11 @@ struct Group {
 
 // Bytes of the sliced-ELL copy of a matrix with this many entries (at most
 // 1.2 slots per entry, 2 in a small matrix, else no copy is made) holding
-// vbytes-byte values, with
-// its chunk offsets and row order (lane slices: up to a chunk per two rows).
+// vbytes-byte values, with its chunk offsets and row order (lane slices: up to
+// a chunk per two rows, and the arrays' alignment).
 static int64_t sell_bytes(int64_t entries, int64_t n, int vbytes) {
   const int64_t slots = entries <= (1 << 18) ? 2 * entries + 1 : entries * 6 / 5 + 1;
-  return slots * (4 + vbytes) + 4 * (n / 2 + 2) + 4 * n;
+  return slots * (4 + vbytes) + 4 * (n / 2 + 2) + 4 * n + 1024;
 }
 
 // Device bytes a request of this size holds once admitted: the matrix, its
