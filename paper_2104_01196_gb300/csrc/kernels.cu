@@ -326,14 +326,14 @@ void launch_resid(gs2_handle* h, const double* b, const double* x, double* r_out
 void launch_resid_matrix(gs2_handle* h, const DevCsr& M, const double* b, const double* x,
                          double* r_out, double* rhat64, float* rhat32, const int* skip) {
   // algorithmic bytes: M once, x, b, D^{-1} read, r / rhat written
-  KernelTimer tm(h, "resid", bytes_csr(M, 8) + 24.0 * h->n + (r_out ? 8.0 * h->n : 0.0) +
+  KernelTimer tm(h, "resid", matrix_bytes(M, 8) + 24.0 * h->n + (r_out ? 8.0 * h->n : 0.0) +
                  (rhat64 ? 8.0 * h->n : 0.0) + (rhat32 ? 4.0 * h->n : 0.0));
   EpiResid e{x, b, h->dinv, r_out, rhat64, rhat32};
   dispatch<double>(h, M, M.va, e, skip);
 }
 
 void launch_spmv(gs2_handle* h, const double* x, double* y, const int* skip) {
-  KernelTimer tm(h, "spmv", bytes_csr(h->A, 8) + 16.0 * h->n);
+  KernelTimer tm(h, "spmv", matrix_bytes(h->A, 8) + 16.0 * h->n);
   EpiSpmv e{x, y};
   dispatch<double>(h, h->A, h->A.va, e, skip);
 }
@@ -341,7 +341,7 @@ void launch_spmv(gs2_handle* h, const double* x, double* y, const int* skip) {
 void launch_spmv_matrix(gs2_handle* h, const DevCsr& M, const double* x, double* y,
                         bool accumulate, const int* skip) {
   KernelTimer tm(h, accumulate ? "amg_prolong" : "amg_restrict",
-                 bytes_csr(M, 8) + 8.0 * M.n * (accumulate ? 3.0 : 2.0));
+                 matrix_bytes(M, 8) + 8.0 * M.n * (accumulate ? 3.0 : 2.0));
   if (accumulate) {
     EpiSpmvAdd e{x, y};
     dispatch<double>(h, M, M.va, e, skip);
@@ -354,7 +354,7 @@ void launch_spmv_matrix(gs2_handle* h, const DevCsr& M, const double* x, double*
 void launch_restrict(gs2_handle* h, const DevCsr& M, const double* x, double* y,
                      const double* dinv, double* rhat64, float* rhat32, const int* skip) {
   KernelTimer tm(h, "amg_restrict",
-                 bytes_csr(M, 8) + 24.0 * M.n + (rhat64 ? 8.0 : 4.0) * M.n);
+                 matrix_bytes(M, 8) + 24.0 * M.n + (rhat64 ? 8.0 : 4.0) * M.n);
   EpiRestrict e{x, dinv, y, rhat64, rhat32};
   dispatch<double>(h, M, M.va, e, skip);
 }
@@ -408,9 +408,10 @@ __global__ void k_to_sell(int n, const int* __restrict__ rp, const int* __restri
 
 // CSR rows into lane slices (DevCsr::sell_lanes), one thread per lane of a row
 template <typename T>
-__global__ void k_to_lanes(int n, int K, bool held, const int* __restrict__ rp, const int* __restrict__ ci,
-                           const T* __restrict__ va, const int* __restrict__ cptr,
-                           const int* __restrict__ perm, int* sci, T* sva) {
+__global__ void k_to_lanes(int n, int K, bool held, const int* __restrict__ rp,
+                           const int* __restrict__ ci, const T* __restrict__ va,
+                           const int* __restrict__ cptr, const int* __restrict__ perm, int* sci,
+                           T* sva) {
   const int64_t total = (int64_t)n * K;
   for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < total;
        t += (int64_t)gridDim.x * blockDim.x) {
@@ -500,7 +501,7 @@ float time_tile_probe(gs2_handle* h, const DevCsr& M, int reps, int role) {
 
 void launch_compact_rhs(gs2_handle* h, const DevCsr& Tother, const double* b, const double* x,
                         double* rhat64, float* rhat32, const int* skip) {
-  KernelTimer tm(h, "compact_rhs", bytes_csr(Tother, 8) + 24.0 * h->n +
+  KernelTimer tm(h, "compact_rhs", matrix_bytes(Tother, 8) + 24.0 * h->n +
                                        (rhat64 ? 8.0 : 4.0) * h->n);
   EpiCompact e{x, b, h->dinv, rhat64, rhat32};
   dispatch<double>(h, Tother, Tother.va, e, skip);
@@ -513,7 +514,7 @@ void launch_jr(gs2_handle* h, const double* b, const double* x_in, double* x_out
 
 void launch_jr_matrix(gs2_handle* h, const DevCsr& M, const double* b, const double* x_in,
                       double* x_out, double omega, const int* skip) {
-  KernelTimer tm(h, "jr", bytes_csr(M, 8) + 32.0 * h->n);
+  KernelTimer tm(h, "jr", matrix_bytes(M, 8) + 32.0 * h->n);
   EpiJr e{x_in, b, h->dinv, x_out, omega};
   dispatch<double>(h, M, M.va, e, skip);
 }
@@ -527,7 +528,7 @@ void launch_inner(gs2_handle* h, const DevCsr& T, int prec, const void* rhat,
   const bool damped = gamma != 1.0;
   const double vb = prec == GS2_FP64 ? 8.0 : (prec == GS2_FP32 ? 4.0 : 2.0);
   const double gb = prec == GS2_FP64 ? 8.0 : 4.0;
-  double bytes = bytes_csr(T, (int)vb) + gb * T.n * (2 + (damped ? 1 : 0)) +
+  double bytes = matrix_bytes(T, (int)vb) + gb * T.n * (2 + (damped ? 1 : 0)) +
                  (mode == INNER_MID ? gb * T.n : (mode == INNER_LAST_ADD ? 16.0 : 8.0) * T.n) +
                  (prec == GS2_FP16_ROWSCALED ? 1.0 * T.n : 0.0);
   KernelTimer tm(h, prec == GS2_FP64 ? "inner64" : (prec == GS2_FP32 ? "inner32" : "inner16"),
@@ -569,7 +570,7 @@ void launch_resid_sweep(gs2_handle* h, int vprec, const int* skip) {
   // read, rhat32 written
   const bool half = vprec == GS2_FP16_ROWSCALED;
   KernelTimer tm(h, half ? "resid16" : "resid32",
-                 bytes_csr(O, half ? 2 : 4) + 12.0 * O.n + (half ? 1.0 * O.n : 0.0));
+                 matrix_bytes(O, half ? 2 : 4) + 12.0 * O.n + (half ? 1.0 * O.n : 0.0));
   if (half) {
     EpiResidSweep<true> e{h->bhat32, h->x32, O.scale16, h->rhat32};
     dispatch<__half>(h, O, O.va16, e, skip);
@@ -584,7 +585,7 @@ void launch_color(gs2_handle* h, const DevCsr& C, const int* rows, const double*
   const bool damped = omega != 1.0;
   // colour matrix once; per row its index, bhat, the written x and (lower
   // bound) one gathered x of another colour; damping re-reads x_r
-  KernelTimer tm(h, "color", bytes_csr(C, 8) + C.n * (28.0 + (damped ? 8.0 : 0.0)));
+  KernelTimer tm(h, "color", matrix_bytes(C, 8) + C.n * (28.0 + (damped ? 8.0 : 0.0)));
   if (damped) {
     EpiColor<true> e{rows, bhat, x, omega};
     dispatch<double>(h, C, C.va, e, skip);

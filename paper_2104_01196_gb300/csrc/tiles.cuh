@@ -613,14 +613,14 @@ k_stencil(int n, int nchunks, const int* __restrict__ cptr, const int* __restric
 
 // Lane slices (DevCsr::sell_lanes): K lanes per row, 32 / K rows a warp, each
 // lane its consecutive part of the row as in the row tiles, read slot by slot
-// as coalesced loads.  One warp per chunk: the
-// rows of a window are sorted longest first, so the long chunks of every
-// window start early and the hardware's block scheduler fills in the short
-// ones.  The next group's four slots are loaded while the current group's
-// gathers are in flight; padding slots (column -1) gather nothing, so an
-// infinity elsewhere cannot reach the row.  HELD (DevCsr::sell_held): the last
-// slot of a row's first lane is its last entry, which joins the sum after the
-// lanes' parts.
+// as coalesced loads.  One warp per chunk: the rows of a window are sorted
+// longest first, so the long chunks of every window start early and the
+// hardware's block scheduler fills in the short ones.  The next group's four
+// slots are loaded while the current group's gathers are in flight; padding
+// slots (column -1) gather nothing, so an infinity elsewhere cannot reach the
+// row.  The last group is written out, without slot tests in the others.  HELD
+// (DevCsr::sell_held): the last slot of a row's first lane is its last entry,
+// which joins the sum after the lanes' parts.
 // (Five resident blocks: at the 66 registers ptxas takes unasked, three fit
 // and the uneven rows' sweep takes 91 instead of 70 us; at eight it takes 101.)
 template <int K, bool HELD, typename VT, class Epi>
@@ -785,7 +785,8 @@ inline void launch_sell(gs2_handle* h, const DevCsr& M, const VT* sv, const Epi&
   // 46 registers) keep k_sell: inner sweep 19 against 23 us on 7-point rows'
   // triangles, n = 3.4M.
   bool pair = false;
-  auto fn = M.mean_row > kShortRowMean ? k_sell<VT, Epi, true, false> : k_sell<VT, Epi, false, false>;
+  auto fn = M.mean_row > kShortRowMean ? k_sell<VT, Epi, true, false>
+                                       : k_sell<VT, Epi, false, false>;
   if constexpr (sizeof(VT) < sizeof(double)) {
     if (M.mean_row >= 4.5 && M.mean_row <= 8.0) {
       pair = true;
@@ -834,8 +835,14 @@ inline void dispatch(gs2_handle* h, const DevCsr& M, const VT* va, const Epi& ep
   }
 }
 
-inline double bytes_csr(const DevCsr& M, int vbytes) {
-  return (double)M.nnz * (4.0 + vbytes) + 4.0 * (M.n + 1);
+// Bytes of M that a row kernel reads: values, columns where the layout stores
+// them (the chunks of an offset layout share a short list), row or chunk
+// pointers and the row order.
+inline double matrix_bytes(const DevCsr& M, int vbytes) {
+  if (!M.sell) return (double)M.nnz * (4.0 + vbytes) + 4.0 * (M.n + 1);
+  const double cols = 1.0 - (double)M.sell_offset_chunks / std::max(M.sell_chunks, 1);
+  return (double)M.nnz * (4.0 * cols + vbytes) + 8.0 * M.sell_chunks +
+         (M.sell_row ? 4.0 * M.n : 0.0);
 }
 
 }  // namespace gs2
