@@ -341,7 +341,7 @@ static bool sell_layout(const std::vector<int>& rp, const int* ci, int n, const 
 constexpr int kLaneWindow = 1024;    // rows sorted together
 constexpr int kLaneWarpsPerSm = 16;  // warps that a matrix should give each SM
 constexpr int kLaneMaxSlots = 128;   // of one chunk: longer rows need a whole block
-constexpr int kSellWarpsPerSm = 32;  // resident warps of k_sell on long rows
+constexpr int kLaneResident = 40;    // warps that an SM holds of k_lanes
 
 // Lanes per row: at most 24 entries a lane on average; with fewer than 16
 // warps per SM more lanes, down to 4 entries each (a warp's groups of four
@@ -449,12 +449,13 @@ static void upload_sell(gs2_handle* h, DevCsr& M, const std::vector<int>& rp, co
     M.sell_lanes = longest <= kLaneMaxSlots * K && lane_layout(rp, n, K, lanes) ? K : 0;
     return M.sell_lanes > 0;
   };
-  // a long-row A of less than two waves of warps: one lane a row, but a warp
-  // per chunk instead of a persistent grid whose last wave is nearly empty
-  // (Q1 elasticity on 40^3 nodes, residual 39.5 -> 34.8 us; no gain on 50^3,
-  // 3% lost on 64^3)
+  // a long-row A whose chunks are all resident at once in the lane kernel: one
+  // lane a row, a warp per chunk; k_sell holds 32 warps an SM on long rows and
+  // runs a second, nearly empty wave from there on (Q1 elasticity, residual: 37^3
+  // nodes 28.5 -> 26.8 us, 40^3 39.4 -> 33.1; with 1.3 waves of the lane kernel,
+  // 44^3, 45.5 against 55.8)
   const bool few = &M == &h->A && !short_rows && streams &&
-                   n < 2 * 32 * (int64_t)kSellWarpsPerSm * h->nsm && try_lanes(1);
+                   n <= 32 * (int64_t)kLaneResident * h->nsm && try_lanes(1);
   bool sliced = !few && (short_rows || streams) && sell_layout(rp, ci, n, origin, zeros, lay);
   // short rows with explicit columns, too few for the SMs' warps at one lane
   // each (the 64,560 rows of a second multigrid level, 15 entries in a
