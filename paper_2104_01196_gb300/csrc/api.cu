@@ -257,14 +257,14 @@ void retile(gs2_handle* h, DevCsr& M, const std::vector<int>& rp, int K, int RPT
 // row-tile shape, 8 lanes per row).  Long rows of smaller matrices (coarse
 // multigrid levels) are latency-bound: K lanes per row shorten each row's
 // chain of dependent gathers.  They, and matrices of uneven rows, get lane
-// slices, which reduce a row in K segments as the row
-// tiles do without staging it through shared memory (the stages limit a tile
-// kernel to 2 to 3 blocks per SM, and its barriers idle the short rows'
-// lanes): symmetric FP64 sweep on 300,007 uneven rows 115 -> 70 us, on Q1
-// elasticity with 28^3 nodes 105 -> 58.  FP32 and FP16 values follow where the
-// slices have the row tiles' lanes, whose rounding they keep (inner sweep on
-// 40^3 nodes 16.9 -> 13.8 us, on 28^3 8.5 -> 6.8; whole-sweep residual there
-// 13.0 -> 10.5), and stay in the row tiles elsewhere.
+// slices, which reduce a row in K segments as the row tiles do without staging
+// it through shared memory (the stages limit a tile kernel to 2 to 3 blocks
+// per SM, and its barriers idle the short rows' lanes): symmetric FP64 sweep on
+// 300,007 uneven rows 116 -> 63 us, on Q1 elasticity with 28^3 nodes 106 -> 53.
+// FP32 and FP16 values follow where the slices have the row tiles' lanes, whose
+// rounding they keep (inner sweep on 40^3 nodes 17.3 -> 13.5 us, on 28^3 8.4 ->
+// 6.3; whole-sweep residual there 12.1 -> 8.5), and stay in the row tiles
+// elsewhere.
 constexpr int kSellC = 32;                       // rows per chunk (one warp)
 constexpr double kSellMaxPadding = 1.2;          // slots / entries
 constexpr int kSellSmall = 1 << 18;  // entries up to which lane slices may pad to double
@@ -345,12 +345,14 @@ constexpr int kLaneResident = 40;    // warps that an SM holds of k_lanes
 
 // Lanes per row: at most 24 entries a lane on average; with fewer than 16
 // warps per SM more lanes, down to 4 entries each (a warp's groups of four
-// slots wait one after another, 0.4 us each out of L2: Q1 elasticity on 16^3
-// nodes, SpMV 7.1 -> 5.0 us with 8 lanes instead of 4); and two where the
-// longest row exceeds 32 entries a lane (the 300,007 uneven rows, 64 at most:
-// a symmetric sweep 79 -> 70 us).  With more than 16 warps per SM further
-// lanes only add shuffles and FP64 adds (elasticity on 28^3 nodes: 58 us with
-// 4 lanes, 98 with 16).  A pack's lanes do not depend on its size.
+// slots wait one after another, 0.4 us each out of L2: symmetric sweep on 2,000
+// uneven rows, 11 entries on average, 22.9 -> 13.4 us with 4 lanes instead of
+// one, V-cycle on a 24^3 grid 62 -> 49 us; Q1 elasticity on 16^3 nodes 19.7 ->
+// 19.1); and two where the longest row exceeds 32 entries a lane (the 300,007
+// uneven rows, 64 at most: a symmetric sweep 69 -> 63 us).  With more than 16
+// warps per SM further lanes only add shuffles and FP64 adds (elasticity on
+// 28^3 nodes: 53 us with 4 lanes, 90 with 16).  A pack's lanes do not depend on
+// its size.
 //
 // Where A has more lanes than its row tiles, a row's last entry is held back
 // until the lanes' parts are added up (sell_held): in rows that store the
@@ -458,8 +460,8 @@ static void upload_sell(gs2_handle* h, DevCsr& M, const std::vector<int>& rp, co
                    n <= 32 * (int64_t)kLaneResident * h->nsm && try_lanes(1);
   bool sliced = !few && (short_rows || streams) && sell_layout(rp, ci, n, origin, zeros, lay);
   // short rows with explicit columns, too few for the SMs' warps at one lane
-  // each (the 64,560 rows of a second multigrid level, 15 entries in a
-  // triangle: inner sweep 12.6 -> 8.6 us with two lanes); long rows here
+  // each (SGS2(1,2) on 10,001 rows of 19 to 22 entries 24.6 -> 18.9 us, on 3,001
+  // rows of 13 to 15 20.2 -> 15.4; even from 60,000 rows on); long rows here
   // stream and keep one lane (Q1 elasticity on 64^3 nodes, residual 126 us
   // against 150 with four)
   if (sliced && short_rows && lay.offset_chunks == 0 && !h->for_pack &&

@@ -563,8 +563,9 @@ __device__ __forceinline__ AT stencil_rows(AT s, int L, int at, const int* __res
 // dependent round trip to memory where k_sell's loop costs three.  Rows are
 // reduced in the same order.  On the 150^3 convection-diffusion matrix
 // (n = 3.4M) against k_sell: SpMV 52 -> 45 us (5.4 TB/s; the FP64 pipe needs
-// 40), FP64 inner sweep 30 -> 28, FP32 inner sweep 22 -> 18; on the 1000^2
-// Laplacian SpMV 18 -> 13 us, residual 19 -> 16, FP64 inner sweep 12 -> 8.
+// 40), JR 78 -> 74, FP32 inner sweep 22 -> 18, FP64 inner sweep even at 35; on
+// the 1000^2 Laplacian SpMV 18 -> 13 us, residual 21 -> 19, FP64 inner sweep 13
+// -> 10.
 // (The explicit minimum of one resident block lets ptxas hold all slots of a
 // row in registers -- 54 instead of 32 for the 7-point SpMV -- where its
 // default aims at full occupancy and puts the loads one after another again.)
@@ -621,8 +622,9 @@ k_stencil(int n, int nchunks, const int* __restrict__ cptr, const int* __restric
 // row.  The last group is written out, without slot tests in the others.  HELD
 // (DevCsr::sell_held): the last slot of a row's first lane is its last entry,
 // which joins the sum after the lanes' parts.
-// (Five resident blocks: at the 66 registers ptxas takes unasked, three fit
-// and the uneven rows' sweep takes 91 instead of 70 us; at eight it takes 101.)
+// (Five resident blocks: the uneven rows' sweep takes 63 us, as with the
+// registers that ptxas takes unasked; at eight it takes 79, and Q1 elasticity
+// on 40^3 nodes 129 instead of 107.)
 template <int K, bool HELD, typename VT, class Epi>
 __global__ void __launch_bounds__(kRowThreads, 5)
 k_lanes(int n, int nchunks, const int* __restrict__ cptr, const int* __restrict__ ci,
@@ -777,8 +779,8 @@ inline void launch_sell(gs2_handle* h, const DevCsr& M, const VT* sv, const Epi&
   // Stencils (offset chunks only, at most 8 slots) take the unrolled form up
   // to the width at which it is the faster one for the epilogue: for the FP64
   // residual 6 slots (its two more row operands and 7 slots need 56
-  // registers, half the resident warps: 58 against 53 us on 7-point rows,
-  // n = 3.4M), for the compact right-hand side 2 (a compact symmetric sweep on
+  // registers, half the resident warps: a symmetric sweep without inner sweeps
+  // on 7-point rows 179 against 171 us, n = 4.1M), for the compact right-hand side 2 (a compact symmetric sweep on
   // the 100^3 convection-diffusion matrix, 3-entry triangles, 47.0 against 42.7
   // us; on the 1000^2 Laplacian, 2 entries, 37.8 against 41.6), for the
   // whole-sweep residual 4.  FP16 values (whose conversion and row scale cost it

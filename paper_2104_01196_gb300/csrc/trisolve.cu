@@ -22,10 +22,11 @@
 // co-resident grid.  Waits are bounded all the same; a warp that gives up
 // records GS2_ERR_TIMEOUT and leaves.
 //
-// Measured, a symmetric sweep (two half sweeps, residuals included): 100^3
-// Laplacian (298 levels) 2908 -> 512 us, 0.8 us a level; 500^2 Laplacian (999
-// levels) 6508 -> 1099; 40^2 426 -> 75; Q1 elasticity on 20^3 nodes 5931 ->
-// 900.  One, two and four blocks per SM differ by 3%.
+// Measured, a symmetric sweep (two half sweeps, residuals included), against a
+// launch per level: 100^3 Laplacian (298 levels) 2894 -> 535 us, 0.85 us a
+// level; 200^2 Laplacian (399 levels) 2359 -> 452; a chain of 3,000 rows 11,700
+// -> 2980; Q1 elasticity on 28^3 nodes 10,080 -> 1395.  One, two and four blocks
+// per SM differ by 3%.
 #include <algorithm>
 #include <cstring>
 #include <vector>
